@@ -71,12 +71,19 @@ int minres_fused_batch(Op &op, int N, const float4 *r, float4 *e, float4 *const 
                        FusedState *ms, double *partials, const double *d_tol,
                        const dlz_params &p, int &iters, HostScratch &hs, bool e_init = false);
 // Fused FP32 CG on the normal equations for D e = s0 on N right-hand sides
-// (cg_fused.cu); s0 is overwritten, e is updated in place (holds the start).
+// (cg_fused.cu); s0 is read only at the start, e is updated in place (holds the start).
 struct CgFusedState;
+size_t cg_state_bytes();
+constexpr int kCgResiduals = 6;
+// Work vectors, each of N x 6 V float4: the image t, the direction p and the residuals of a
+// block of iterations.  r[1] and later may be s0's memory.
+struct CgBuffers {
+    float4 *t, *p, *r[kCgResiduals];
+};
 // blocks per right-hand side of the fused CGNR kernels for an N-RHS batch (the size of
 // their partials arrays)
 long cgnr_blocks_per_rhs(const Op &op, int N);
-int cgnr_fused_batch(Op &op, int N, float4 *s0, float4 *e, float4 *const bufs[5], CgFusedState *ms,
+int cgnr_fused_batch(Op &op, int N, const float4 *s0, float4 *e, const CgBuffers &bufs, CgFusedState *ms,
                      double *partials, const double *d_tol, const dlz_params &p, int &iters);
 // FP32 D-MinRes with FP64 defect correction on many lattices at once
 // (minres_multi.cu); B[l], X[l]: nrhs[l] <= 16 internal FP64 vectors of lattice l,

@@ -17,28 +17,11 @@
 
 #include "dlz_internal.cuh"
 #include "krylov_util.cuh"
+#include "minres_state.cuh"
 #include "prec.cuh"
 #include "reduce.cuh"
 #include "small_dense.h"
 #include "solvers.h"
-
-namespace dlz {
-
-namespace {
-
-// scalar scratch of the inner solvers (sized for either state: FusedState of the
-// fused MinRes or CgFusedState of the fused CGNR)
-struct InnerState {
-    double beta, alpha, beta_next, inv_beta;
-    double c, s, c_old, s_old, phibar;
-    double eps, delta, gamma, tau;
-    double rr, ss, pq;
-    float fa, fb;
-};
-
-}  // namespace
-
-}  // namespace dlz
 
 // ------------------------------------------------------------------ batched form
 // N <= kMaxBatch right-hand sides share every launch: the stencil processes all
@@ -62,14 +45,14 @@ int dsolve_mixed_batch(Op &op, const dlz_defl_s *d, bool minres, const double2 *
         return fail(DLZ_ERR_BADARG, "even-odd operators: FP32 D-MinRes is not built (use DLZ_F64, or D-CG)");
     const long n64 = 12L * op.g.V;
     const long n32 = 6L * op.g.V;
-    DevBuf bp, x, r, tmp, corr, dots, scal, f32;
+    DevBuf bp, x, r, tmp, scal, f32;
     DLZ_TRY(bp.alloc((size_t)N * n64 * sizeof(double2)));
     DLZ_TRY(x.alloc((size_t)N * n64 * sizeof(double2)));
     DLZ_TRY(r.alloc((size_t)N * n64 * sizeof(double2)));
     DLZ_TRY(tmp.alloc((size_t)N * n64 * sizeof(double2)));
-    DLZ_TRY(corr.alloc(n64 * sizeof(double2)));
-    DLZ_TRY(dots.alloc((size_t)std::max(1, d ? d->k : 1) * sizeof(double2)));
-    DLZ_TRY(scal.alloc((size_t)(kMaxBatch * 24 + 4 * kMaxBatch) * sizeof(double)));
+    // scalars of the inner solver, then ||r_q||, its inverse, the tolerances and ||b_q||
+    const size_t state_doubles = (kMaxBatch * std::max(sizeof(FusedState), cg_state_bytes()) + 7) / 8;
+    DLZ_TRY(scal.alloc((state_doubles + 4 * kMaxBatch) * sizeof(double)));
     DLZ_TRY(f32.alloc((size_t)8 * N * n32 * sizeof(float4)));
     float4 *w32[8];
     for (int i = 0; i < 8; ++i) w32[i] = f32.as<float4>() + (size_t)i * N * n32;
@@ -80,8 +63,8 @@ int dsolve_mixed_batch(Op &op, const dlz_defl_s *d, bool minres, const double2 *
     }
     const long k1_blocks = std::max((long)((op.g.V + 127) / 128), minres ? 0L : cgnr_blocks_per_rhs(op, N)) * N;
     DLZ_TRY(fpart.alloc((size_t)2 * k1_blocks * sizeof(double)));   // K1 and K2a partials
-    InnerState *ist = reinterpret_cast<InnerState *>(scal.as<double>());
-    double *d_rn = scal.as<double>() + kMaxBatch * 24;        // ||r_q||
+    double *ist = scal.as<double>();
+    double *d_rn = ist + state_doubles;                       // ||r_q||
     double *d_inv = d_rn + kMaxBatch, *d_tol = d_inv + kMaxBatch, *d_bn = d_tol + kMaxBatch;
     HostScratch hs;
     DLZ_TRY(hs.ensure(1024));
@@ -242,7 +225,10 @@ int dsolve_mixed_batch(Op &op, const dlz_defl_s *d, bool minres, const double2 *
             mv_batch += iters - it0;
         } else {
             if (!proj) DLZ_CUDA_TRY(cudaMemsetAsync(w32[1], 0, (size_t)N * n32 * sizeof(float4), op.stream));
-            float4 *const bufs[5] = {w32[2], w32[3], w32[4], w32[5], w32[6]};
+            // the FP64 work vectors of the residual are idle during the inner solve: one of
+            // the residual buffers lies in them, another is s0's own
+            const CgBuffers bufs = {w32[3], w32[4],
+                                    {w32[2], w32[5], w32[6], w32[7], w32[0], reinterpret_cast<float4 *>(pt)}};
             DLZ_TRY(cgnr_fused_batch(op, N, w32[0], w32[1], bufs, reinterpret_cast<CgFusedState *>(ist),
                                      fpart.as<double>(), d_tol, p, iters));
             mv_batch += 2L * (iters - it0);
