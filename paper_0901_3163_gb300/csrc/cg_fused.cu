@@ -365,7 +365,7 @@ long cgnr_blocks_per_rhs(const Op &op, int N) {
 }
 
 int cgnr_fused_batch(Op &op, int N, const float4 *S, float4 *e, const CgBuffers &bf, CgFusedState *ms,
-                     double *partials, const double *d_tol, const dlz_params &p, int &iters) {
+                     double *partials, const double *d_tol, const dlz_params &p, int &iters, GraphExec &ge) {
     const long n = 6L * op.g.V;
     const Geom g = op.g;
     const float kappa = (float)op.kappa, kappa2 = (float)(op.kappa * op.kappa);
@@ -431,7 +431,6 @@ int cgnr_fused_batch(Op &op, int N, const float4 *S, float4 *e, const CgBuffers 
         DLZ_CUDA_TRY(cudaGetLastError());
         return DLZ_OK;
     };
-    GraphExec ge;
     auto six = [&]() -> int {
         for (int slot = 0; slot < kCgBlock; ++slot) DLZ_TRY(iteration(slot));
         return DLZ_OK;

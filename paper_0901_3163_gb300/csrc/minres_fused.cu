@@ -1,22 +1,22 @@
 // Fused FP32 MinRes iteration for a batch of right-hand sides (the inner
 // solve of the mixed-precision D-MinRes, arXiv:0901.3163 Sec. 2).
 //
-// Two full passes over the vectors per iteration:
+// Two passes over the vectors per iteration, and a third per block of six:
 //   K1 (stencil + epilogue, one block = 128 sites of one right-hand side):
 //        v_j   = u_j / beta_j                      (u_j: unnormalised Lanczos vector; the
 //                                                   v's are never stored, only the u's)
 //        w     = Q v_j - beta_j v_{j-1}            (Q u_j / beta_j: Q is linear)
 //        alpha_j partial = Re <v_j, w>
-//        d_{j-1} = (v_{j-1} - delta d_{j-2} - eps d_{j-3}) / gamma,  e += tau d_{j-1}
-//        (the direction update of the previous step: its Givens rotation needed
-//         beta_j, known only now)
 //   K2a: u_{j+1} = w - alpha_j v_j and the block partials of ||u_{j+1}||^2;
 //   K1b: alpha_j = sum of K1's block partials (one block per right-hand side);
-//   K2b: beta_{j+1}, and the Givens rotation of step j (one block per right-hand side);
-// for a single right-hand side K1b and K2b are folded into the last block of K1 and
-// K2a to finish.  The partials (block b belongs to right-hand side b mod N) are summed
-// in a fixed order, so results are deterministic.  Buffers rotate with periods 3 and 2, so a group of 6 iterations is
-// captured once as a CUDA graph and replayed.
+//   K2b: beta_{j+1}, the Givens rotation of step j and the coefficients of its direction
+//        (one block per right-hand side);
+//   after the fifth iteration of a block: the deferred update of the directions and the
+//        iterate (minres_state.cuh has the scheme, the buffers and the traffic).
+// For a single right-hand side K1b and K2b are folded into the last block of K1 and K2a to
+// finish.  The partials are summed in a fixed order, so results are deterministic.  A block
+// of six iterations is captured once as a CUDA graph and replayed.
+// Measured on 16^3 x 32 with 11 right-hand sides: see k_minres_k1.
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -28,6 +28,7 @@
 #include "reduce.cuh"
 #include "solvers.h"
 #include "minres_state.cuh"
+#include "slab_walk.cuh"
 #include "wilson_site.cuh"
 
 namespace dlz {
@@ -39,20 +40,18 @@ namespace {
 constexpr int kThreads = 128;
 
 
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, 7)
 k_minres_k1(const float4 *__restrict__ Ub, const float4 *__restrict__ Up, float4 *__restrict__ W,
-            const float4 *__restrict__ D2, float4 *__restrict__ D3, float4 *__restrict__ E,
-            const float4 *__restrict__ links, Geom g, float kappa, int N,
+            const float4 *__restrict__ links, Geom g, SlabWalk w, float kappa, int N,
             FusedState *__restrict__ st, double *__restrict__ partials, unsigned *__restrict__ counters) {
     const int q = blockIdx.x % N;
-    const int s = (blockIdx.x / N) * blockDim.x + threadIdx.x;
-    const long nel = 6L * g.V;
-    const size_t base = (size_t)q * nel;
+    int s0, nb;
+    slab_block(w, blockIdx.x / N, s0, nb);
+    const int s = s0 + threadIdx.x;
+    const size_t base = (size_t)q * 6 * g.V;
     float facc = 0.f;
-    if (s < g.V) {
-        facc = minres_k1_site(s, g, kappa, Ub + base, Up + base, W + base, D2 + base, D3 + base, E + base,
-                              links, st[q]);
-    }
+    if ((int)threadIdx.x < nb)
+        facc = minres_k1_site(s, g, kappa, Ub + base, Up + base, W + base, links, st[q]);
     // block partials of alpha_q; with counters, the last block of q to finish forms
     // alpha_q (one right-hand side: saves a launch); without, k_minres_alpha does
     const int nbq = gridDim.x / N;
@@ -67,16 +66,15 @@ k_minres_k1(const float4 *__restrict__ Ub, const float4 *__restrict__ Up, float4
 }
 
 __global__ void __launch_bounds__(kThreads)
-k_minres_k2a(float4 *__restrict__ W, const float4 *__restrict__ Vc, Geom g, int N,
+k_minres_k2a(const float4 *W, const float4 *Vc, float4 *Out, float4 *Copy, Geom g, int N, int iter,
              FusedState *__restrict__ st, double *__restrict__ partials, unsigned *__restrict__ counters) {
     // Vc: the unnormalised u_j; alpha_j v_j = (alpha_j / beta_j) u_j
     const int q = blockIdx.x % N;
     const int s = (blockIdx.x / N) * blockDim.x + threadIdx.x;
     const size_t base = (size_t)q * 6 * g.V;
     float facc = 0.f;
-    if (s < g.V) {
-        facc = minres_k2a_site(s, g.V, W + base, Vc + base, st[q]);
-    }
+    if (s < g.V)
+        facc = minres_k2a_site(s, g.V, W + base, Vc + base, Out + base, Copy ? Copy + base : nullptr, st[q]);
     // the last block of q to finish: beta_{j+1} and the Givens rotation of step j
     // (with counters; without, k_minres_k2b does it)
     const int nbq = gridDim.x / N;
@@ -85,22 +83,30 @@ k_minres_k2a(float4 *__restrict__ W, const float4 *__restrict__ Vc, Geom g, int 
         return;
     }
     double r2;
-    if (partial_then_last_sum<kThreads>(facc, partials + (size_t)q * nbq, blockIdx.x / N, nbq, counters + q, &r2) &&
-        threadIdx.x == 0) {
-        FusedState t = st[q];
-        fused_givens(t, r2);
-        st[q] = t;
-    }
+    if (partial_then_last_sum<kThreads>(facc, partials + (size_t)q * nbq, blockIdx.x / N, nbq, counters + q, &r2))
+        fused_givens(st[q], r2, iter);
+}
+
+// the deferred update of a block (LAST: of the one step left at the end), n float4 per
+// right-hand side, blockIdx.y the right-hand side
+template <bool LAST>
+__global__ void __launch_bounds__(256)
+k_minres_directions(MinresVectors b, const FusedState *__restrict__ st, long n) {
+    const long j = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= n) return;
+    const size_t i = (size_t)blockIdx.y * n + j;
+    if (LAST) minres_last_direction(b, i, st[blockIdx.y]);
+    else minres_directions_elem(b, i, st[blockIdx.y]);
 }
 
 // alpha_q = sum of the block partials of right-hand side q (block q of the grid),
 // in a fixed order
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(1024)
 k_minres_alpha(const double *__restrict__ partials, int nbq, FusedState *__restrict__ st) {
     const int q = blockIdx.x;
     double t = 0.0;
     for (int b = threadIdx.x; b < nbq; b += blockDim.x) t += partials[(size_t)q * nbq + b];
-    __shared__ double sm[8];
+    __shared__ double sm[32];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
     if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = t;
@@ -114,33 +120,39 @@ k_minres_alpha(const double *__restrict__ partials, int nbq, FusedState *__restr
 
 // K2b: beta_{j+1} = sqrt(sum of K2a's partials) and the Givens rotation of step j,
 // one block per right-hand side
-__global__ void __launch_bounds__(256)
-k_minres_k2b(const double *__restrict__ partials, int nbq, FusedState *__restrict__ st) {
+__global__ void __launch_bounds__(1024)
+k_minres_k2b(const double *__restrict__ partials, int nbq, int iter, FusedState *__restrict__ st) {
     const int q = blockIdx.x;
     double t = 0.0;
     for (int b = threadIdx.x; b < nbq; b += blockDim.x) t += partials[(size_t)q * nbq + b];
-    __shared__ double sm[8];
+    __shared__ double sm[32];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
     if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = t;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double r2 = 0.0;
+    double r2 = 0.0;
+    if (threadIdx.x == 0)
         for (int w = 0; w < (int)(blockDim.x / 32); ++w) r2 += sm[w];
-        FusedState s = st[q];
-        fused_givens(s, r2);
-        st[q] = s;
-    }
+    fused_givens(st[q], r2, iter);
 }
-
 
 }  // namespace
 
-int minres_fused_batch(Op &op, int N, const float4 *r, float4 *e, float4 *const bufs[6],
-                       FusedState *ms, double *partials, const double *d_tol,
-                       const dlz_params &p, int &iters, HostScratch &hs, bool e_init) {
+// The slab walk of K1 for an N-RHS batch
+static SlabWalk minres_slab_walk(const Op &op, int N) {
+    const Geom &g = op.g;
+    return make_slab_walk(g.L[0] * g.L[1], g.L[2], g.L[3], N, 900.0);
+}
+
+long minres_blocks_per_rhs(const Op &op, int N) {
+    return std::max(slab_blocks(minres_slab_walk(op, N)), (long)(op.g.V + kThreads - 1) / kThreads);
+}
+
+int minres_fused_batch(Op &op, int N, const MinresVectors &b, FusedState *ms, double *partials, const double *d_tol,
+                       const dlz_params &p, int &iters, GraphExec &ge, bool e_init) {
     const long n = 6L * op.g.V;
-    // beta_1 = ||r_q||, rotations reset, a no-op direction update for step 0
+    const float4 *r = b.c[0];
+    // beta_1 = ||r_q||, rotations reset
     DLZ_TRY(reduce32<16>(op, n, [=] __device__(long i, float (&acc)[16]) {
 #pragma unroll
         for (int q = 0; q < 16; ++q)
@@ -150,51 +162,55 @@ int minres_fused_batch(Op &op, int N, const float4 *r, float4 *e, float4 *const 
             fused_init(ms[q], sqrt(res[q]));
         }
     }));
-    // u_j, u_{j-1} (unnormalised Lanczos vectors), w, d_{j-2}, d_{j-3}
-    float4 *U0 = bufs[0], *Up0 = bufs[1], *W0 = bufs[2], *D20 = bufs[3], *D30 = bufs[4];
-    DLZ_CUDA_TRY(cudaMemcpyAsync(U0, r, (size_t)N * n * sizeof(float4), cudaMemcpyDeviceToDevice, op.stream));
-    for (float4 *z : {Up0, D20, D30})
+    // u_0 = r is in place; u_{-1} and the directions start at zero
+    for (float4 *z : {b.c[6], b.d1, b.d2})
         DLZ_CUDA_TRY(cudaMemsetAsync(z, 0, (size_t)N * n * sizeof(float4), op.stream));
-    if (!e_init) DLZ_CUDA_TRY(cudaMemsetAsync(e, 0, (size_t)N * n * sizeof(float4), op.stream));
+    if (!e_init) DLZ_CUDA_TRY(cudaMemsetAsync(b.e, 0, (size_t)N * n * sizeof(float4), op.stream));
     const Geom g = op.g;
     const float kappa = (float)op.kappa;
     const float4 *links = op.gauge32.as<float4>();
-    const unsigned blocks = (unsigned)(((g.V + kThreads - 1) / kThreads) * N);
-    double *partials2 = partials + blocks;    // K2a's partials after K1's
-    DevBuf cnt;                               // per-RHS block counters (reset by their last block)
-    DLZ_TRY(cnt.alloc((size_t)N * sizeof(unsigned)));
-    DLZ_CUDA_TRY(cudaMemsetAsync(cnt.p, 0, (size_t)N * sizeof(unsigned), op.stream));
-    unsigned *counters = cnt.as<unsigned>();
-    auto iteration = [&](float4 *U, float4 *Up, float4 *W, float4 *D2, float4 *D3) -> int {
-        // K1 moves 192 reals per site and right-hand side: u_j, u_{j-1}, d_{j-2}, d_{j-3}, e
-        // read; w, d_{j-1}, e written (24 each), plus the links once per site
-        op.prof.stencil_start(op.stream, true, g.V, N, 192, 1);
+    const SlabWalk w = minres_slab_walk(op, N);
+    const unsigned blocks1 = (unsigned)(slab_blocks(w) * N), blocks = (unsigned)(((g.V + kThreads - 1) / kThreads) * N);
+    const int st1 = blocks1 / N > 512 ? 1024 : 256, st2 = blocks / N > 512 ? 1024 : 256;
+    double *partials2 = partials + minres_blocks_per_rhs(op, N) * N;   // K2a's partials after K1's
+    unsigned *counters = nullptr;             // block counter, reset by the last block
+    if (N == 1) {
         // one right-hand side: the sums are taken by the kernels' last blocks (latency);
         // several: by one-block-per-RHS kernels (cheaper than a tail in every block)
-        unsigned *cn = N == 1 ? counters : nullptr;
-        k_minres_k1<<<blocks, kThreads, 0, op.stream>>>(U, Up, W, D2, D3, e, links, g, kappa, N, ms, partials, cn);
+        counters = reinterpret_cast<unsigned *>(partials2 + minres_blocks_per_rhs(op, N) * N);
+        DLZ_CUDA_TRY(cudaMemsetAsync(counters, 0, sizeof(unsigned), op.stream));
+    }
+    auto iteration = [&](int i) -> int {
+        // K1 moves 72 reals per site and right-hand side: u_j gathered, u_{j-1} read and w
+        // written (24 each), plus the links once per site
+        const float4 *U = b.c[mr_u(i)];
+        float4 *W = b.c[mr_w(i)];
+        if (i == kMrBlock - 1) {
+            k_minres_directions<false><<<dim3((unsigned)((n + 255) / 256), N), 256, 0, op.stream>>>(b, ms, n);
+            op.prof.launches++;
+        }
+        op.prof.stencil_start(op.stream, true, g.V, N, 72, 1);
+        k_minres_k1<<<blocks1, kThreads, 0, op.stream>>>(U, b.c[mr_up(i)], W, links, g, w, kappa, N, ms, partials,
+                                                        counters);
         op.prof.stencil_stop(op.stream);
-        if (!cn) k_minres_alpha<<<N, 256, 0, op.stream>>>(partials, (int)(blocks / N), ms);
-        op.prof.launches += cn ? 1 : 2;
+        if (!counters) k_minres_alpha<<<N, st1, 0, op.stream>>>(partials, (int)(blocks1 / N), ms);
+        op.prof.launches += counters ? 1 : 2;
         DLZ_CUDA_TRY(cudaGetLastError());
         // u_{j+1} = w - alpha v_j ; beta_{j+1} ; Givens rotation of step j
-        k_minres_k2a<<<blocks, kThreads, 0, op.stream>>>(W, U, g, N, ms, partials2, cn);
-        if (!cn) k_minres_k2b<<<N, 256, 0, op.stream>>>(partials2, (int)(blocks / N), ms);
-        op.prof.launches += cn ? 1 : 2;
+        k_minres_k2a<<<blocks, kThreads, 0, op.stream>>>(W, U, b.c[mr_out(i)], i == kMrBlock - 1 ? b.c[6] : nullptr, g,
+                                                        N, i, ms, partials2, counters);
+        if (!counters) k_minres_k2b<<<N, st2, 0, op.stream>>>(partials2, (int)(blocks / N), i, ms);
+        op.prof.launches += counters ? 1 : 2;
         DLZ_CUDA_TRY(cudaGetLastError());
         return DLZ_OK;
     };
-    GraphExec ge;
     auto six = [&]() -> int {
-        float4 *U = U0, *Up = Up0, *W = W0, *D2 = D20, *D3 = D30;
-        for (int sub = 0; sub < 6; ++sub) {
-            DLZ_TRY(iteration(U, Up, W, D2, D3));
-            float4 *tUp = Up;
-            Up = U; U = W; W = tUp;               // (U, Up, W) -> (W, U, Up): period 3
-            std::swap(D2, D3);                     // period 2
-        }
+        for (int i = 0; i < kMrBlock; ++i) DLZ_TRY(iteration(i));
         return DLZ_OK;
     };
+    std::vector<FusedState> h(N);
+    std::vector<double> tol(N);
+    DLZ_TRY(d2h_sync(op, tol.data(), d_tol, N * sizeof(double)));
     const int check = std::max(6, (p.check_every / 6) * 6);
     int it = 0;
     // DLZ_TRACE=1: time the replays of the 6-iteration group (diagnostics)
@@ -221,16 +237,12 @@ int minres_fused_batch(Op &op, int N, const float4 *r, float4 *e, float4 *const 
         iters += 6;
         it += 6;
         if (it % check == 0 || iters >= p.max_iter) {
-            DLZ_TRY(d2h_sync(op, hs.p, ms, N * sizeof(FusedState)));
+            DLZ_TRY(d2h_sync(op, h.data(), ms, N * sizeof(FusedState)));
             ge.sample(op.prof);
-            const FusedState *h = reinterpret_cast<const FusedState *>(hs.p);
             bool done = true;
-            for (int q = 0; q < N; ++q)
-                if (!std::isfinite(h[q].phibar)) return fail(DLZ_ERR_NONFINITE, "MinRes residual not finite");
-            DLZ_TRY(d2h_sync(op, hs.p + 512, d_tol, N * sizeof(double)));
             for (int q = 0; q < N; ++q) {
-                const FusedState *hq = reinterpret_cast<const FusedState *>(hs.p) + q;
-                if (!(std::fabs(hq->phibar) <= hs.p[512 + q] * hq->r0 || hq->beta_next == 0.0)) done = false;
+                if (!std::isfinite(h[q].phibar)) return fail(DLZ_ERR_NONFINITE, "MinRes residual not finite");
+                if (!(std::fabs(h[q].phibar) <= tol[q] * h[q].r0 || h[q].beta_next == 0.0)) done = false;
             }
             if (done) break;
         }
@@ -239,16 +251,10 @@ int minres_fused_batch(Op &op, int N, const float4 *r, float4 *e, float4 *const 
         std::fprintf(stderr, "[dlz] fused MinRes N=%d: %d iterations, graph replay %.4f ms per iteration (%d timed)\n",
                      N, iters, n_timed ? t_graph / (6.0 * n_timed) : 0.0, n_timed);
     }
-    // the direction update of the last step (after 6k steps the buffers are back
-    // in their starting roles: u_J in Up, d_{J-1} in D2, d_{J-2} in D3; v_J = u_J / beta_J)
-    {
-        const float4 *vj = Up0, *d2 = D20, *d3 = D30;
-        float4 *ee = e;
-        DLZ_TRY(map(op, n * N, [=] __device__(long i) {
-            const int q = (int)(i / n);
-            minres_last_direction(vj[i], d2[i], d3[i], ee[i], ms[q]);
-        }));
-    }
+    // the direction update of the last step
+    k_minres_directions<true><<<dim3((unsigned)((n + 255) / 256), N), 256, 0, op.stream>>>(b, ms, n);
+    op.prof.launches++;
+    DLZ_CUDA_TRY(cudaGetLastError());
     return DLZ_OK;
 }
 

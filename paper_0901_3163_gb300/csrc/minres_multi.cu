@@ -108,7 +108,6 @@ k_mm_init(const double *__restrict__ partials, const SlotDesc *__restrict__ sd, 
 template <int B>
 __global__ void __launch_bounds__(B * kMT)
 k_mm_k1(const float4 *__restrict__ U, const float4 *__restrict__ Up, float4 *__restrict__ W,
-        const float4 *__restrict__ D2, float4 *__restrict__ D3, float4 *__restrict__ E,
         const SlotDesc *__restrict__ sd, const int2 *__restrict__ table, const FusedState *__restrict__ st,
         const int *__restrict__ active, double *__restrict__ partials) {
     const int2 t = table[blockIdx.x];
@@ -121,9 +120,27 @@ k_mm_k1(const float4 *__restrict__ U, const float4 *__restrict__ Up, float4 *__r
     const int s = t.y * kMT + threadIdx.x;
     float facc = 0.f;
     if (s < d.g.V)
-        facc = minres_k1_site(s, d.g, d.kappa, U + d.off, Up + d.off, W + d.off, D2 + d.off, D3 + d.off,
-                              E + d.off, d.links, st[t.x]);
+        facc = minres_k1_site(s, d.g, d.kappa, U + d.off, Up + d.off, W + d.off, d.links, st[t.x]);
     chunk_partials<B>(facc, partials + d.blk0 + t.y, d.nb - t.y);
+}
+
+// the deferred update of a block of iterations (minres_state.cuh); LAST: of the one step
+// left at the end, for every slot (a finished slot's step is still in its state)
+template <int B, bool LAST>
+__global__ void __launch_bounds__(B * kMT)
+k_mm_directions(MinresVectors v, const SlotDesc *__restrict__ sd, const int2 *__restrict__ table,
+                const FusedState *__restrict__ st, const int *__restrict__ active) {
+    const int2 t = table[blockIdx.x];
+    const SlotDesc d = sd[t.x];
+    if (!LAST && !active[t.x]) return;
+    const int s = t.y * kMT + threadIdx.x;
+    if (s >= d.g.V) return;
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+        const size_t i = d.off + (size_t)c * d.g.V + s;
+        if (LAST) minres_last_direction(v, i, st[t.x]);
+        else minres_directions_elem(v, i, st[t.x]);
+    }
 }
 
 __global__ void __launch_bounds__(256)
@@ -137,7 +154,7 @@ k_mm_alpha(const double *__restrict__ partials, const SlotDesc *__restrict__ sd,
 
 template <int B>
 __global__ void __launch_bounds__(B * kMT)
-k_mm_k2a(float4 *__restrict__ W, const float4 *__restrict__ U, const SlotDesc *__restrict__ sd,
+k_mm_k2a(const float4 *W, const float4 *U, float4 *Out, float4 *Copy, const SlotDesc *__restrict__ sd,
          const int2 *__restrict__ table, const FusedState *__restrict__ st, const int *__restrict__ active,
          double *__restrict__ partials) {
     const int2 t = table[blockIdx.x];
@@ -149,40 +166,18 @@ k_mm_k2a(float4 *__restrict__ W, const float4 *__restrict__ U, const SlotDesc *_
     }
     const int s = t.y * kMT + threadIdx.x;
     float facc = 0.f;
-    if (s < d.g.V) facc = minres_k2a_site(s, d.g.V, W + d.off, U + d.off, st[t.x]);
+    if (s < d.g.V)
+        facc = minres_k2a_site(s, d.g.V, W + d.off, U + d.off, Out + d.off, Copy ? Copy + d.off : nullptr, st[t.x]);
     chunk_partials<B>(facc, partials + d.blk0 + t.y, d.nb - t.y);
 }
 
 __global__ void __launch_bounds__(256)
 k_mm_k2b(const double *__restrict__ partials, const SlotDesc *__restrict__ sd, FusedState *__restrict__ st,
-         const int *__restrict__ active) {
+         const int *__restrict__ active, int iter) {
     if (!active[blockIdx.x]) return;
     const SlotDesc d = sd[blockIdx.x];
     const double r2 = slot_sum(partials, d.blk0, d.nb);
-    if (threadIdx.x == 0) {
-        FusedState s = st[blockIdx.x];
-        fused_givens(s, r2);
-        st[blockIdx.x] = s;
-    }
-}
-
-template <int B>
-__global__ void __launch_bounds__(B * kMT)
-k_mm_last(const float4 *__restrict__ Uj, const float4 *__restrict__ D2, const float4 *__restrict__ D3,
-          float4 *__restrict__ E, const SlotDesc *__restrict__ sd, const int2 *__restrict__ table,
-          const FusedState *__restrict__ st) {
-    const int2 t = table[blockIdx.x];
-    const SlotDesc d = sd[t.x];
-    const int s = t.y * kMT + threadIdx.x;
-    if (s >= d.g.V) return;
-    const FusedState q = st[t.x];
-#pragma unroll
-    for (int c = 0; c < 6; ++c) {
-        const size_t i = d.off + (size_t)c * d.g.V + s;
-        float4 ev = E[i];
-        minres_last_direction(Uj[i], D2[i], D3[i], ev, q);
-        E[i] = ev;
-    }
+    fused_givens(st[blockIdx.x], r2, iter);
 }
 
 // ------------------------------------------------------------------ persistent form
@@ -236,14 +231,13 @@ __device__ inline bool grid_wait(GridBar *gb, long long limit) {
 // both forms give the same bits), and the kernel ends once every slot is frozen.
 template <int B>
 __global__ void __launch_bounds__(B * kMT)
-k_mm_persistent(float4 *__restrict__ U0, float4 *__restrict__ Up0, float4 *__restrict__ W0, float4 *__restrict__ D20,
-                float4 *__restrict__ D30, float4 *__restrict__ E, const SlotDesc *__restrict__ sd,
-                const int2 *__restrict__ table, int ntab, int NS, FusedState *__restrict__ st, int *__restrict__ active,
+k_mm_persistent(MinresVectors v, const SlotDesc *__restrict__ sd, const int2 *__restrict__ table, int ntab, int NS, FusedState *__restrict__ st, int *__restrict__ active,
                 double *__restrict__ partials, double *__restrict__ partials2, const double *__restrict__ tol,
                 int it0, int check, int ngroups, GridBar *gb, long long limit) {
-    float4 *U = U0, *Up = Up0, *W = W0, *D2 = D20, *D3 = D30;
     for (int grp = 0; grp < ngroups; ++grp) {
-        for (int sub = 0; sub < 6; ++sub) {
+        for (int sub = 0; sub < kMrBlock; ++sub) {
+            const float4 *U = v.c[mr_u(sub)], *Up = v.c[mr_up(sub)];
+            float4 *W = v.c[mr_w(sub)], *Out = v.c[mr_out(sub)], *Copy = sub == kMrBlock - 1 ? v.c[6] : nullptr;
             for (int item = blockIdx.x; item < ntab; item += gridDim.x) {
                 const int2 t = table[item];
                 const SlotDesc d = sd[t.x];
@@ -254,9 +248,14 @@ k_mm_persistent(float4 *__restrict__ U0, float4 *__restrict__ Up0, float4 *__res
                 }
                 const int s = t.y * kMT + threadIdx.x;
                 float facc = 0.f;
-                if (s < d.g.V)
-                    facc = minres_k1_site(s, d.g, d.kappa, U + d.off, Up + d.off, W + d.off, D2 + d.off, D3 + d.off,
-                                          E + d.off, d.links, st[t.x]);
+                if (s < d.g.V) {
+                    // the block's deferred update reads c[6] at this site, which K1 overwrites
+                    // (as the separate launch before K1 in the graph form)
+                    if (sub == kMrBlock - 1)
+                        for (int c = 0; c < 6; ++c)
+                            minres_directions_elem(v, d.off + (size_t)c * d.g.V + s, st[t.x]);
+                    facc = minres_k1_site(s, d.g, d.kappa, U + d.off, Up + d.off, W + d.off, d.links, st[t.x]);
+                }
                 chunk_partials<B>(facc, partials + d.blk0 + t.y, d.nb - t.y);
             }
             if (!grid_wait(gb, limit)) return;
@@ -278,7 +277,9 @@ k_mm_persistent(float4 *__restrict__ U0, float4 *__restrict__ Up0, float4 *__res
                 }
                 const int s = t.y * kMT + threadIdx.x;
                 float facc = 0.f;
-                if (s < d.g.V) facc = minres_k2a_site(s, d.g.V, W + d.off, U + d.off, st[t.x]);
+                if (s < d.g.V)
+                    facc = minres_k2a_site(s, d.g.V, W + d.off, U + d.off, Out + d.off, Copy ? Copy + d.off : nullptr,
+                                           st[t.x]);
                 chunk_partials<B>(facc, partials2 + d.blk0 + t.y, d.nb - t.y);
             }
             if (!grid_wait(gb, limit)) return;
@@ -286,17 +287,9 @@ k_mm_persistent(float4 *__restrict__ U0, float4 *__restrict__ Up0, float4 *__res
                 if (!active[q]) continue;
                 const SlotDesc d = sd[q];
                 const double r2 = slot_sum(partials2, d.blk0, d.nb);
-                if (threadIdx.x == 0) {
-                    FusedState v = st[q];
-                    fused_givens(v, r2);
-                    st[q] = v;
-                }
-                __syncthreads();
+                fused_givens(st[q], r2, sub);
             }
             if (!grid_wait(gb, limit)) return;
-            float4 *tUp = Up;
-            Up = U; U = W; W = tUp;
-            float4 *tD = D2; D2 = D3; D3 = tD;
         }
         const int it = it0 + 6 * (grp + 1);
         if (blockIdx.x == 0 && threadIdx.x == 0) gb->groups = grp + 1;
@@ -305,8 +298,8 @@ k_mm_persistent(float4 *__restrict__ U0, float4 *__restrict__ Up0, float4 *__res
         // read the same flags after the barrier
         for (int q = blockIdx.x; q < NS; q += gridDim.x)
             if (threadIdx.x == 0 && active[q]) {
-                const FusedState v = st[q];
-                if (fabs(v.phibar) <= tol[q] * v.r0 || v.beta_next == 0.0) active[q] = 0;
+                const FusedState &f = st[q];
+                if (fabs(f.phibar) <= tol[q] * f.r0 || f.beta_next == 0.0) active[q] = 0;
             }
         if (!grid_wait(gb, limit)) return;
         __shared__ int any;
@@ -329,26 +322,30 @@ struct Tile {
     int nblocks;
 };
 
-// The fused FP32 MinRes over all slots (r: normalised residuals in the arena; e:
-// corrections, holding the start if e_init).  bufs: 5 arena-sized work vectors.
+// The fused FP32 MinRes over all slots (minres_state.cuh: v.c[0] holds the normalised
+// residuals; v.e the corrections, holding the start if e_init).
 // A slot whose inner residual has met its tolerance at a check is frozen: its blocks
-// return at once and its state stops changing (the buffer roles repeat every 6
-// iterations and checks fall on multiples of 6, so the frozen slot's pending
-// direction update is still found where k_mm_last looks for it).
-// Tiles: the first three 6-iteration groups capture a graph per tile (128, 256 and
-// 512 threads per block), the next three time one replay each (CUDA events), and the
-// fastest serves the rest (DLZ_MULTI_TILE=1|2|4 forces one).  The partials are per
-// 128-site chunk whatever the tile, so every tile gives bit-identical results.
+// return at once and its state stops changing (checks fall on multiples of a block of 6
+// iterations, where every slot's vectors are in the same buffers, so the frozen slot's
+// pending direction is still found where k_mm_directions<.., true> looks for it).
+// The launch form is chosen once per call: MultiRun keeps the choice and the captured
+// graphs from one inner solve of the defect correction to the next (the autotuner's nine
+// candidates, run again in every inner solve, took 180 of 563 ms on nine lattices of
+// 8^4 .. 16^4 with 8 right-hand sides).
+struct MultiRun {
+    GraphExec ge[3];         // the graph form's block of iterations, by tile
+    int best = -1;           // the chosen candidate (-1: not chosen yet)
+};
 // persistent launch of up to `ngroups` 6-iteration groups with B chunks per work item and
 // `grid` blocks; returns the groups run (device count) or a DLZ error
-static int launch_persistent(Op &op, int B, int grid, float4 *U0, float4 *Up0, float4 *W0, float4 *D20, float4 *D30,
-                             float4 *e, const SlotDesc *sd, const Tile &t, int NS, FusedState *ms, int *active,
+static int launch_persistent(Op &op, int B, int grid, const MinresVectors &vec, const SlotDesc *sd, const Tile &t, int NS, FusedState *ms, int *active,
                              double *partials, double *partials2, const double *d_tol, int it0, int check, int ngroups,
                              GridBar *gb, long long limit, int &groups_run) {
     DLZ_CUDA_TRY(cudaMemsetAsync(gb, 0, sizeof(GridBar), op.stream));
     int ntab = t.nblocks;
     const int2 *table = t.table;
-    void *args[] = {&U0, &Up0, &W0, &D20, &D30, &e, (void *)&sd, (void *)&table, &ntab, &NS, &ms, &active,
+    MinresVectors v = vec;
+    void *args[] = {&v, (void *)&sd, (void *)&table, &ntab, &NS, &ms, &active,
                     &partials, &partials2, (void *)&d_tol, &it0, &check, &ngroups, &gb, &limit};
     void *fn = B == 1 ? (void *)k_mm_persistent<1> : B == 2 ? (void *)k_mm_persistent<2> : (void *)k_mm_persistent<4>;
     DLZ_CUDA_TRY(cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(B * kMT), args, 0, op.stream));
@@ -373,45 +370,40 @@ static int persistent_grid(int B, int frac_half) {
 }
 
 int minres_multi_batch(Op &op, int NS, const SlotDesc *sd, const Tile *tiles, int nchunks, size_t arena,
-                       const float4 *r, float4 *e, float4 *const bufs[5], FusedState *ms, double *partials,
-                       int *active, const double *d_tol, const dlz_params &p, int &iters, bool e_init,
-                       GridBar *gb) {
+                       const MinresVectors &v, FusedState *ms, double *partials, int *active, const double *d_tol,
+                       const dlz_params &p, int &iters, GridBar *gb, MultiRun &run) {
     double *partials2 = partials + nchunks;
-    k_mm_norm<1><<<tiles[0].nblocks, kMT, 0, op.stream>>>(r, sd, tiles[0].table, partials);
+    k_mm_norm<1><<<tiles[0].nblocks, kMT, 0, op.stream>>>(v.c[0], sd, tiles[0].table, partials);
     k_mm_init<<<NS, 256, 0, op.stream>>>(partials, sd, ms);
     op.prof.launches += 2;
     DLZ_CUDA_TRY(cudaGetLastError());
-    float4 *U0 = bufs[0], *Up0 = bufs[1], *W0 = bufs[2], *D20 = bufs[3], *D30 = bufs[4];
-    DLZ_CUDA_TRY(cudaMemcpyAsync(U0, r, arena * sizeof(float4), cudaMemcpyDeviceToDevice, op.stream));
-    for (float4 *z : {Up0, D20, D30}) DLZ_CUDA_TRY(cudaMemsetAsync(z, 0, arena * sizeof(float4), op.stream));
-    if (!e_init) DLZ_CUDA_TRY(cudaMemsetAsync(e, 0, arena * sizeof(float4), op.stream));
-    auto iteration = [&](const Tile &t, float4 *U, float4 *Up, float4 *W, float4 *D2, float4 *D3) -> int {
+    for (float4 *z : {v.c[6], v.d1, v.d2}) DLZ_CUDA_TRY(cudaMemsetAsync(z, 0, arena * sizeof(float4), op.stream));
+    auto iteration = [&](const Tile &t, int i) -> int {
+        const float4 *U = v.c[mr_u(i)], *Up = v.c[mr_up(i)];
+        float4 *W = v.c[mr_w(i)], *Out = v.c[mr_out(i)], *Copy = i == kMrBlock - 1 ? v.c[6] : nullptr;
+        if (i == kMrBlock - 1) {
+            k_mm_directions<1, false><<<tiles[0].nblocks, kMT, 0, op.stream>>>(v, sd, tiles[0].table, ms, active);
+            op.prof.launches++;
+        }
         switch (t.B) {
-        case 1: k_mm_k1<1><<<t.nblocks, kMT, 0, op.stream>>>(U, Up, W, D2, D3, e, sd, t.table, ms, active, partials); break;
-        case 2: k_mm_k1<2><<<t.nblocks, 2 * kMT, 0, op.stream>>>(U, Up, W, D2, D3, e, sd, t.table, ms, active, partials); break;
-        default: k_mm_k1<4><<<t.nblocks, 4 * kMT, 0, op.stream>>>(U, Up, W, D2, D3, e, sd, t.table, ms, active, partials);
+        case 1: k_mm_k1<1><<<t.nblocks, kMT, 0, op.stream>>>(U, Up, W, sd, t.table, ms, active, partials); break;
+        case 2: k_mm_k1<2><<<t.nblocks, 2 * kMT, 0, op.stream>>>(U, Up, W, sd, t.table, ms, active, partials); break;
+        default: k_mm_k1<4><<<t.nblocks, 4 * kMT, 0, op.stream>>>(U, Up, W, sd, t.table, ms, active, partials);
         }
         k_mm_alpha<<<NS, 256, 0, op.stream>>>(partials, sd, ms, active);
         switch (t.B) {
-        case 1: k_mm_k2a<1><<<t.nblocks, kMT, 0, op.stream>>>(W, U, sd, t.table, ms, active, partials2); break;
-        case 2: k_mm_k2a<2><<<t.nblocks, 2 * kMT, 0, op.stream>>>(W, U, sd, t.table, ms, active, partials2); break;
-        default: k_mm_k2a<4><<<t.nblocks, 4 * kMT, 0, op.stream>>>(W, U, sd, t.table, ms, active, partials2);
+        case 1: k_mm_k2a<1><<<t.nblocks, kMT, 0, op.stream>>>(W, U, Out, Copy, sd, t.table, ms, active, partials2); break;
+        case 2: k_mm_k2a<2><<<t.nblocks, 2 * kMT, 0, op.stream>>>(W, U, Out, Copy, sd, t.table, ms, active, partials2); break;
+        default: k_mm_k2a<4><<<t.nblocks, 4 * kMT, 0, op.stream>>>(W, U, Out, Copy, sd, t.table, ms, active, partials2);
         }
-        k_mm_k2b<<<NS, 256, 0, op.stream>>>(partials2, sd, ms, active);
+        k_mm_k2b<<<NS, 256, 0, op.stream>>>(partials2, sd, ms, active, i);
         op.prof.launches += 4;
         DLZ_CUDA_TRY(cudaGetLastError());
         return DLZ_OK;
     };
-    GraphExec ge[3];
     int cur = 0;
     auto six = [&]() -> int {
-        float4 *U = U0, *Up = Up0, *W = W0, *D2 = D20, *D3 = D30;
-        for (int sub = 0; sub < 6; ++sub) {
-            DLZ_TRY(iteration(tiles[cur], U, Up, W, D2, D3));
-            float4 *tUp = Up;
-            Up = U; U = W; W = tUp;
-            std::swap(D2, D3);
-        }
+        for (int i = 0; i < kMrBlock; ++i) DLZ_TRY(iteration(tiles[cur], i));
         return DLZ_OK;
     };
     // Autotuner over the launch forms: the graph form with 1, 2 or 4 chunks of 128 sites
@@ -454,14 +446,16 @@ int minres_multi_batch(Op &op, int NS, const SlotDesc *sd, const Tile *tiles, in
     DLZ_TRY(d2h_sync(op, tol.data(), d_tol, NS * sizeof(double)));
     std::vector<int> act(NS, 1);
     DLZ_TRY(h2d(op, active, act.data(), NS * sizeof(int)));
-    // the schedule: capture (graph candidates), then one timed group per candidate, then the best
+    // the schedule of the call's first inner solve: capture (graph candidates), then one timed
+    // group per candidate, then the best; later inner solves start with the best
     std::vector<int> sched;
+    const bool search = cands.size() > 1 && run.best < 0;
     for (size_t c = 0; c < cands.size(); ++c)
-        if (cands[c].form == 0 && cands.size() > 1) sched.push_back((int)c);      // capture groups (untimed)
+        if (cands[c].form == 0 && search) sched.push_back((int)c);                // capture groups (untimed)
     const size_t ncapture = sched.size();
-    if (cands.size() > 1)
+    if (search)
         for (size_t c = 0; c < cands.size(); ++c) sched.push_back((int)c);        // timed groups
-    int it = 0, group = 0, best = 0;
+    int it = 0, group = 0, best = std::max(0, run.best);
     bool all_done = false;
     auto host_check = [&]() -> int {
         DLZ_TRY(d2h_sync(op, h.data(), ms, NS * sizeof(FusedState)));
@@ -484,7 +478,7 @@ int minres_multi_batch(Op &op, int NS, const SlotDesc *sd, const Tile *tiles, in
         if (c.form == 0) {
             cur = c.tile;
             if (timed) DLZ_CUDA_TRY(cudaEventRecord(ev0.e, op.stream));
-            DLZ_TRY(run_graph(op, ge[cur], six));
+            DLZ_TRY(run_graph(op, run.ge[cur], six));
             if (timed) DLZ_CUDA_TRY(cudaEventRecord(ev1.e, op.stream));
             iters += 6;
             it += 6;
@@ -494,7 +488,7 @@ int minres_multi_batch(Op &op, int NS, const SlotDesc *sd, const Tile *tiles, in
             const int ngroups = tuning ? 1 : std::max(1, (p.max_iter - iters + 5) / 6);
             int ran = 0;
             if (timed) DLZ_CUDA_TRY(cudaEventRecord(ev0.e, op.stream));
-            DLZ_TRY(launch_persistent(op, 1 << c.tile, c.grid, U0, Up0, W0, D20, D30, e, sd, tiles[c.tile], NS, ms,
+            DLZ_TRY(launch_persistent(op, 1 << c.tile, c.grid, v, sd, tiles[c.tile], NS, ms,
                                       active, partials, partials2, d_tol, it, check, ngroups, gb, limit, ran));
             if (timed) DLZ_CUDA_TRY(cudaEventRecord(ev1.e, op.stream));
             iters += 6 * ran;
@@ -512,14 +506,16 @@ int minres_multi_batch(Op &op, int NS, const SlotDesc *sd, const Tile *tiles, in
                 cudaGetLastError();
                 tms[ci] = 1e30f;
             }
-            if ((size_t)group + 1 == sched.size())
-                for (size_t v = 0; v < cands.size(); ++v)
-                    if (tms[v] < tms[best]) best = (int)v;
+            if ((size_t)group + 1 == sched.size()) {
+                for (size_t k = 0; k < cands.size(); ++k)
+                    if (tms[k] < tms[best]) best = (int)k;
+                run.best = best;
+            }
         }
         ++group;
     }
     op.multi_choice = cands[best].form * 100 + (1 << cands[best].tile) * 10 + cands[best].half;
-    k_mm_last<1><<<tiles[0].nblocks, kMT, 0, op.stream>>>(Up0, D20, D30, e, sd, tiles[0].table, ms);
+    k_mm_directions<1, true><<<tiles[0].nblocks, kMT, 0, op.stream>>>(v, sd, tiles[0].table, ms, active);
     op.prof.launches += 1;
     DLZ_CUDA_TRY(cudaGetLastError());
     return DLZ_OK;
@@ -559,7 +555,7 @@ int dminres_multi(int nlat, Op *const *ops, const dlz_defl_s *const *defls, cons
     const int NS = (int)hsd.size();
     if (NS == 0) return DLZ_OK;
     Op &op = *ops[0];
-    DevBuf dsd, dtab[3], f32, part, scal, gbar;
+    DevBuf dsd, dtab[3], f32, fr, ft, part, scal, gbar;
     DLZ_TRY(gbar.alloc(sizeof(GridBar)));
     DLZ_TRY(dsd.alloc(NS * sizeof(SlotDesc)));
     Tile tiles[3];
@@ -573,13 +569,22 @@ int dminres_multi(int nlat, Op *const *ops, const dlz_defl_s *const *defls, cons
     DLZ_TRY(scal.alloc((size_t)NS * (sizeof(FusedState) + 2 * sizeof(double) + sizeof(int))));
     DLZ_TRY(h2d(op, dsd.p, hsd.data(), NS * sizeof(SlotDesc)));
     float4 *r32 = f32.as<float4>(), *e32 = r32 + arena;
-    float4 *const bufs[5] = {r32 + 2 * arena, r32 + 3 * arena, r32 + 4 * arena, r32 + 5 * arena, r32 + 6 * arena};
+    // FP64 residuals and Q x of every slot.  Both are idle during an inner solve, so its
+    // directions and one of its Lanczos vectors lie in them (an FP64 vector holds two)
+    DLZ_TRY(fr.alloc(2 * arena * sizeof(float4)));
+    DLZ_TRY(ft.alloc(2 * arena * sizeof(float4)));
+    float4 *t32 = ft.as<float4>();
+    const MinresVectors mv = {{r32, r32 + 2 * arena, r32 + 3 * arena, r32 + 4 * arena, r32 + 5 * arena,
+                               r32 + 6 * arena, fr.as<float4>()},
+                              t32, t32 + arena, e32};
+    MultiRun run;
     FusedState *ms = reinterpret_cast<FusedState *>(scal.p);
     double *d_tol = reinterpret_cast<double *>(ms + NS);
     int *d_active = reinterpret_cast<int *>(d_tol + 2 * NS);
-    // per-lattice FP64 work: b' = gamma5 b, x, r, Q x
+    // per-lattice FP64 work: b' = gamma5 b, x, r, Q x (r and t in the arenas above)
     struct Lat {
-        DevBuf bp, x, r, t, dots, nrm;
+        DevBuf bp, x, dots, nrm;
+        double2 *r = nullptr, *t = nullptr;
         std::vector<double> bn, rn;
     };
     std::vector<Lat> L(nlat);
@@ -591,8 +596,11 @@ int dminres_multi(int nlat, Op *const *ops, const dlz_defl_s *const *defls, cons
         Lat &a = L[l];
         DLZ_TRY(a.bp.alloc((size_t)N * n64 * sizeof(double2)));
         DLZ_TRY(a.x.alloc((size_t)N * n64 * sizeof(double2)));
-        DLZ_TRY(a.r.alloc((size_t)N * n64 * sizeof(double2)));
-        DLZ_TRY(a.t.alloc((size_t)N * n64 * sizeof(double2)));
+        if (N > 0) {
+            // slot offsets count float4 of FP32 vectors: an FP64 vector takes twice as many bytes
+            a.r = fr.as<double2>() + 2 * hsd[lat_slot0[l]].off;
+            a.t = ft.as<double2>() + 2 * hsd[lat_slot0[l]].off;
+        }
         DLZ_TRY(a.nrm.alloc(16 * sizeof(double)));
         if (defls[l] && defls[l]->k > 0) {
             DLZ_TRY(a.dots.alloc((size_t)N * defls[l]->k * sizeof(double2)));
@@ -630,9 +638,9 @@ int dminres_multi(int nlat, Op *const *ops, const dlz_defl_s *const *defls, cons
             Lat &a = L[l];
             const int N = nrhs[l];
             const long n64 = 12L * o.g.V;
-            DLZ_TRY(wilson64_batch(o, a.t.as<double2>(), a.x.as<double2>(), DLZ_Q, N));
-            const double2 *pbp = a.bp.as<double2>(), *pt = a.t.as<double2>();
-            double2 *pr = a.r.as<double2>();
+            DLZ_TRY(wilson64_batch(o, a.t, a.x.as<double2>(), DLZ_Q, N));
+            const double2 *pbp = a.bp.as<double2>(), *pt = a.t;
+            double2 *pr = a.r;
             double *dn = a.nrm.as<double>();
             DLZ_TRY(reduce<16>(o, n64, [=] __device__(long i, double (&acc)[16]) {
 #pragma unroll
@@ -670,7 +678,7 @@ int dminres_multi(int nlat, Op *const *ops, const dlz_defl_s *const *defls, cons
             const int V = o.g.V;
             const long n64 = 12L * V, n32 = 6L * V;
             float4 *rl = r32 + hsd[lat_slot0[l]].off, *el = e32 + hsd[lat_slot0[l]].off;
-            const double2 *pr = a.r.as<double2>();
+            const double2 *pr = a.r;
             Scales16 scv;
             for (int r = 0; r < N; ++r) scv.v[r] = inv[lat_slot0[l] + r];
             DLZ_TRY(map(o, n32 * N, [=] __device__(long i) {
@@ -700,7 +708,7 @@ int dminres_multi(int nlat, Op *const *ops, const dlz_defl_s *const *defls, cons
                 DLZ_TRY(h2d(o, pd, hc.data(), hc.size() * sizeof(double2)));
                 for (int r = 0; r < N; ++r)
                     DLZ_TRY(combine<P32>(o, el + (size_t)r * n32, n32, 1, V32, n32, k, pd + (size_t)r * k, 1, false, false));
-                float4 *qe = bufs[0] + hsd[lat_slot0[l]].off;      // scratch: Q e0
+                float4 *qe = mv.c[1] + hsd[lat_slot0[l]].off;      // scratch: Q e0
                 DLZ_TRY(wilson32_batch(o, qe, el, DLZ_Q, N));
                 DLZ_TRY(map(o, n32 * N, [=] __device__(long i) {
                     const float4 u = rl[i], w = qe[i];
@@ -712,8 +720,8 @@ int dminres_multi(int nlat, Op *const *ops, const dlz_defl_s *const *defls, cons
             DLZ_CUDA_TRY(cudaStreamSynchronize(o.stream));
         }
         DLZ_TRY(h2d(op, d_tol, tl.data(), NS * sizeof(double)));
-        DLZ_TRY(minres_multi_batch(op, NS, dsd.as<SlotDesc>(), tiles, nchunks, arena, r32, e32, bufs, ms,
-                                   part.as<double>(), d_active, d_tol, p, iters, true, gbar.as<GridBar>()));
+        DLZ_TRY(minres_multi_batch(op, NS, dsd.as<SlotDesc>(), tiles, nchunks, arena, mv, ms, part.as<double>(),
+                                   d_active, d_tol, p, iters, gbar.as<GridBar>(), run));
         DLZ_CUDA_TRY(cudaStreamSynchronize(op.stream));
         // x += ||r|| e, lattice by lattice
         for (int l = 0; l < nlat; ++l) {

@@ -64,14 +64,18 @@ int build_deflation(Op &op, int which, const double2 *Vk, int k, dlz_defl_s **ou
 int deflation_factor(Op &op, dlz_defl_s *d);
 int prepare_kernels(Op &op);
 struct FusedState;
-struct HostScratch;
-// Fused two-kernel FP32 MinRes on N right-hand sides (minres_fused.cu).
-// e_init: e holds a starting guess (r is then the residual of that guess).
-int minres_fused_batch(Op &op, int N, const float4 *r, float4 *e, float4 *const bufs[6],
-                       FusedState *ms, double *partials, const double *d_tol,
-                       const dlz_params &p, int &iters, HostScratch &hs, bool e_init = false);
+struct MinresVectors;
+struct GraphExec;
+// Fused two-kernel FP32 MinRes on N right-hand sides (minres_fused.cu): b.c[0] holds the
+// right-hand sides and is overwritten; e_init: b.e holds a starting guess (b.c[0] is then
+// the residual of that guess).  partials: 2 minres_blocks_per_rhs N + 1 doubles.  ge: the
+// graph of a block of iterations, empty or of an earlier call with the same arguments.
+long minres_blocks_per_rhs(const Op &op, int N);
+int minres_fused_batch(Op &op, int N, const MinresVectors &b, FusedState *ms, double *partials, const double *d_tol,
+                       const dlz_params &p, int &iters, GraphExec &ge, bool e_init = false);
 // Fused FP32 CG on the normal equations for D e = s0 on N right-hand sides
 // (cg_fused.cu); s0 is read only at the start, e is updated in place (holds the start).
+// ge as in minres_fused_batch.
 struct CgFusedState;
 size_t cg_state_bytes();
 constexpr int kCgResiduals = 6;
@@ -84,7 +88,7 @@ struct CgBuffers {
 // their partials arrays)
 long cgnr_blocks_per_rhs(const Op &op, int N);
 int cgnr_fused_batch(Op &op, int N, const float4 *s0, float4 *e, const CgBuffers &bufs, CgFusedState *ms,
-                     double *partials, const double *d_tol, const dlz_params &p, int &iters);
+                     double *partials, const double *d_tol, const dlz_params &p, int &iters, GraphExec &ge);
 // FP32 D-MinRes with FP64 defect correction on many lattices at once
 // (minres_multi.cu); B[l], X[l]: nrhs[l] <= 16 internal FP64 vectors of lattice l,
 // st: one entry per (lattice, right-hand side) in order.

@@ -61,13 +61,11 @@ int dsolve_mixed_batch(Op &op, const dlz_defl_s *d, bool minres, const double2 *
         DLZ_TRY(pdot.alloc((size_t)N * d->k * sizeof(double2)));
         DLZ_TRY(reserve_multidot(op, d->k));
     }
-    const long k1_blocks = std::max((long)((op.g.V + 127) / 128), minres ? 0L : cgnr_blocks_per_rhs(op, N)) * N;
-    DLZ_TRY(fpart.alloc((size_t)2 * k1_blocks * sizeof(double)));   // K1 and K2a partials
+    const long k1_blocks = (minres ? minres_blocks_per_rhs(op, N) : cgnr_blocks_per_rhs(op, N)) * N;
+    DLZ_TRY(fpart.alloc((size_t)(2 * k1_blocks + 1) * sizeof(double)));   // partials of both kernels, a counter
     double *ist = scal.as<double>();
     double *d_rn = ist + state_doubles;                       // ||r_q||
     double *d_inv = d_rn + kMaxBatch, *d_tol = d_inv + kMaxBatch, *d_bn = d_tol + kMaxBatch;
-    HostScratch hs;
-    DLZ_TRY(hs.ensure(1024));
     double2 *pbp = bp.as<double2>(), *px = x.as<double2>(), *pr = r.as<double2>(), *pt = tmp.as<double2>();
     // b'_q = gamma5 b_q (MinRes on Q) or b_q (CG on the normal equations, residual of D) ; ||b_q||
     {
@@ -94,6 +92,7 @@ int dsolve_mixed_batch(Op &op, const dlz_defl_s *d, bool minres, const double2 *
         DLZ_CUDA_TRY(cudaMemcpyAsync(px, X_init, (size_t)N * n64 * sizeof(double2), cudaMemcpyDeviceToDevice, op.stream));
     else
         DLZ_CUDA_TRY(cudaMemsetAsync(px, 0, (size_t)N * n64 * sizeof(double2), op.stream));
+    GraphExec ge;                             // the inner solver's block of iterations
     std::vector<char> done(N, 0);
     std::vector<double> rn(N);
     int iters = 0, outer = 0;
@@ -219,9 +218,12 @@ int dsolve_mixed_batch(Op &op, const dlz_defl_s *d, bool minres, const double2 *
         }
         const int it0 = iters;
         if (minres) {
-            float4 *const bufs[6] = {w32[2], w32[3], w32[4], w32[5], w32[6], w32[7]};
-            DLZ_TRY(minres_fused_batch(op, N, w32[0], w32[1], bufs, reinterpret_cast<FusedState *>(ist),
-                                       fpart.as<double>(), d_tol, p, iters, hs, proj));
+            // the directions lie in the FP64 work vectors, idle during the inner solve
+            float4 *d1 = reinterpret_cast<float4 *>(pt);
+            const MinresVectors mv = {{w32[0], w32[2], w32[3], w32[4], w32[5], w32[6], w32[7]},
+                                      d1, d1 + (size_t)N * n32, w32[1]};
+            DLZ_TRY(minres_fused_batch(op, N, mv, reinterpret_cast<FusedState *>(ist), fpart.as<double>(), d_tol, p,
+                                       iters, ge, proj));
             mv_batch += iters - it0;
         } else {
             if (!proj) DLZ_CUDA_TRY(cudaMemsetAsync(w32[1], 0, (size_t)N * n32 * sizeof(float4), op.stream));
@@ -230,7 +232,7 @@ int dsolve_mixed_batch(Op &op, const dlz_defl_s *d, bool minres, const double2 *
             const CgBuffers bufs = {w32[3], w32[4],
                                     {w32[2], w32[5], w32[6], w32[7], w32[0], reinterpret_cast<float4 *>(pt)}};
             DLZ_TRY(cgnr_fused_batch(op, N, w32[0], w32[1], bufs, reinterpret_cast<CgFusedState *>(ist),
-                                     fpart.as<double>(), d_tol, p, iters));
+                                     fpart.as<double>(), d_tol, p, iters, ge));
             mv_batch += 2L * (iters - it0);
         }
         // x_q += ||r_q|| e_q
