@@ -43,6 +43,43 @@ int DevBuf::alloc(size_t nbytes) {
     bytes = nbytes;
     return DLZ_OK;
 }
+DevBuf *ScratchPool::take(size_t bytes, int &rc) {
+    {
+        std::lock_guard<std::mutex> lk(mu);
+        int best = -1;
+        for (int i = 0; i < (int)idle.size(); ++i)
+            if (idle[i]->bytes >= bytes && (best < 0 || idle[i]->bytes < idle[best]->bytes)) best = i;
+        if (best >= 0) {
+            DevBuf *b = idle[best];
+            idle.erase(idle.begin() + best);
+            rc = DLZ_OK;
+            return b;
+        }
+    }
+    DevBuf *b = new DevBuf();
+    rc = b->alloc(bytes);
+    if (rc != DLZ_OK) {
+        delete b;
+        return nullptr;
+    }
+    return b;
+}
+void ScratchPool::give(DevBuf *b) {
+    if (b->bytes <= kKeepBytes) {
+        std::lock_guard<std::mutex> lk(mu);
+        if ((int)idle.size() < kKeep) {
+            idle.push_back(b);
+            return;
+        }
+        // full: the smallest one goes
+        auto it = std::min_element(idle.begin(), idle.end(), [](DevBuf *x, DevBuf *y) { return x->bytes < y->bytes; });
+        if ((*it)->bytes < b->bytes) std::swap(*it, b);
+    }
+    delete b;
+}
+ScratchPool::~ScratchPool() {
+    for (DevBuf *b : idle) delete b;
+}
 void DevBuf::release() {
     if (p) cudaFree(p);
     p = nullptr;
@@ -511,38 +548,20 @@ int dlz_apply(dlz_op_t h, int which, const void *in, void *out, int dtype, int n
     Staged si, so;
     DLZ_TRY(si.in(op, in, bytes));
     DLZ_TRY(so.out(op, out, bytes));
-    DevBuf a, b, t;
-    DLZ_TRY(a.alloc(n * esz));
-    DLZ_TRY(b.alloc(n * esz));
-    DLZ_TRY(t.alloc(n * esz));
-    for (int r = 0; r < nrhs; ++r) {
-        if (dtype == DLZ_F64) {
-            const double2 *src = (const double2 *)si.dev + (size_t)r * n;
-            double2 *dst = (double2 *)so.dev + (size_t)r * n;
-            DLZ_TRY(pack64(op, a.as<double2>(), src));
-            DLZ_TRY(apply64(op, b.as<double2>(), a.as<double2>(), which, t.as<double2>()));
-            DLZ_TRY(unpack64(op, dst, b.as<double2>()));
-        } else if (dtype == DLZ_F32) {
-            const float2 *src = (const float2 *)si.dev + (size_t)r * n;
-            float2 *dst = (float2 *)so.dev + (size_t)r * n;
-            DLZ_TRY(pack32(op, a.as<float4>(), src));
-            DLZ_TRY(apply32(op, b.as<float4>(), a.as<float4>(), which, t.as<float4>()));
-            DLZ_TRY(unpack32(op, dst, b.as<float4>()));
-        } else {
-            // bfloat16 storage: D^dag D is Q applied twice, rounded to bfloat16 in between
-            const float2 *src = (const float2 *)si.dev + (size_t)r * n;
-            float2 *dst = (float2 *)so.dev + (size_t)r * n;
-            DLZ_TRY(pack_bf16(op, a.as<uint2>(), src));
-            if (which == DLZ_DDAGD) {
-                DLZ_TRY(wilson_bf16_batch(op, t.as<uint2>(), a.as<uint2>(), DLZ_Q, 1));
-                DLZ_TRY(wilson_bf16_batch(op, b.as<uint2>(), t.as<uint2>(), DLZ_Q, 1));
-            } else {
-                DLZ_TRY(wilson_bf16_batch(op, b.as<uint2>(), a.as<uint2>(), which, 1));
-            }
-            DLZ_TRY(unpack_bf16(op, dst, b.as<uint2>()));
-        }
+    const size_t per = apply_user_scratch(op, which, si.dev, so.dev, dtype, nrhs);
+    // as many right-hand sides at a time as the pool's buffers hold, at least one
+    size_t want = per * std::min<size_t>(nrhs, per ? std::max<size_t>(1, ScratchPool::kKeepBytes / per) : 1);
+    ScratchLease ws(op.pool, op.stream);
+    int rc = ws.take(want);
+    if (rc == DLZ_ERR_OOM && want > per) {          // a full device: one right-hand side at a time
+        want = per;
+        rc = ws.take(want);
     }
-    return so.flush(op);
+    DLZ_TRY(rc);
+    DLZ_TRY(apply_user(op, which, si.dev, so.dev, dtype, nrhs, ws.b ? ws.b->p : nullptr, want));
+    DLZ_TRY(so.flush(op));
+    ws.done = true;
+    return DLZ_OK;
 }
 
 int dlz_apply_noalloc(dlz_op_t h, int which, const void *in, void *out, int dtype, int nrhs) {
@@ -567,23 +586,7 @@ int dlz_apply_noalloc(dlz_op_t h, int which, const void *in, void *out, int dtyp
     void *scratch = nullptr;
     DLZ_TRY(noalloc_scratch(&scratch));
     op.prof.begin(false, false);
-    // packed input, packed output and (D^dag D only) the intermediate Q vector
-    unsigned char *sa = (unsigned char *)scratch, *sb = sa + vec, *st = sb + vec;
-    for (int r = 0; r < nrhs; ++r) {
-        if (dtype == DLZ_F64) {
-            const double2 *src = (const double2 *)in + (size_t)r * n;
-            double2 *dst = (double2 *)out + (size_t)r * n;
-            DLZ_TRY(pack64(op, (double2 *)sa, src));
-            DLZ_TRY(apply64(op, (double2 *)sb, (const double2 *)sa, which, (double2 *)st));
-            DLZ_TRY(unpack64(op, dst, (const double2 *)sb));
-        } else {
-            const float2 *src = (const float2 *)in + (size_t)r * n;
-            float2 *dst = (float2 *)out + (size_t)r * n;
-            DLZ_TRY(pack32(op, (float4 *)sa, src));
-            DLZ_TRY(apply32(op, (float4 *)sb, (const float4 *)sa, which, (float4 *)st));
-            DLZ_TRY(unpack32(op, dst, (const float4 *)sb));
-        }
-    }
+    DLZ_TRY(apply_user(op, which, in, out, dtype, nrhs, scratch, DLZ_NOALLOC_SCRATCH_BYTES));
     DLZ_CUDA_TRY(cudaStreamSynchronize(op.stream));
     return DLZ_OK;
 }

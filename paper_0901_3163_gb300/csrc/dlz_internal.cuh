@@ -16,6 +16,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -168,6 +169,42 @@ struct GrowBuf {
     void *ptr() const { return b.p; }
     template <typename T> T *as() const { return reinterpret_cast<T *>(b.p); }
 };
+// Device work memory that an operator keeps between calls: a call takes a buffer for its
+// own use and gives it back when its work is complete, so calls of several host threads
+// never share one.  At most kKeep buffers of at most kKeepBytes each are kept (a cudaMalloc
+// and cudaFree pair costs about as much as a whole application on a 8^4 lattice); larger
+// ones are freed at once, all of them with the operator.
+struct ScratchPool {
+    static constexpr int kKeep = 4;
+    static constexpr size_t kKeepBytes = (size_t)64 << 20;
+    std::mutex mu;
+    std::vector<DevBuf *> idle;
+    // the smallest idle buffer that is large enough, or a new one; null: out of memory
+    DevBuf *take(size_t bytes, int &rc);
+    void give(DevBuf *b);
+    ~ScratchPool();
+};
+// a pool buffer for one call; waits for the stream before giving it back unless the call
+// has already waited (done)
+struct ScratchLease {
+    ScratchPool &pool;
+    cudaStream_t stream;
+    DevBuf *b = nullptr;
+    bool done = false;
+    ScratchLease(ScratchPool &p, cudaStream_t s) : pool(p), stream(s) {}
+    ScratchLease(const ScratchLease &) = delete;
+    ScratchLease &operator=(const ScratchLease &) = delete;
+    int take(size_t bytes) {
+        int rc = DLZ_OK;
+        if (bytes) b = pool.take(bytes, rc);
+        return rc;
+    }
+    ~ScratchLease() {
+        if (!b) return;
+        if (!done) cudaStreamSynchronize(stream);
+        pool.give(b);
+    }
+};
 // scratch of the tensor-core basis products (tc_gemm.cu)
 struct TcScratch {
     GrowBuf coef, part, err;
@@ -205,6 +242,7 @@ struct Op {
     DevBuf md_scratch;   // block partials of the FP32 multi-dot (grown on demand, outside graphs)
     int multi_choice = 0;   // launch form the multi-lattice autotuner chose last (100 form + 10 chunks + half)
     TcScratch tc;           // scratch of the tensor-core basis products
+    ScratchPool pool;       // work memory of dlz_apply
     DevBuf stage_err;       // int: set by a stencil kernel whose staging wait gave up
 };
 
@@ -319,14 +357,18 @@ int apply64(Op &op, double2 *out, const double2 *in, int which, double2 *tmp);
 int apply32(Op &op, float4 *out, const float4 *in, int which, float4 *tmp);
 
 // pack / unpack between canonical complex [V][12] and internal planes
-int pack64(Op &op, double2 *dst, const double2 *src_canon);
-int unpack64(Op &op, double2 *dst_canon, const double2 *src);
-int pack32(Op &op, float4 *dst, const float2 *src_canon);
-int unpack32(Op &op, float2 *dst_canon, const float4 *src);
+// (nrhs vectors one after another)
+int pack64(Op &op, double2 *dst, const double2 *src_canon, int nrhs = 1);
+int unpack64(Op &op, double2 *dst_canon, const double2 *src, int nrhs = 1);
+int pack32(Op &op, float4 *dst, const float2 *src_canon, int nrhs = 1);
+int unpack32(Op &op, float2 *dst_canon, const float4 *src, int nrhs = 1);
 // bfloat16 spinors (uint2 planes [6][V]) with FP32 arithmetic (wilson_bf16.cu)
 int wilson_bf16_batch(Op &op, uint2 *out, const uint2 *in, int which, int nrhs);
-int pack_bf16(Op &op, uint2 *dst, const float2 *src_canon);
-int unpack_bf16(Op &op, float2 *dst_canon, const uint2 *src);
+int pack_bf16(Op &op, uint2 *dst, const float2 *src_canon, int nrhs = 1);
+int unpack_bf16(Op &op, float2 *dst_canon, const uint2 *src, int nrhs = 1);
+// out = A in on nrhs user vectors (device); scratch: apply_user_scratch() bytes or more
+size_t apply_user_scratch(const Op &op, int which, const void *in, const void *out, int dtype, int nrhs);
+int apply_user(Op &op, int which, const void *in, void *out, int dtype, int nrhs, void *scratch, size_t bytes);
 int convert64to32(Op &op, float4 *dst, const double2 *src);
 int convert32to64(Op &op, double2 *dst, const float4 *src);
 

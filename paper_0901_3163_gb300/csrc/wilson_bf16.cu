@@ -94,24 +94,26 @@ k_wilson_bf16_batch(uint2 *__restrict__ out, const uint2 *__restrict__ in, const
 __global__ void k_pack_bf16(uint2 *__restrict__ dst, const float2 *__restrict__ src, int V) {
     const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;   // s*6 + c
     if (i >= 6L * V) return;
+    const size_t base = (size_t)blockIdx.y * 6 * V;       // blockIdx.y: the right-hand side
     const int s = (int)(i / 6), c = (int)(i % 6);
-    const float2 a = src[(size_t)s * 12 + 2 * c], b = src[(size_t)s * 12 + 2 * c + 1];
+    const float2 a = src[2 * base + (size_t)s * 12 + 2 * c], b = src[2 * base + (size_t)s * 12 + 2 * c + 1];
     const __nv_bfloat162 x = __floats2bfloat162_rn(a.x, a.y), y = __floats2bfloat162_rn(b.x, b.y);
     uint2 q;
     memcpy(&q.x, &x, 4);
     memcpy(&q.y, &y, 4);
-    dst[(size_t)c * V + s] = q;
+    dst[base + (size_t)c * V + s] = q;
 }
 __global__ void k_unpack_bf16(float2 *__restrict__ dst, const uint2 *__restrict__ src, int V) {
     const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= 6L * V) return;
+    const size_t base = (size_t)blockIdx.y * 6 * V;
     const int s = (int)(i / 6), c = (int)(i % 6);
-    const uint2 q = src[(size_t)c * V + s];
+    const uint2 q = src[base + (size_t)c * V + s];
     __nv_bfloat162 x, y;
     memcpy(&x, &q.x, 4);
     memcpy(&y, &q.y, 4);
-    dst[(size_t)s * 12 + 2 * c] = __bfloat1622float2(x);
-    dst[(size_t)s * 12 + 2 * c + 1] = __bfloat1622float2(y);
+    dst[2 * base + (size_t)s * 12 + 2 * c] = __bfloat1622float2(x);
+    dst[2 * base + (size_t)s * 12 + 2 * c + 1] = __bfloat1622float2(y);
 }
 
 }  // namespace
@@ -133,16 +135,16 @@ int wilson_bf16_batch(Op &op, uint2 *out, const uint2 *in, int which, int nrhs) 
     return DLZ_OK;
 }
 
-int pack_bf16(Op &op, uint2 *dst, const float2 *src) {
+int pack_bf16(Op &op, uint2 *dst, const float2 *src, int nrhs) {
     const long n = 6L * op.g.V;
-    k_pack_bf16<<<(unsigned)((n + 255) / 256), 256, 0, op.stream>>>(dst, src, op.g.V);
+    k_pack_bf16<<<dim3((unsigned)((n + 255) / 256), nrhs), 256, 0, op.stream>>>(dst, src, op.g.V);
     DLZ_CUDA_TRY(cudaGetLastError());
     return DLZ_OK;
 }
 
-int unpack_bf16(Op &op, float2 *dst, const uint2 *src) {
+int unpack_bf16(Op &op, float2 *dst, const uint2 *src, int nrhs) {
     const long n = 6L * op.g.V;
-    k_unpack_bf16<<<(unsigned)((n + 255) / 256), 256, 0, op.stream>>>(dst, src, op.g.V);
+    k_unpack_bf16<<<dim3((unsigned)((n + 255) / 256), nrhs), 256, 0, op.stream>>>(dst, src, op.g.V);
     DLZ_CUDA_TRY(cudaGetLastError());
     return DLZ_OK;
 }

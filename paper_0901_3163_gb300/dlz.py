@@ -164,6 +164,11 @@ def _ptr(a):
     return a.data_ptr()
 
 
+def _count(a):
+    """Number of elements of a torch tensor or numpy array."""
+    return a.size if isinstance(a, np.ndarray) else a.numel()
+
+
 def _empty_like(a, dtype=None):
     if isinstance(a, np.ndarray):
         return np.empty(a.shape, dtype=dtype or a.dtype)
@@ -205,12 +210,15 @@ class Operator:
         self.dims = tuple(dims)
         self.kappa = kappa
         self.bc_t = bc_t
+        self._volume = None
 
     @property
     def volume(self):
-        v = ctypes.c_longlong()
-        _check(lib.dlz_op_volume(self.handle, ctypes.byref(v)))
-        return v.value
+        if self._volume is None:
+            v = ctypes.c_longlong()
+            _check(lib.dlz_op_volume(self.handle, ctypes.byref(v)))
+            self._volume = v.value
+        return self._volume
 
     def __del__(self):
         if getattr(self, "handle", None):
@@ -274,8 +282,7 @@ def apply(op, which, x, out=None, dtype=None):
         dtype = F32 if str(x.dtype).endswith("complex64") else F64
     if out is None:
         out = _empty_like(x)
-    V = op.volume
-    nrhs = int(np.prod(x.shape)) // (12 * V) if np.prod(x.shape) else 0
+    nrhs = _count(x) // (12 * op.volume)
     _check(lib.dlz_apply(op.handle, int(which), _ptr(x), _ptr(out), int(dtype), nrhs))
     return out
 
