@@ -548,7 +548,7 @@ int dlz_apply(dlz_op_t h, int which, const void *in, void *out, int dtype, int n
     Staged si, so;
     DLZ_TRY(si.in(op, in, bytes));
     DLZ_TRY(so.out(op, out, bytes));
-    const size_t per = apply_user_scratch(op, which, si.dev, so.dev, dtype, nrhs);
+    const size_t per = apply_user_scratch(op, which, si.dev, so.dev, dtype);
     // as many right-hand sides at a time as the pool's buffers hold, at least one
     size_t want = per * std::min<size_t>(nrhs, per ? std::max<size_t>(1, ScratchPool::kKeepBytes / per) : 1);
     ScratchLease ws(op.pool, op.stream);

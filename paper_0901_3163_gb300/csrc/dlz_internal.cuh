@@ -207,7 +207,7 @@ struct ScratchLease {
 };
 // scratch of the tensor-core basis products (tc_gemm.cu)
 struct TcScratch {
-    GrowBuf coef, part, err;
+    GrowBuf buf;
 };
 // Tensor-core (tcgen05, 3xTF32) products of FP32 basis vectors on stream st:
 //   tc_combine32: out[j] (len floats, stride ldo) = sum_i c_ij in[i] (stride ldv), i < nin,
@@ -367,7 +367,7 @@ int wilson_bf16_batch(Op &op, uint2 *out, const uint2 *in, int which, int nrhs);
 int pack_bf16(Op &op, uint2 *dst, const float2 *src_canon, int nrhs = 1);
 int unpack_bf16(Op &op, float2 *dst_canon, const uint2 *src, int nrhs = 1);
 // out = A in on nrhs user vectors (device); scratch: apply_user_scratch() bytes or more
-size_t apply_user_scratch(const Op &op, int which, const void *in, const void *out, int dtype, int nrhs);
+size_t apply_user_scratch(const Op &op, int which, const void *in, const void *out, int dtype);
 int apply_user(Op &op, int which, const void *in, void *out, int dtype, int nrhs, void *scratch, size_t bytes);
 int convert64to32(Op &op, float4 *dst, const double2 *src);
 int convert32to64(Op &op, double2 *dst, const float4 *src);

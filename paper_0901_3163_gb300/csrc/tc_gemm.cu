@@ -31,20 +31,31 @@ namespace dlz {
 
 namespace {
 
-constexpr int kTcThreads = 256;     // 8 warps: staging, epilogue (two per TMEM lane quarter)
+// Warps of a block: the first kEpiWarps read the accumulators (warp w: TMEM lane quarter w % 4)
+// and store the results, the next one issues the MMAs, four copy raw FP32 chunks into a ring of
+// shared-memory slots, and S groups of four warps split them into the operand stages, group g the chunks
+// g, g + S, ... into stage g.  They meet only at mbarriers, so copies, splits, MMAs and stores
+// of different chunks overlap.  The restart of 121 vectors of 16^3 x 32 to 61, and the dots
+// of 121 with 16 vectors (ncu, one GB300): 1.81 and 0.93 ms with one role for all threads, two
+// block barriers per chunk and one chunk loaded ahead; 0.66 and 0.71 ms with roles but the
+// splitting warps copying their own chunks; 0.62 and 0.64 ms in this form (3.7 and 2.7 TB/s).
+// No single stage bounds it now: without its copies the combine takes 0.61 ms, with a twelfth
+// of its MMAs 0.53 ms, without its split stores 0.66 ms.
+constexpr int kEpiWarps = 8;
+constexpr int kFill = 128;                                   // threads of a group, and of the copying warps
+constexpr int tc_threads(int groups) { return 32 * (kEpiWarps + 1) + (groups + 1) * kFill; }
 constexpr int kKC = 32;             // K chunk staged per pipeline stage
-constexpr long long kWaitPolls = 1LL << 26;
-constexpr int kTcMaxSmem = 2 * (2 * 128 * kKC * 4 + 2 * 256 * kKC * 4);   // 192 KB
+constexpr int kWaitPolls = 1 << 22;     // (each poll may suspend the thread for a while)
+constexpr int kTcMaxSmem = 226 * 1024;      // dynamic shared memory a block may ask for
+constexpr int kABytes = 128 * kKC * 4;      // one part (hi or lo) of an A chunk
 
 __device__ __forceinline__ uint32_t su32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-__device__ __forceinline__ uint64_t sdesc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
-    uint64_t d = (uint64_t)((saddr >> 4) & 0x3FFF);
-    d |= (uint64_t)((lbo >> 4) & 0x3FFF) << 16;
-    d |= (uint64_t)((sbo >> 4) & 0x3FFF) << 32;
-    d |= (uint64_t)1 << 46;          // descriptor version of the sm_100 family; no swizzle
-    return d;
-}
+// Operand descriptor at shared address `saddr`: 14 address bits (16-byte units) and the
+// leading byte offset in the low word, stride byte offset and the descriptor version of the
+// sm_100 family (no swizzle) in the high word.  Only the low word changes along K.
+__device__ __forceinline__ uint32_t sdesc_lo(uint32_t saddr) { return ((saddr >> 4) & 0x3FFF) | (128u >> 4) << 16; }
+constexpr uint32_t kDescHi = (1024u >> 4) | 1u << 14;
 
 // instruction descriptor: D FP32 (bits 4-5), A and B TF32 (7-9, 10-12), both K-major
 // (bits 15, 16 zero), N / 8 (17-22), M / 16 (24-28) with M = 128
@@ -52,41 +63,71 @@ __device__ __forceinline__ uint32_t idesc_tf32(int n, uint32_t a_mn) {
     return (1u << 4) | (2u << 7) | (2u << 10) | (a_mn << 15) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
 }
 
-__device__ __forceinline__ void mma_tf32(uint32_t taddr, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc) {
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                 "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(taddr),
-                 "l"(da), "l"(db), "r"(idesc), "r"(acc));
+template <bool ACC>
+__device__ __forceinline__ void mma_tf32(uint32_t taddr, uint32_t da, uint32_t db, uint32_t idesc, bool acc = true) {
+    asm volatile("{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\tmov.b64 a, {%1, %5};\n\tmov.b64 b, {%2, %5};\n\t"
+                 "setp.ne.b32 p, %4, 0;\n\t"
+                 "tcgen05.mma.cta_group::1.kind::tf32 [%0], a, b, %3, p;\n\t}\n" ::"r"(taddr),
+                 "r"(da), "r"(db), "r"(idesc), "r"(ACC ? 1u : (acc ? 1u : 0u)), "r"(kDescHi));
 }
 
 __device__ __forceinline__ void commit_to(uint64_t *mbar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(su32(mbar)));
 }
 
-// bounded wait for the completion of phase `parity` of an mbarrier
-__device__ __forceinline__ bool mbar_wait(uint64_t *mbar, uint32_t parity) {
+// Bounded wait for the completion of phase `parity` of an mbarrier.  A wait that gives up
+// sets the block's fail word, which ends the other waits as well.
+__device__ __forceinline__ bool mbar_wait(uint64_t *mbar, uint32_t parity, volatile int *failed) {
     uint32_t done = 0;
-    for (long long it = 0; it < kWaitPolls && !done; ++it) {
+    for (int it = 0; it < kWaitPolls && !done; ++it) {
         asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
                      "selp.u32 %0, 1, 0, p;\n\t}\n"
-                     : "=r"(done) : "r"(su32(mbar)), "r"(parity));
+                     : "=r"(done) : "r"(su32(mbar)), "r"(parity) : "memory");
+        if (!done && *failed) return false;
     }
+    if (!done) *failed = 1;
     return done != 0;
 }
-
-__device__ __forceinline__ float tf32_hi(float x) {
-    uint32_t r;
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-    return __uint_as_float(r);
+__device__ __forceinline__ void mbar_arrive(uint64_t *mbar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(su32(mbar)) : "memory");
+}
+__device__ __forceinline__ void mbar_init(uint64_t *mbar, uint32_t count) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(mbar)), "r"(count));
 }
 
-__device__ __forceinline__ void tmem_ld8(uint32_t addr, float (&v)[8]) {
-    uint32_t r[8];
+// Asynchronous 16-byte copy of the raw ring; valid = false fills the slot with zeros.
+__device__ __forceinline__ void ring_load(float4 *slot, const float *src, bool valid) {
+    asm volatile("cp.async.cg.shared.global.L2::256B [%0], [%1], 16, %2;" ::"r"(su32(slot)), "l"(src), "r"(valid ? 16 : 0)
+                 : "memory");
+}
+// arrive on mbar once this thread's copies so far have landed
+__device__ __forceinline__ void ring_arrive(uint64_t *mbar) {
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(su32(mbar)) : "memory");
+}
+
+// x rounded to TF32 (10 mantissa bits, nearest, ties away from zero) by two integer operations
+__device__ __forceinline__ float tf32_hi(float x) {
+    return __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xffffe000u);
+}
+
+__device__ __forceinline__ void tmem_wait(uint32_t (&r)[16]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                   "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]));
+}
+// columns addr .. addr + 15, or the first 8 of them
+__device__ __forceinline__ void tmem_read(uint32_t addr, bool wide, float (&v)[16]) {
+    uint32_t r[16] = {};
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
                  : "r"(addr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;");
+    if (wide)
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                     : "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+                     : "r"(addr + 8));
+    tmem_wait(r);
 #pragma unroll
-    for (int j = 0; j < 8; ++j) v[j] = __uint_as_float(r[j]);
+    for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
 }
 
 __device__ __forceinline__ void st_split(float *hi, float *lo, int off_floats, float4 v) {
@@ -112,34 +153,46 @@ struct CombineArgs {
     int *err;
 };
 
-// A pipeline stage is reused only after the MMAs that last read it are complete: every
-// commit to a stage's mbarrier completes one phase, and `issued` / `seen` count, per stage,
-// the commits made and the completions waited for (all threads keep the same counts).
-struct StageSync {
-    uint32_t issued[2] = {0u, 0u}, seen[2] = {0u, 0u};
-    // wait until stage st has no MMA in flight; false if a wait gave up
-    __device__ bool drain(uint64_t *mbar, int st) {
-        while (seen[st] < issued[st]) {
-            if (!mbar_wait(&mbar[st], seen[st] & 1u)) return false;
-            ++seen[st];
-        }
-        return true;
-    }
+// The block's synchronisation.  Ring slot r of R: raw_full[r] completes when every copying
+// thread's part has landed, raw_empty[r] when the group that took it has read it.  Operand
+// stage s of S: full[s] when every warp of its group has written it, empty[s] when the MMAs
+// that read it are done.  Accumulator a of two: acc_full[a] when a tile's MMAs are done,
+// acc_empty[a] when it has been read.  A wait on a phase's parity is only right while the
+// waiter is at most one phase behind: each stage has a group of its own, and R is a multiple
+// of S, so that one group takes all chunks of a slot.
+template <int S, int R> struct TcShared {
+    static_assert(R % S == 0, "ring slots per group");
+    uint64_t raw_full[R], raw_empty[R], full[S], empty[S], acc_full[2], acc_empty[2];
+    uint32_t tbase;
+    int failed;
 };
 
-__device__ __forceinline__ void tc_setup(uint64_t *mbar, uint32_t *tbase, int ncols) {
+// barriers, and `ncols` columns of tensor memory (warp 0); returns their address
+template <int S, int R> __device__ __forceinline__ uint32_t tc_setup(TcShared<S, R> &sh, int ncols) {
     if (threadIdx.x == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(su32(&mbar[0])));
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(su32(&mbar[1])));
+        sh.failed = 0;
+        for (int i = 0; i < R; ++i) {
+            mbar_init(&sh.raw_full[i], kFill);
+            mbar_init(&sh.raw_empty[i], kFill / 32);
+        }
+        for (int i = 0; i < S; ++i) {
+            mbar_init(&sh.full[i], kFill / 32);
+            mbar_init(&sh.empty[i], 1);
+        }
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(&sh.acc_full[i], 1);
+            mbar_init(&sh.acc_empty[i], kEpiWarps);
+        }
         asm volatile("fence.mbarrier_init.release.cluster;");
     }
     if ((threadIdx.x >> 5) == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tbase)), "r"(ncols));
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(&sh.tbase)), "r"(ncols));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
+    return sh.tbase;
 }
 
 __device__ __forceinline__ void tc_teardown(uint32_t taddr, int ncols) {
@@ -149,67 +202,101 @@ __device__ __forceinline__ void tc_teardown(uint32_t taddr, int ncols) {
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols));
 }
 
-__device__ __forceinline__ int tmem_cols(int n) { return n <= 32 ? 32 : n <= 64 ? 64 : n <= 128 ? 128 : 256; }
-
-// The combine's A operand for one thread: vectors 4 kq .. 4 kq + 3 of K chunk kc at rows
-// r .. r + 3 (zero beyond the data; for complex coefficients the second half of K holds
-// i times the vectors)
-__device__ __forceinline__ void combine_load_a(const CombineArgs &a, int kc, int kq, long r, float4 (&v)[4]) {
+// One chunk's MMAs into the accumulator at `acc`: hi hi + hi lo + lo hi over 32 k, from the
+// low words of the operands' descriptors.  (The issuing warp is kept uniform, one lane issuing:
+// a lone thread that built every descriptor took longer than the MMAs.)
+__device__ __forceinline__ void chunk_mmas(uint32_t acc, uint32_t ah, uint32_t al, uint32_t bh, uint32_t bl,
+                                           uint32_t idesc, bool first) {
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const int k = kc * kKC + 4 * kq + j;
-        v[j] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (r < a.rows) {
-            if (k < a.nin) {
-                v[j] = *reinterpret_cast<const float4 *>(a.V + (size_t)k * a.ldv + r);
-            } else if (a.cplx && k < 2 * a.nin) {
-                const float4 u = *reinterpret_cast<const float4 *>(a.V + (size_t)(k - a.nin) * a.ldv + r);
-                v[j] = make_float4(-u.y, u.x, -u.w, u.z);        // i times the complex pairs
-            }
-        }
+    for (int ks = 0; ks < kKC / 8; ++ks) {
+        const uint32_t k = ks * (256 >> 4);
+        if (ks == 0) mma_tf32<false>(acc, ah, bh, idesc, !first);
+        else mma_tf32<true>(acc, ah + k, bh + k, idesc);
+        mma_tf32<true>(acc, ah + k, bl + k, idesc);
+        mma_tf32<true>(acc, al + k, bh + k, idesc);
     }
 }
 
-__global__ void __launch_bounds__(kTcThreads, 1) k_tc_combine(CombineArgs a) {
+__device__ __forceinline__ int tmem_cols(int n) { return n <= 32 ? 32 : n <= 64 ? 64 : n <= 128 ? 128 : n <= 256 ? 256 : 512; }
+
+// The combine's A operand, item (row quad, k quad kq) of a chunk: vectors 4 kq .. 4 kq + 3 of
+// K chunk kc at rows r .. r + 3 (zero beyond the data; for complex coefficients the second
+// half of K holds i times the vectors, made by combine_take_a)
+__device__ __forceinline__ void combine_load_a(const CombineArgs &a, int kc, int kq, long r, float4 *slot) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const int k = kc * kKC + 4 * kq + j;
+        const int v = k < a.nin ? k : k - a.nin;
+        const bool ok = r < a.rows && (k < a.nin || (a.cplx && k < 2 * a.nin));
+        ring_load(slot + j * kFill, ok ? a.V + (size_t)v * a.ldv + r : a.V, ok);
+    }
+}
+__device__ __forceinline__ void combine_take_a(const CombineArgs &a, int kc, int kq, const float4 *slot, float4 (&v)[4]) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const float4 u = slot[j * kFill];
+        v[j] = kc * kKC + 4 * kq + j < a.nin ? u : make_float4(-u.y, u.x, -u.w, u.z);   // i times the complex pairs
+    }
+}
+
+// Bound by memory: (nin + nout) vectors move.  Shared memory is next: a chunk's 16 KB pass
+// it as raw copy, read, two split parts and three MMA operand reads, about 1000 cycles of
+// the SM against 740 of its share of the memory bandwidth for the reads alone.  RES: both
+// parts of the coefficient matrix stay in shared memory for the whole kernel (when they fit
+// beside two stages); otherwise every chunk's part is copied from L2.
+template <int S, int R, bool RES>
+__global__ void __launch_bounds__(tc_threads(S), 1) k_tc_combine(CombineArgs a) {
     extern __shared__ __align__(1024) unsigned char smem[];
-    const int a_bytes = 128 * kKC * 4, b_bytes = a.npad * kKC * 4;
-    const int stage_bytes = 2 * a_bytes + 2 * b_bytes;
-    __shared__ __align__(8) uint64_t mbar[2];
-    __shared__ uint32_t tbase;
-    __shared__ int fail_s;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int ncols = tmem_cols(a.npad);
-    if (tid == 0) fail_s = 0;
-    tc_setup(mbar, &tbase, ncols);
-    const uint32_t taddr = tbase;
-    const long ntiles = (a.rows + 127) / 128;
+    __shared__ __align__(8) TcShared<S, R> sh;
+    const int b_bytes = a.npad * kKC * 4;
+    const int stage_bytes = 2 * kABytes + (RES ? 0 : 2 * b_bytes);
     const int nkc = a.kpad / kKC;
-    const uint32_t idesc = idesc_tf32(a.npad, 0u);
-    StageSync ss;
-    // A chunk: 128 rows x 32 k, K-major.  Thread (row quad rq, k quad kq) loads the four
-    // vectors 4 kq .. 4 kq + 3 at rows 4 rq .. 4 rq + 3 (float4 each, 64 contiguous bytes
-    // per vector across the 4 lanes of equal kq), transposes the 4 x 4 block and stores
-    // one 16-byte k quad per row; lane l stores its rows in the order (c + l % 4) so that
-    // the eight lanes of a store instruction with equal row parity hit different banks.
-    // The loads of the next chunk (or of the next tile's first chunk) are issued right
-    // after the current chunk's MMAs, so they are in flight during the MMAs, the next
-    // stage's wait and the epilogue.
-    const int kq = tid & 7, rq = tid >> 3;                                    // 8 k quads x 32 row quads
-    float4 v[4];
-    if ((long)blockIdx.x < ntiles) combine_load_a(a, 0, kq, (long)blockIdx.x * 128 + 4 * rq, v);
-    for (long t = blockIdx.x; t < ntiles; t += gridDim.x) {
-        const long r0 = t * 128;
-        for (int kc = 0; kc < nkc; ++kc) {
-            const int st = kc & 1;
-            unsigned char *sbase = smem + st * stage_bytes;
-            float *Ahi = reinterpret_cast<float *>(sbase), *Alo = reinterpret_cast<float *>(sbase + a_bytes);
-            float *Bhi = reinterpret_cast<float *>(sbase + 2 * a_bytes);
-            float *Blo = reinterpret_cast<float *>(sbase + 2 * a_bytes + b_bytes);
-            if (!ss.drain(mbar, st) && tid == 0) fail_s = 1;
-            __syncthreads();
-            if (fail_s) break;
-            {
-                const int rot = tid & 3;
+    float4 *ring = reinterpret_cast<float4 *>(smem + S * stage_bytes);             // [R][2 x 4][kFill]
+    unsigned char *bres = smem + S * stage_bytes + R * kABytes;                    // RES: [nkc][hi, lo]
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+    const int ncols = tmem_cols(2 * a.npad);
+    const long ntiles = (a.rows + 127) / 128;
+    // B chunk kc: npad rows (outputs) x 32 k, K-major, from the pre-split global copies
+    auto load_b = [&](int kc, unsigned char *dst, int t0, int nt) {
+        float *Bhi = reinterpret_cast<float *>(dst), *Blo = reinterpret_cast<float *>(dst + b_bytes);
+        for (int w = t0; w < a.npad * (kKC / 4); w += nt) {
+            const int j = w % a.npad, q = w / a.npad;                        // k = 4 q .. 4 q + 3
+            const size_t gi = (size_t)j * a.kpad + kc * kKC + 4 * q;
+            const int off = (j / 8) * 256 + q * 32 + (j % 8) * 4;
+            *reinterpret_cast<float4 *>(Bhi + off) = *reinterpret_cast<const float4 *>(a.Bhi + gi);
+            *reinterpret_cast<float4 *>(Blo + off) = *reinterpret_cast<const float4 *>(a.Blo + gi);
+        }
+    };
+    if (RES) {
+        for (int kc = 0; kc < nkc; ++kc) load_b(kc, bres + (size_t)kc * 2 * b_bytes, threadIdx.x, blockDim.x);
+        asm volatile("fence.proxy.async.shared::cta;");
+    }
+    const uint32_t taddr = tc_setup(sh, ncols);
+    volatile int *failed = &sh.failed;
+    // A chunk: 128 rows x 32 k.  Item (row quad rq, k quad kq): the four vectors 4 kq .. 4 kq
+    // + 3 at rows 4 rq .. 4 rq + 3 (float4 each, 128 contiguous bytes per vector across the 8
+    // lanes of equal kq); a thread takes the row quads rq and rq + 16.
+    const int ft = threadIdx.x - 32 * (kEpiWarps + 1), tid = ft % kFill;
+    const int rq = (tid & 7) + 8 * (tid >> 6), kq = (tid >> 3) & 7;
+    float4 *slots = ring + tid;
+    const long mine = ((ntiles - blockIdx.x + gridDim.x - 1) / gridDim.x) * nkc;   // the block's chunks
+    if (ft >= kFill) {
+        // ---- split.  An item is a 4 x 4 block, transposed and stored K-major as one 16-byte
+        // k quad per row; a lane stores its rows in the order (c + rot) so that the eight
+        // lanes of a store phase (rq = 0 .. 7) hit eight different 16-byte banks.
+        const int grp = ft / kFill - 1, rot = (tid >> 1) & 3;
+        unsigned char *sbase = smem + grp * stage_bytes;
+        float *Ahi = reinterpret_cast<float *>(sbase), *Alo = reinterpret_cast<float *>(sbase + kABytes);
+        int kc = grp % nkc, slot = grp;
+        uint32_t round = 0, rround = 0;        // uses of the stage and of the slot before this one
+        for (long q = grp; q < mine; q += S, ++round) {
+            const float4 *raw = slots + (size_t)slot * 8 * kFill;
+            if (!__all_sync(0xffffffffu, mbar_wait(&sh.raw_full[slot], rround & 1u, failed))) break;
+            if (round > 0 && !__all_sync(0xffffffffu, mbar_wait(&sh.empty[grp], (round - 1) & 1u, failed))) break;
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+                float4 v[4];
+                combine_take_a(a, kc, kq, raw + half * 4 * kFill, v);
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
                     const int cc = (c + rot) & 3;                             // the row this lane stores now
@@ -218,62 +305,88 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_combine(CombineArgs a) {
                     w4.y = cc == 0 ? v[1].x : cc == 1 ? v[1].y : cc == 2 ? v[1].z : v[1].w;
                     w4.z = cc == 0 ? v[2].x : cc == 1 ? v[2].y : cc == 2 ? v[2].z : v[2].w;
                     w4.w = cc == 0 ? v[3].x : cc == 1 ? v[3].y : cc == 2 ? v[3].z : v[3].w;
-                    const int row = 4 * rq + cc;
+                    const int row = 4 * rq + 64 * half + cc;
                     st_split(Ahi, Alo, (row >> 3) * 256 + kq * 32 + (row & 7) * 4, w4);
                 }
             }
-            // B chunk: npad rows (outputs) x 32 k, K-major, from the pre-split global copies
-            for (int w = tid; w < a.npad * (kKC / 4); w += kTcThreads) {
-                const int j = w % a.npad, kq = w / a.npad;                   // k = 4 kq .. 4 kq + 3
-                const size_t gi = (size_t)j * a.kpad + kc * kKC + 4 * kq;
-                const int off = (j / 8) * 256 + kq * 32 + (j % 8) * 4;
-                *reinterpret_cast<float4 *>(Bhi + off) = *reinterpret_cast<const float4 *>(a.Bhi + gi);
-                *reinterpret_cast<float4 *>(Blo + off) = *reinterpret_cast<const float4 *>(a.Blo + gi);
-            }
+            if (!RES) load_b(kc, sbase + 2 * kABytes, tid, kFill);
             asm volatile("fence.proxy.async.shared::cta;");
-            __syncthreads();
-            if (tid == 0) {
+            __syncwarp();
+            if (lane == 0) {
+                mbar_arrive(&sh.raw_empty[slot]);
+                mbar_arrive(&sh.full[grp]);
+            }
+            for (kc += S; kc >= nkc;) kc -= nkc;
+            if ((slot += S) >= R) { slot = grp; ++rround; }
+        }
+    } else if (ft >= 0) {
+        // ---- copy
+        long t = blockIdx.x;
+        int kc = 0, slot = 0;
+        uint32_t round = 0;
+        for (long q = 0; q < mine; ++q) {
+            if (round > 0 && !mbar_wait(&sh.raw_empty[slot], (round - 1) & 1u, failed)) break;
+            float4 *raw = slots + (size_t)slot * 8 * kFill;
+            combine_load_a(a, kc, kq, t * 128 + 4 * rq, raw);
+            combine_load_a(a, kc, kq, t * 128 + 4 * rq + 64, raw + 4 * kFill);
+            ring_arrive(&sh.raw_full[slot]);
+            if (++kc == nkc) { kc = 0; t += gridDim.x; }
+            if (++slot == R) { slot = 0; ++round; }
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");       // no copy may land after the block has ended
+    } else if (warp == kEpiWarps) {
+        // ---- MMA (the warp is uniform; lane 0 issues)
+        const uint32_t idesc = idesc_tf32(a.npad, 0u);
+        const uint32_t d_stage = sdesc_lo(su32(smem)), d_res = RES ? sdesc_lo(su32(bres)) : 0u;
+        const uint32_t w_stage = stage_bytes >> 4, w_b = b_bytes >> 4;
+        int st = 0, n = 0;
+        uint32_t round = 0;
+        bool ok = true;
+        for (long t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++n) {
+            const int acc = n & 1;
+            if (n >= 2 && !__all_sync(0xffffffffu, mbar_wait(&sh.acc_empty[acc], ((n >> 1) - 1) & 1, failed))) break;
+            for (int kc = 0; kc < nkc; ++kc) {
+                ok = __all_sync(0xffffffffu, mbar_wait(&sh.full[st], round & 1u, failed));
+                if (!ok) break;
                 asm volatile("tcgen05.fence::after_thread_sync;");
-#pragma unroll
-                for (int ks = 0; ks < kKC / 8; ++ks) {
-                    const uint64_t ah = sdesc(su32(Ahi) + ks * 256, 128, 1024);
-                    const uint64_t al = sdesc(su32(Alo) + ks * 256, 128, 1024);
-                    const uint64_t bh = sdesc(su32(Bhi) + ks * 256, 128, 1024);
-                    const uint64_t bl = sdesc(su32(Blo) + ks * 256, 128, 1024);
-                    mma_tf32(taddr, ah, bh, idesc, (kc > 0 || ks > 0) ? 1u : 0u);
-                    mma_tf32(taddr, ah, bl, idesc, 1u);
-                    mma_tf32(taddr, al, bh, idesc, 1u);
+                const uint32_t da = d_stage + st * w_stage;
+                const uint32_t db = RES ? d_res + 2 * kc * w_b : da + (2 * kABytes >> 4);
+                if (lane == 0) {
+                    chunk_mmas(taddr + acc * a.npad, da, da + (kABytes >> 4), db, db + w_b, idesc, kc == 0);
+                    commit_to(&sh.empty[st]);
                 }
-                commit_to(&mbar[st]);
+                if (++st == S) { st = 0; ++round; }
             }
-            ++ss.issued[st];
-            if (kc + 1 < nkc) combine_load_a(a, kc + 1, kq, r0 + 4 * rq, v);
-            else if (t + gridDim.x < ntiles) combine_load_a(a, 0, kq, (t + gridDim.x) * 128 + 4 * rq, v);
+            if (ok && lane == 0) commit_to(&sh.acc_full[acc]);
         }
-        // epilogue: every MMA of the tile complete, then each warp reads its lane quarter
-        // and half of the columns
-        bool okd = ss.drain(mbar, 0);
-        okd = ss.drain(mbar, 1) && okd;
-        if (!okd && tid == 0) fail_s = 1;
-        __syncthreads();
-        if (fail_s) break;
-        asm volatile("tcgen05.fence::after_thread_sync;");
-        const int lq = warp & 3, half = warp >> 2;
-        const int c_lo = half * (a.npad / 2), c_hi = c_lo + a.npad / 2;
-        const long r = r0 + 32 * lq + lane;
-        for (int c0 = c_lo; c0 < c_hi; c0 += 8) {
-            float v[8];
-            tmem_ld8(taddr + ((uint32_t)(32 * lq) << 16) + (uint32_t)c0, v);
-            if (r < a.rows) {
+        __syncwarp();
+    } else {
+        // ---- results: warp w reads rows 32 (w % 4) .. of each tile, half of the columns (with
+        // four warps and 8 columns per read the stores, not the loads, set the pace)
+        int n = 0;
+        const int lq = warp & 3, c_lo = (warp >> 2) * (a.npad / 2), c_hi = min(c_lo + a.npad / 2, a.nout);
+        for (long t = blockIdx.x; t < ntiles; t += gridDim.x, ++n) {
+            const int acc = n & 1;
+            if (!__all_sync(0xffffffffu, mbar_wait(&sh.acc_full[acc], (n >> 1) & 1, failed))) break;
+            asm volatile("tcgen05.fence::after_thread_sync;");
+            const long r = t * 128 + 32 * lq + lane;
+            for (int c0 = c_lo; c0 < c_hi; c0 += 16) {
+                float v[16];
+                tmem_read(taddr + ((uint32_t)(32 * lq) << 16) + (uint32_t)(acc * a.npad + c0), c0 + 8 < c_lo + a.npad / 2, v);
+                float *o = a.Out + (size_t)c0 * a.ldo + r;
+                if (r < a.rows) {
 #pragma unroll
-                for (int j = 0; j < 8; ++j)
-                    if (c0 + j < a.nout) a.Out[(size_t)(c0 + j) * a.ldo + r] = v[j];
+                    for (int j = 0; j < 16; ++j, o += a.ldo)
+                        if (c0 + j < c_hi) *o = v[j];
+                }
             }
+            asm volatile("tcgen05.fence::before_thread_sync;");
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sh.acc_empty[acc]);
         }
-        asm volatile("tcgen05.fence::before_thread_sync;");
-        __syncthreads();
     }
-    if (fail_s && tid == 0) atomicExch(a.err, 1);
+    __syncthreads();
+    if (sh.failed && threadIdx.x == 0) atomicExch(a.err, 1);
     tc_teardown(taddr, ncols);
 }
 
@@ -282,8 +395,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_combine(CombineArgs a) {
 // over the floats of the vectors: A rows = the nin basis vectors (rows >= nin are zero),
 // B rows c < nq = R_c, nq <= c < 2 nq = rot(R_{c-nq}) with (re, im) -> (im, -re), so that
 // for complex vectors sum_k A[i][k] B[c][k] = Re <v_i, r_c> and the rotated rows give
-// Im <v_i, r_c>.  Each block takes segments of kSeg floats in turn; after each segment
-// the FP32 accumulator is added into FP64 registers and the next segment starts afresh.
+// Im <v_i, r_c>.  After each segment of kSegChunks chunks the FP32 accumulator is added into
+// FP64 registers and the next segment starts afresh.
 struct DotsArgs {
     const float *V;
     long ldv;
@@ -297,130 +410,169 @@ struct DotsArgs {
 };
 constexpr int kSegChunks = 64;      // 64 chunks of 32 floats per segment
 
-// The dots' operands of one thread for chunk ch: A items w = tid + 256 i (i < 4; row
-// 8 (w >> 6) + (w & 7), k quad (w >> 3) & 7) and at most one B item w = tid (npad <= 32)
-__device__ __forceinline__ void dots_load(const DotsArgs &a, long ch, int tid, float4 (&va)[4], float4 &vb) {
+// The dots' operands of one thread of a group for chunk ch: A items w = tid + 128 i (i < 8;
+// row 8 (w >> 6) + (w & 7), k quad (w >> 3) & 7), and B items w = tid + 128 i < 8 npad (i < 2;
+// rows nq .. 2 nq - 1 are rotated when taken from the ring)
+__device__ __forceinline__ void dots_load(const DotsArgs &a, long ch, int tid, float4 *slot) {
     const long k0 = ch * kKC;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int w = tid + kTcThreads * q;
+    for (int q = 0; q < 10; ++q) {
+        const int w = tid + kFill * (q < 8 ? q : q - 8);
+        if (q >= 8 && w >= a.npad * (kKC / 4)) break;
         const int i = 8 * (w >> 6) + (w & 7), kq = (w >> 3) & 7;
-        va[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (i < a.nin) va[q] = *reinterpret_cast<const float4 *>(a.V + (size_t)i * a.ldv + k0 + 4 * kq);
-    }
-    vb = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (tid < a.npad * (kKC / 4)) {
-        const int c = 8 * (tid >> 6) + (tid & 7), kq = (tid >> 3) & 7;
-        if (c < a.nq) {
-            vb = *reinterpret_cast<const float4 *>(a.R + (size_t)c * a.ldr + k0 + 4 * kq);
-        } else if (c < 2 * a.nq) {
-            const float4 u = *reinterpret_cast<const float4 *>(a.R + (size_t)(c - a.nq) * a.ldr + k0 + 4 * kq);
-            vb = make_float4(u.y, -u.x, u.w, -u.z);
+        const float *src = a.V;
+        bool ok;
+        if (q < 8) {
+            ok = i < a.nin;
+            if (ok) src = a.V + (size_t)i * a.ldv + k0 + 4 * kq;
+        } else {
+            ok = i < 2 * a.nq;
+            if (ok) src = a.R + (size_t)(i < a.nq ? i : i - a.nq) * a.ldr + k0 + 4 * kq;
         }
+        ring_load(slot + q * kFill, src, ok);
     }
 }
 
-__global__ void __launch_bounds__(kTcThreads, 1) k_tc_dots(DotsArgs a) {
+// Bound by memory: nin + nq vectors are read, 128 x npad partial sums written per block.
+// Every block takes consecutive segments, one FP32 accumulation of kSegChunks chunks each.
+constexpr int kDotsStages = 2, kDotsRing = 6;
+__global__ void __launch_bounds__(tc_threads(kDotsStages), 1) k_tc_dots(DotsArgs a) {
     extern __shared__ __align__(1024) unsigned char smem[];
-    const int a_bytes = 128 * kKC * 4, b_bytes = a.npad * kKC * 4;
-    const int stage_bytes = 2 * a_bytes + 2 * b_bytes;
-    __shared__ __align__(8) uint64_t mbar[2];
-    __shared__ uint32_t tbase;
-    __shared__ int fail_s;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int ncols = tmem_cols(a.npad);
-    if (tid == 0) fail_s = 0;
-    tc_setup(mbar, &tbase, ncols);
-    const uint32_t taddr = tbase;
-    const uint32_t idesc = idesc_tf32(a.npad, 0u);
-    const long nchunks = a.len / kKC;
-    const long nseg = (nchunks + kSegChunks - 1) / kSegChunks;
-    // per thread: its TMEM row (lane quarter warp & 3) and half of the columns, in FP64
-    const int lq = warp & 3, half = warp >> 2;
-    const int c_lo = half * (a.npad / 2);
-    double acc[16];
+    __shared__ __align__(8) TcShared<kDotsStages, kDotsRing> sh;
+    const int b_bytes = a.npad * kKC * 4;
+    const int stage_bytes = 2 * kABytes + 2 * b_bytes;
+    float4 *ring = reinterpret_cast<float4 *>(smem + kDotsStages * stage_bytes);   // [ring][8 A + 2 B][kFill]
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+    const int ncols = tmem_cols(2 * a.npad);
+    const long nchunks = a.len / kKC, nseg = (nchunks + kSegChunks - 1) / kSegChunks;
+    const long first = nseg * blockIdx.x / gridDim.x * kSegChunks;
+    const long last = min(nchunks, nseg * (blockIdx.x + 1) / gridDim.x * kSegChunks);
+    const uint32_t taddr = tc_setup(sh, ncols);
+    volatile int *failed = &sh.failed;
+    const int ft = threadIdx.x - 32 * (kEpiWarps + 1), tid = ft % kFill;
+    float4 *slots = ring + tid;
+    const long mine = last - first;
+    if (ft >= kFill) {
+        // ---- split.  A chunk: 128 rows x 32 k, K-major; a warp instruction covers 8 rows x 4
+        // k quads
+        const int grp = ft / kFill - 1;
+        unsigned char *sbase = smem + grp * stage_bytes;
+        float *Ahi = reinterpret_cast<float *>(sbase), *Alo = reinterpret_cast<float *>(sbase + kABytes);
+        float *Bhi = reinterpret_cast<float *>(sbase + 2 * kABytes);
+        float *Blo = reinterpret_cast<float *>(sbase + 2 * kABytes + b_bytes);
+        int slot = grp;
+        uint32_t round = 0, rround = 0;        // uses of the stage and of the slot before this one
+        for (long q = grp; q < mine; q += kDotsStages, ++round) {
+            const float4 *raw = slots + (size_t)slot * 10 * kFill;
+            if (!__all_sync(0xffffffffu, mbar_wait(&sh.raw_full[slot], rround & 1u, failed))) break;
+            if (round > 0 && !__all_sync(0xffffffffu, mbar_wait(&sh.empty[grp], (round - 1) & 1u, failed))) break;
 #pragma unroll
-    for (int j = 0; j < 16; ++j) acc[j] = 0.0;
-    StageSync ss;
-    // operands of the next chunk are loaded into registers while the current MMAs run
-    float4 va[4], vb;
-    if ((long)blockIdx.x < nseg) dots_load(a, (long)blockIdx.x * kSegChunks, tid, va, vb);
-    for (long sg = blockIdx.x; sg < nseg; sg += gridDim.x) {
-        const long ch0 = sg * kSegChunks, ch1 = min(nchunks, ch0 + kSegChunks);
-        for (long ch = ch0; ch < ch1; ++ch) {
-            const int st = (int)((ch - ch0) & 1);
-            unsigned char *sbase = smem + st * stage_bytes;
-            float *Ahi = reinterpret_cast<float *>(sbase), *Alo = reinterpret_cast<float *>(sbase + a_bytes);
-            float *Bhi = reinterpret_cast<float *>(sbase + 2 * a_bytes);
-            float *Blo = reinterpret_cast<float *>(sbase + 2 * a_bytes + b_bytes);
-            if (!ss.drain(mbar, st) && tid == 0) fail_s = 1;
-            __syncthreads();
-            if (fail_s) break;
-            // A chunk: 128 rows x 32 k, K-major; a warp instruction covers 8 rows x 4 k quads
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int w = tid + kTcThreads * q;
-                st_split(Ahi, Alo, (w >> 6) * 256 + ((w >> 3) & 7) * 32 + (w & 7) * 4, va[q]);
+            for (int k = 0; k < 8; ++k) {
+                const int w = tid + kFill * k;
+                st_split(Ahi, Alo, (w >> 6) * 256 + ((w >> 3) & 7) * 32 + (w & 7) * 4, raw[k * kFill]);
             }
-            if (tid < a.npad * (kKC / 4))
-                st_split(Bhi, Blo, (tid >> 6) * 256 + ((tid >> 3) & 7) * 32 + (tid & 7) * 4, vb);
-            asm volatile("fence.proxy.async.shared::cta;");
-            __syncthreads();
-            if (tid == 0) {
-                asm volatile("tcgen05.fence::after_thread_sync;");
 #pragma unroll
-                for (int ks = 0; ks < kKC / 8; ++ks) {
-                    const uint64_t ah = sdesc(su32(Ahi) + ks * 256, 128, 1024);
-                    const uint64_t al = sdesc(su32(Alo) + ks * 256, 128, 1024);
-                    const uint64_t bh = sdesc(su32(Bhi) + ks * 256, 128, 1024);
-                    const uint64_t bl = sdesc(su32(Blo) + ks * 256, 128, 1024);
-                    mma_tf32(taddr, ah, bh, idesc, (ch > ch0 || ks > 0) ? 1u : 0u);
-                    mma_tf32(taddr, ah, bl, idesc, 1u);
-                    mma_tf32(taddr, al, bh, idesc, 1u);
+            for (int k = 0; k < 2; ++k) {
+                const int w = tid + kFill * k;
+                if (w < a.npad * (kKC / 4)) {
+                    float4 u = raw[(8 + k) * kFill];
+                    if (8 * (w >> 6) + (w & 7) >= a.nq) u = make_float4(u.y, -u.x, u.w, -u.z);
+                    st_split(Bhi, Blo, (w >> 6) * 256 + ((w >> 3) & 7) * 32 + (w & 7) * 4, u);
                 }
-                commit_to(&mbar[st]);
             }
-            ++ss.issued[st];
-            if (ch + 1 < ch1) dots_load(a, ch + 1, tid, va, vb);
-            else if (sg + gridDim.x < nseg) dots_load(a, (sg + gridDim.x) * kSegChunks, tid, va, vb);
+            asm volatile("fence.proxy.async.shared::cta;");
+            __syncwarp();
+            if (lane == 0) {
+                mbar_arrive(&sh.raw_empty[slot]);
+                mbar_arrive(&sh.full[grp]);
+            }
+            if ((slot += kDotsStages) >= kDotsRing) { slot = grp; ++rround; }
         }
-        if (fail_s) break;
-        bool okd = ss.drain(mbar, 0);
-        okd = ss.drain(mbar, 1) && okd;
-        if (!okd && tid == 0) fail_s = 1;
-        __syncthreads();
-        if (fail_s) break;
-        asm volatile("tcgen05.fence::after_thread_sync;");
-        for (int c0 = 0; c0 < a.npad / 2; c0 += 8) {
-            float v[8];
-            tmem_ld8(taddr + ((uint32_t)(32 * lq) << 16) + (uint32_t)(c_lo + c0), v);
+    } else if (ft >= 0) {
+        // ---- copy
+        int slot = 0;
+        uint32_t round = 0;
+        for (long q = 0; q < mine; ++q) {
+            if (round > 0 && !mbar_wait(&sh.raw_empty[slot], (round - 1) & 1u, failed)) break;
+            dots_load(a, first + q, tid, slots + (size_t)slot * 10 * kFill);
+            ring_arrive(&sh.raw_full[slot]);
+            if (++slot == kDotsRing) { slot = 0; ++round; }
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");       // no copy may land after the block has ended
+    } else if (warp == kEpiWarps) {
+        // ---- MMA: one accumulator per segment (the warp is uniform; lane 0 issues)
+        const uint32_t idesc = idesc_tf32(a.npad, 0u);
+        const uint32_t d_stage = sdesc_lo(su32(smem)), w_stage = stage_bytes >> 4, w_b = b_bytes >> 4;
+        int st = 0, n = 0;
+        uint32_t round = 0;
+        bool ok = true;
+        for (long ch0 = first; ch0 < last && ok; ch0 += kSegChunks, ++n) {
+            const int acc = n & 1, nch = (int)(min(last, ch0 + kSegChunks) - ch0);
+            if (n >= 2 && !__all_sync(0xffffffffu, mbar_wait(&sh.acc_empty[acc], ((n >> 1) - 1) & 1, failed))) break;
+            for (int ch = 0; ch < nch; ++ch) {
+                ok = __all_sync(0xffffffffu, mbar_wait(&sh.full[st], round & 1u, failed));
+                if (!ok) break;
+                asm volatile("tcgen05.fence::after_thread_sync;");
+                const uint32_t da = d_stage + st * w_stage, db = da + (2 * kABytes >> 4);
+                if (lane == 0) {
+                    chunk_mmas(taddr + acc * a.npad, da, da + (kABytes >> 4), db, db + w_b, idesc, ch == 0);
+                    commit_to(&sh.empty[st]);
+                }
+                if (++st == kDotsStages) { st = 0; ++round; }
+            }
+            if (ok && lane == 0) commit_to(&sh.acc_full[acc]);
+        }
+        __syncwarp();
+    } else {
+        // ---- sums over the segments in FP64: a thread has one row (basis vector) and half of
+        // the columns
+        double sum[16];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) acc[c0 + j] += (double)v[j];
+        for (int j = 0; j < 16; ++j) sum[j] = 0.0;
+        int n = 0;
+        const int lq = warp & 3, c_lo = (warp >> 2) * (a.npad / 2);
+        for (long ch0 = first; ch0 < last; ch0 += kSegChunks, ++n) {
+            const int acc = n & 1;
+            if (!__all_sync(0xffffffffu, mbar_wait(&sh.acc_full[acc], (n >> 1) & 1, failed))) break;
+            asm volatile("tcgen05.fence::after_thread_sync;");
+            float v[16];
+            tmem_read(taddr + ((uint32_t)(32 * lq) << 16) + (uint32_t)(acc * a.npad + c_lo), a.npad == 32, v);
+#pragma unroll
+            for (int j = 0; j < 16; ++j)
+                if (j < a.npad / 2) sum[j] += (double)v[j];
+            asm volatile("tcgen05.fence::before_thread_sync;");
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sh.acc_empty[acc]);
         }
-        asm volatile("tcgen05.fence::before_thread_sync;");
-        __syncthreads();
+        double *out = a.Cpart + ((size_t)blockIdx.x * 128 + 32 * lq + lane) * a.npad + c_lo;
+#pragma unroll
+        for (int j = 0; j < 16; ++j)
+            if (j < a.npad / 2) out[j] = sum[j];
     }
-    const int row = 32 * lq + lane;
-    double *out = a.Cpart + ((size_t)blockIdx.x * 128 + row) * a.npad + c_lo;
-    for (int j = 0; j < a.npad / 2; ++j) out[j] = acc[j];
-    if (fail_s && tid == 0) atomicExch(a.err, 1);
+    __syncthreads();
+    if (sh.failed && threadIdx.x == 0) atomicExch(a.err, 1);
     tc_teardown(taddr, ncols);
 }
 
 // C[i][q] (complex) = sum over blocks of Cpart[blk][i][q] + i Cpart[blk][i][nq + q], in a
-// fixed order (one thread per entry)
-__global__ void k_tc_dots_sum(const double *__restrict__ Cpart, int nblk, int nin, int nq, int npad,
-                              double2 *__restrict__ C) {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= nin * nq) return;
-    const int i = e / nq, q = e % nq;
+// fixed order.  One block per basis vector i; its threads are (group of partials, column),
+// so a group's reads are one contiguous row (one thread per entry, striding over all blocks'
+// partials, took 156 us for 121 x 16 entries).
+__global__ void __launch_bounds__(256)
+k_tc_dots_sum(const double *__restrict__ Cpart, int nblk, int nin, int nq, int npad, double2 *__restrict__ C) {
+    __shared__ double sm[256];
+    const int i = blockIdx.x, col = threadIdx.x % npad, grp = threadIdx.x / npad, ngrp = 256 / npad;
+    double t = 0.0;
+    for (int b = grp; b < nblk; b += ngrp) t += Cpart[((size_t)b * 128 + i) * npad + col];
+    sm[threadIdx.x] = t;
+    __syncthreads();
+    if ((int)threadIdx.x >= nq) return;
     double re = 0.0, im = 0.0;
-    for (int b = 0; b < nblk; ++b) {
-        const double *p = Cpart + ((size_t)b * 128 + i) * npad;
-        re += p[q];
-        im += p[nq + q];
+    for (int k = 0; k < ngrp; ++k) {
+        re += sm[k * npad + threadIdx.x];
+        im += sm[k * npad + nq + threadIdx.x];
     }
-    C[(size_t)q * nin + i] = make_double2(re, im);
+    C[(size_t)threadIdx.x * nin + i] = make_double2(re, im);
 }
 
 // round to the 10-bit TF32 mantissa (nearest, ties away), as cvt.rna.tf32.f32 does
@@ -445,28 +597,43 @@ int num_sms() {
     return n;
 }
 
-int check_err(TcScratch &sc, cudaStream_t st) {
-    int h = 0;
-    DLZ_CUDA_TRY(cudaMemcpyAsync(&h, sc.err.ptr(), sizeof(int), cudaMemcpyDeviceToHost, st));
-    DLZ_CUDA_TRY(cudaStreamSynchronize(st));
-    if (h) return fail(DLZ_ERR_DEVICE_TIMEOUT, "a tensor-core kernel's mbarrier wait gave up");
-    return DLZ_OK;
+constexpr size_t kErrBytes = 256;      // the error word at the start of a call's scratch
+
+// The combine's launch: stages, raw chunks in the ring, and whether the coefficients stay in
+// shared memory (with as many raw chunks as fit beside them) or are copied per chunk
+typedef void (*CombineKernel)(CombineArgs);
+struct CombineForm {
+    CombineKernel fn;
+    int stages, smem;
+};
+CombineForm pick_combine(int npad, int kpad) {
+    const int b_all = 2 * npad * kpad * 4, b_stage = 2 * npad * kKC * 4;
+    // hi and lo of an A chunk per stage, R raw chunks
+    if (10 * kABytes + b_all <= kTcMaxSmem) return {k_tc_combine<2, 6, true>, 2, 10 * kABytes + b_all};
+    if (8 * kABytes + b_all <= kTcMaxSmem) return {k_tc_combine<2, 4, true>, 2, 8 * kABytes + b_all};
+    if (10 * kABytes + 2 * b_stage <= kTcMaxSmem) return {k_tc_combine<2, 6, false>, 2, 10 * kABytes + 2 * b_stage};
+    if (8 * kABytes + 2 * b_stage <= kTcMaxSmem) return {k_tc_combine<2, 4, false>, 2, 8 * kABytes + 2 * b_stage};
+    return {k_tc_combine<1, 4, false>, 1, 6 * kABytes + b_stage};
 }
 
 }  // namespace
 
 int tc_prepare() {
-    // dynamic shared memory beyond 48 KB (set once, outside any graph capture): at most
-    // two stages of 2 x 16 KB (A) + 2 x 32 KB (B, npad = 256) = 192 KB; the opt-in limit
-    // (227 KB) also covers the kernels' static shared memory
+    // dynamic shared memory beyond 48 KB (set once, outside any graph capture); the opt-in
+    // limit (227 KB) also covers the kernels' static shared memory
     static int done = 0;
     if (done) return DLZ_OK;
-    DLZ_CUDA_TRY(cudaFuncSetAttribute(k_tc_combine, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcMaxSmem));
+    for (CombineKernel k : {(CombineKernel)k_tc_combine<2, 6, true>, (CombineKernel)k_tc_combine<2, 4, true>,
+                            (CombineKernel)k_tc_combine<2, 6, false>, (CombineKernel)k_tc_combine<2, 4, false>,
+                            (CombineKernel)k_tc_combine<1, 4, false>})
+        DLZ_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcMaxSmem));
     DLZ_CUDA_TRY(cudaFuncSetAttribute(k_tc_dots, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcMaxSmem));
     done = 1;
     return DLZ_OK;
 }
 
+// Both calls keep everything they need on the device in one allocation of the scratch (the
+// error word first), and read the error word back with the results.
 int tc_combine32(TcScratch &sc, cudaStream_t st, float *out, long ldo, const float *in, long ldv, int nin, long len,
                  const double *coef, int nout, bool cplx, long long *launches) {
     if (nin < 1 || nout < 1 || len < 1) return DLZ_OK;
@@ -474,14 +641,17 @@ int tc_combine32(TcScratch &sc, cudaStream_t st, float *out, long ldo, const flo
     DLZ_TRY(tc_prepare());
     const int K = cplx ? 2 * nin : nin;
     const int kpad = round_up(K, kKC), npad = std::max(16, round_up(nout, 16));
-    // Bt[j][k] (K contiguous): real coef[i][j] at k = i; complex: Re at k = i, Im at k = nin + i
-    std::vector<float> hi((size_t)npad * kpad, 0.f), lo((size_t)npad * kpad, 0.f);
+    // the error word (0), then Bt[j][k] (K contiguous) in two parts: real coef[i][j] at
+    // k = i; complex: Re at k = i, Im at k = nin + i
+    const size_t nb = (size_t)npad * kpad, ne = kErrBytes / sizeof(float);
+    std::vector<float> h(ne + 2 * nb, 0.f);
+    float *hi = h.data() + ne, *lo = hi + nb;
     for (int j = 0; j < nout; ++j)
         for (int i = 0; i < nin; ++i) {
             const float re = (float)(cplx ? coef[2 * ((size_t)i * nout + j)] : coef[(size_t)i * nout + j]);
-            const float h = tf32_round_host(re);
-            hi[(size_t)j * kpad + i] = h;
-            lo[(size_t)j * kpad + i] = re - h;
+            const float hr = tf32_round_host(re);
+            hi[(size_t)j * kpad + i] = hr;
+            lo[(size_t)j * kpad + i] = re - hr;
             if (cplx) {
                 const float im = (float)coef[2 * ((size_t)i * nout + j) + 1];
                 const float hm = tf32_round_host(im);
@@ -489,25 +659,22 @@ int tc_combine32(TcScratch &sc, cudaStream_t st, float *out, long ldo, const flo
                 lo[(size_t)j * kpad + nin + i] = im - hm;
             }
         }
-    const size_t nb = hi.size() * sizeof(float);
-    DLZ_TRY(sc.coef.reserve(2 * nb));
-    float *dhi = sc.coef.as<float>(), *dlo = dhi + hi.size();
-    DLZ_CUDA_TRY(cudaMemcpyAsync(dhi, hi.data(), nb, cudaMemcpyHostToDevice, st));
-    DLZ_CUDA_TRY(cudaMemcpyAsync(dlo, lo.data(), nb, cudaMemcpyHostToDevice, st));
-    DLZ_TRY(sc.err.reserve(sizeof(int)));
-    DLZ_CUDA_TRY(cudaMemsetAsync(sc.err.ptr(), 0, sizeof(int), st));
+    DLZ_TRY(sc.buf.reserve(h.size() * sizeof(float)));
+    DLZ_CUDA_TRY(cudaMemcpyAsync(sc.buf.ptr(), h.data(), h.size() * sizeof(float), cudaMemcpyHostToDevice, st));
     CombineArgs a;
-    a.V = in; a.ldv = ldv; a.nin = nin; a.rows = len; a.Bhi = dhi; a.Blo = dlo;
+    a.V = in; a.ldv = ldv; a.nin = nin; a.rows = len; a.Bhi = sc.buf.as<float>() + ne; a.Blo = a.Bhi + nb;
     a.kpad = kpad; a.npad = npad; a.nout = nout; a.cplx = cplx ? 1 : 0; a.Out = out; a.ldo = ldo;
-    a.err = sc.err.as<int>();
-    const int smem = 2 * (2 * 128 * kKC * 4 + 2 * npad * kKC * 4);
+    a.err = sc.buf.as<int>();
+    const CombineForm f = pick_combine(npad, kpad);
     const long ntiles = (len + 127) / 128;
-    const int per_sm = smem <= 100 * 1024 ? 2 : 1;
-    const int grid = (int)std::min<long>(ntiles, (long)per_sm * num_sms());
-    k_tc_combine<<<grid, kTcThreads, smem, st>>>(a);
+    f.fn<<<(int)std::min<long>(ntiles, num_sms()), tc_threads(f.stages), f.smem, st>>>(a);
     if (launches) *launches += 1;
     DLZ_CUDA_TRY(cudaGetLastError());
-    return check_err(sc, st);
+    int err = 0;
+    DLZ_CUDA_TRY(cudaMemcpyAsync(&err, sc.buf.ptr(), sizeof(int), cudaMemcpyDeviceToHost, st));
+    DLZ_CUDA_TRY(cudaStreamSynchronize(st));
+    if (err) return fail(DLZ_ERR_DEVICE_TIMEOUT, "a tensor-core kernel's mbarrier wait gave up");
+    return DLZ_OK;
 }
 
 int tc_dots32(TcScratch &sc, cudaStream_t st, double2 *C_host, const float *V, long ldv, int nin, const float *R,
@@ -516,26 +683,29 @@ int tc_dots32(TcScratch &sc, cudaStream_t st, double2 *C_host, const float *V, l
     if (nin > 128 || nq > 16 || len % kKC || ldv % 4 || ldr % 4) return fail(DLZ_ERR_BADARG, "tensor-core dots: shape");
     DLZ_TRY(tc_prepare());
     const int npad = std::max(16, round_up(2 * nq, 16));
-    const long nchunks = len / kKC, nseg = (nchunks + kSegChunks - 1) / kSegChunks;
-    const int smem = 2 * (2 * 128 * kKC * 4 + 2 * npad * kKC * 4);
-    const int per_sm = smem <= 100 * 1024 ? 2 : 1;
-    const int grid = (int)std::max<long>(1, std::min<long>(nseg, (long)per_sm * num_sms()));
-    DLZ_TRY(sc.part.reserve((size_t)grid * 128 * npad * sizeof(double) + (size_t)nin * nq * sizeof(double2)));
-    double *part = sc.part.as<double>();
-    double2 *Cd = reinterpret_cast<double2 *>(part + (size_t)grid * 128 * npad);
-    DLZ_TRY(sc.err.reserve(sizeof(int)));
-    DLZ_CUDA_TRY(cudaMemsetAsync(sc.err.ptr(), 0, sizeof(int), st));
+    const int smem = kDotsStages * (2 * kABytes + 2 * npad * kKC * 4) + kDotsRing * 10 * kFill * (int)sizeof(float4);
+    static_assert(kDotsStages * (2 * kABytes + 2 * 32 * kKC * 4) + kDotsRing * 10 * kFill * 16 <= kTcMaxSmem, "ring depth");
+    const long nseg = (len / kKC + kSegChunks - 1) / kSegChunks;
+    const int grid = (int)std::max<long>(1, std::min<long>(nseg, num_sms()));
+    const size_t ne = (size_t)nin * nq, npart = (size_t)grid * 128 * npad;
+    DLZ_TRY(sc.buf.reserve(kErrBytes + ne * sizeof(double2) + npart * sizeof(double)));
+    double2 *Cd = reinterpret_cast<double2 *>(sc.buf.as<char>() + kErrBytes);
+    double *part = reinterpret_cast<double *>(Cd + ne);
+    DLZ_CUDA_TRY(cudaMemsetAsync(sc.buf.ptr(), 0, sizeof(int), st));
     DotsArgs a;
     a.V = V; a.ldv = ldv; a.nin = nin; a.R = R; a.ldr = ldr; a.nq = nq; a.npad = npad; a.len = len;
-    a.Cpart = part; a.err = sc.err.as<int>();
-    k_tc_dots<<<grid, kTcThreads, smem, st>>>(a);
-    const int ne = nin * nq;
-    k_tc_dots_sum<<<(ne + 127) / 128, 128, 0, st>>>(part, grid, nin, nq, npad, Cd);
+    a.Cpart = part; a.err = sc.buf.as<int>();
+    k_tc_dots<<<grid, tc_threads(kDotsStages), smem, st>>>(a);
+    k_tc_dots_sum<<<nin, 256, 0, st>>>(part, grid, nin, nq, npad, Cd);
     if (launches) *launches += 2;
     DLZ_CUDA_TRY(cudaGetLastError());
-    DLZ_TRY(check_err(sc, st));
-    DLZ_CUDA_TRY(cudaMemcpyAsync(C_host, Cd, (size_t)ne * sizeof(double2), cudaMemcpyDeviceToHost, st));
+    std::vector<char> h(kErrBytes + ne * sizeof(double2));
+    DLZ_CUDA_TRY(cudaMemcpyAsync(h.data(), sc.buf.ptr(), h.size(), cudaMemcpyDeviceToHost, st));
     DLZ_CUDA_TRY(cudaStreamSynchronize(st));
+    int err = 0;
+    std::memcpy(&err, h.data(), sizeof(int));
+    if (err) return fail(DLZ_ERR_DEVICE_TIMEOUT, "a tensor-core kernel's mbarrier wait gave up");
+    std::memcpy(C_host, h.data() + kErrBytes, ne * sizeof(double2));
     return DLZ_OK;
 }
 

@@ -134,19 +134,6 @@ template <typename T> struct UserRow {
     static constexpr int W = Field<T>::vec_per_site, RS = W + 1;
 };
 template <typename T, int BT>
-__device__ inline void user_row_to_regs(const typename Field<T>::vec *sm, cx<T> (&v)[12]) {
-    const typename Field<T>::vec *row = sm + threadIdx.x * UserRow<T>::RS;
-#pragma unroll
-    for (int c = 0; c < UserRow<T>::W; ++c) {
-        if constexpr (sizeof(T) == 4) {
-            v[2 * c] = make_float2(row[c].x, row[c].y);
-            v[2 * c + 1] = make_float2(row[c].z, row[c].w);
-        } else {
-            v[c] = row[c];
-        }
-    }
-}
-template <typename T, int BT>
 __device__ inline void user_regs_to_row(typename Field<T>::vec *sm, const cx<T> (&v)[12]) {
     typename Field<T>::vec *row = sm + threadIdx.x * UserRow<T>::RS;
 #pragma unroll
@@ -179,17 +166,15 @@ template <typename T> struct UserGather {
 };
 
 // One application of the stencil for a user's vectors, all right-hand sides in one launch:
-// UIN / UOUT say whether in / out are in the user layout or internal planes.  A user's call
-// is therefore one launch where the neighbours can be read from the user layout, and two
-// (pack, stencil) where they should be packed first:
-//   FP64 is bound by its ALU (888 FP64 instructions per site at 2 per cycle and SM), which
-//   hides the strided reads: always straight from the user layout;
-//   FP32 pays about four times the L1 cycles for strided reads: packed first, except for
-//   few sites (kDirectSites), where the call is a chain of latencies.
-// Measured per call, against a pack, stencil and unpack launch per right-hand side with
-// three temporary device allocations: FP32 D on 8^4, 1 RHS 40.0 -> 14.9 us; FP32 Q on
-// 16^3 x 32, 12 RHS 675 -> 197 us (floor 48 us); FP64 D^dag D on 12 x 10 x 14 x 18, 3 RHS
-// 768 -> 337 us (FP64-ALU floor 256 us).
+// UIN / UOUT say whether in / out are in the user layout or internal planes (the middle
+// vector of D^dag D).  The neighbours are read straight from the user layout.  FP64 is bound
+// by its ALU (888 FP64 instructions per site at 2 per cycle and SM), which hides the strided
+// reads; FP32 pays more L1 cycles for them than for planes, but less than a pass that packs
+// the vectors first.  FP32 Q, direct and packed first: 8^4, 1 RHS 15.0 and 19.3 us; 16^4, 3
+// RHS 33.4 and 35.5 us; 16^3 x 32, 12 RHS 160 and 195 us; 24^3 x 48, 16 RHS 1011 and 1339 us.
+// Against a pack, stencil and unpack launch per right-hand side with three temporary device
+// allocations: FP32 D on 8^4, 1 RHS 40.0 -> 14.9 us; FP32 Q on 16^3 x 32, 12 RHS 675 -> 160 us
+// (floor 48 us); FP64 D^dag D on 12 x 10 x 14 x 18, 3 RHS 768 -> 337 us (FP64-ALU floor 256 us).
 template <typename T, bool G5IN, bool G5OUT, bool UIN, bool UOUT, int BT>
 __global__ void __launch_bounds__(BT, sizeof(T) == 4 ? 768 / BT : 1)
 k_wilson_user(typename Field<T>::vec *__restrict__ out, const typename Field<T>::vec *__restrict__ in,
@@ -225,22 +210,6 @@ k_wilson_user(typename Field<T>::vec *__restrict__ out, const typename Field<T>:
     }
 }
 
-// user layout -> planes through the same rows; blockIdx.y: the right-hand side
-template <typename T>
-__global__ void __launch_bounds__(128)
-k_pack_user(typename Field<T>::vec *__restrict__ dst, const typename Field<T>::vec *__restrict__ src, int V) {
-    __shared__ typename Field<T>::vec sm[128 * UserRow<T>::RS];
-    const int s0 = blockIdx.x * 128, nb = min(128, V - s0);
-    const size_t base = (size_t)blockIdx.y * UserRow<T>::W * V;
-    for (int j = threadIdx.x; j < nb * UserRow<T>::W; j += 128)
-        sm[(j / UserRow<T>::W) * UserRow<T>::RS + j % UserRow<T>::W] = src[base + (size_t)s0 * UserRow<T>::W + j];
-    __syncthreads();
-    if ((int)threadIdx.x >= nb) return;
-    cx<T> v[12];
-    user_row_to_regs<T, 128>(sm, v);
-    Field<T>::store(dst + base, V, s0 + threadIdx.x, v);
-}
-
 // Threads of a plain-order block (32, 64 or 128) for `total` sites of FP64-ALU-bound work:
 // the SM with the most sites ends last, so the size that gives the fullest SMs fewest sites
 // (31680 sites on 152 SMs: 256 with 128 threads, 224 with 32).
@@ -256,9 +225,6 @@ int balanced_threads(int V, int nrhs) {
     }
     return best;
 }
-
-// Sites times right-hand sides up to which an FP32 call reads the user layout directly.
-constexpr long kDirectSites = 40000;
 
 template <typename T, bool UIN, bool UOUT, int BT>
 void launch_user_bt(Op &op, typename Field<T>::vec *out, const typename Field<T>::vec *in,
@@ -289,15 +255,6 @@ int launch_user(Op &op, void *out, const void *in, int which, int nrhs) {
     DLZ_CUDA_TRY(cudaGetLastError());
     return DLZ_OK;
 }
-template <typename T>
-int launch_pack_user(Op &op, void *dst, const void *src, int nrhs) {
-    k_pack_user<T><<<dim3((unsigned)((op.g.V + 127) / 128), nrhs), 128, 0, op.stream>>>(
-        (typename Field<T>::vec *)dst, (const typename Field<T>::vec *)src, op.g.V);
-    op.prof.launches++;
-    DLZ_CUDA_TRY(cudaGetLastError());
-    return DLZ_OK;
-}
-
 // ------------------------------------------------------------------ layout kernels
 __global__ void k_pack64(double2 *__restrict__ dst, const double2 *__restrict__ src, int V) {
     const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;   // canonical index s*12 + a
@@ -392,28 +349,22 @@ int apply32(Op &op, float4 *out, const float4 *in, int which, float4 *tmp) {
 // ------------------------------------------------------------------ a user's call
 // FP32 reads 16-byte words of the user's vectors; a vector that is only 8-byte aligned (a
 // view at an odd complex element) takes the layout kernels that read single complex numbers.
-static bool user_direct(const Op &op, const void *in, const void *out, int dtype, int nrhs, bool &aligned) {
-    aligned = (((uintptr_t)in | (uintptr_t)out) & 15) == 0;
-    if (dtype == DLZ_F64) return true;
-    return aligned && (long)op.g.V * nrhs <= kDirectSites;
+static bool user_direct(const Op &op, const void *in, const void *out, int dtype) {
+    if (op.eo || dtype == DLZ_BF16) return false;
+    return dtype == DLZ_F64 || (((uintptr_t)in | (uintptr_t)out) & 15) == 0;
 }
 
-size_t apply_user_scratch(const Op &op, int which, const void *in, const void *out, int dtype, int nrhs) {
+size_t apply_user_scratch(const Op &op, int which, const void *in, const void *out, int dtype) {
     const size_t vec = (size_t)12 * op.g.V * (dtype == DLZ_F64 ? 16 : dtype == DLZ_F32 ? 8 : 4);
-    const int mid = which == DLZ_DDAGD ? 1 : 0;
-    if (dtype == DLZ_BF16 || op.eo) return (2 + mid) * vec;
-    bool aligned;
-    if (user_direct(op, in, out, dtype, nrhs, aligned)) return mid * vec;
-    return (aligned ? 1 + mid : 2 + mid) * vec;
+    return ((user_direct(op, in, out, dtype) ? 0 : 2) + (which == DLZ_DDAGD ? 1 : 0)) * vec;
 }
 
 // out = A in on nrhs user vectors, `scratch` of at least apply_user_scratch() bytes; takes as
 // many right-hand sides at a time as it holds.  D^dag D = Q Q, the middle vector in planes.
 int apply_user(Op &op, int which, const void *in, void *out, int dtype, int nrhs, void *scratch, size_t bytes) {
     const size_t n = (size_t)12 * op.g.V, esz = dtype == DLZ_F64 ? 16 : 8;
-    const size_t vec = n * (dtype == DLZ_BF16 ? 4 : esz), per = apply_user_scratch(op, which, in, out, dtype, nrhs);
-    bool aligned;
-    const bool direct = user_direct(op, in, out, dtype, nrhs, aligned);
+    const size_t vec = n * (dtype == DLZ_BF16 ? 4 : esz), per = apply_user_scratch(op, which, in, out, dtype);
+    const bool direct = user_direct(op, in, out, dtype);
     // (the launches' grids: at most 65535 right-hand sides in y, 2^31 - 1 blocks in x)
     const long most = std::max(1L, std::min(65535L, (1L << 30) / ((op.g.V + 31) / 32)));
     const int chunk = (int)std::min<size_t>({(size_t)nrhs, (size_t)most, per ? std::max<size_t>(1, bytes / per) : (size_t)nrhs});
@@ -435,29 +386,19 @@ int apply_user(Op &op, int which, const void *in, void *out, int dtype, int nrhs
             DLZ_TRY(eo_apply64(op, (double2 *)b, (const double2 *)a, first, nb));
             if (two) DLZ_TRY(eo_apply64(op, (double2 *)c, (const double2 *)b, DLZ_Q, nb));
             DLZ_TRY(unpack64(op, (double2 *)dst, (const double2 *)(two ? c : b), nb));
-        } else if (op.eo || (dtype == DLZ_F32 && !aligned)) {
+        } else if (!direct) {
             DLZ_TRY(pack32(op, (float4 *)a, (const float2 *)src, nb));
             DLZ_TRY(wilson32_batch(op, (float4 *)b, (const float4 *)a, first, nb));
             if (two) DLZ_TRY(wilson32_batch(op, (float4 *)c, (const float4 *)b, DLZ_Q, nb));
             DLZ_TRY(unpack32(op, (float2 *)dst, (const float4 *)(two ? c : b), nb));
         } else if (dtype == DLZ_F64) {
-            if (two) {
-                DLZ_TRY((launch_user<double, true, false>(op, a, src, DLZ_Q, nb)));
-                DLZ_TRY((launch_user<double, false, true>(op, dst, a, DLZ_Q, nb)));
-            } else {
-                DLZ_TRY((launch_user<double, true, true>(op, dst, src, which, nb)));
-            }
-        } else if (direct) {
-            if (two) {
-                DLZ_TRY((launch_user<float, true, false>(op, a, src, DLZ_Q, nb)));
-                DLZ_TRY((launch_user<float, false, true>(op, dst, a, DLZ_Q, nb)));
-            } else {
-                DLZ_TRY((launch_user<float, true, true>(op, dst, src, which, nb)));
-            }
+            if (two) DLZ_TRY((launch_user<double, true, false>(op, a, src, DLZ_Q, nb)));
+            if (two) DLZ_TRY((launch_user<double, false, true>(op, dst, a, DLZ_Q, nb)));
+            else DLZ_TRY((launch_user<double, true, true>(op, dst, src, which, nb)));
         } else {
-            DLZ_TRY(launch_pack_user<float>(op, a, src, nb));
-            if (two) DLZ_TRY(wilson32_batch(op, (float4 *)b, (const float4 *)a, DLZ_Q, nb));
-            DLZ_TRY((launch_user<float, false, true>(op, dst, two ? b : a, first, nb)));
+            if (two) DLZ_TRY((launch_user<float, true, false>(op, a, src, DLZ_Q, nb)));
+            if (two) DLZ_TRY((launch_user<float, false, true>(op, dst, a, DLZ_Q, nb)));
+            else DLZ_TRY((launch_user<float, true, true>(op, dst, src, which, nb)));
         }
     }
     return DLZ_OK;

@@ -1,6 +1,5 @@
-"""dlz_apply over the routes it chooses between, at the sizes where they change: straight
-from the user layout (FP64, and FP32 with few sites) or packed first (many sites), blocks of
-32, 64 and 128 sites with remainders, one and several right-hand sides in a launch, and FP32
+"""dlz_apply over the routes it chooses between, at the sizes where they change: blocks of 32,
+64 and 128 sites with remainders, one and several right-hand sides in a launch, and FP32
 vectors that are only 8-byte aligned, which must give the bits of the aligned call.  FP64
 elements against the FP64 oracle to 1e-14 of the largest element, FP32 to 3e-6 (rounding of
 the input and 24-bit arithmetic over a sum of about 100 terms)."""
@@ -15,7 +14,7 @@ pytestmark = pytest.mark.gpu
 REFS = {"D": wilson.apply_D, "DDAG": wilson.apply_Ddag, "Q": wilson.apply_Q, "DDAGD": wilson.apply_DdagD}
 
 
-# sites x right-hand sides below, at and above 152 * 64 (32-thread blocks) and 40000 (direct FP32)
+# sites x right-hand sides below, at and above 152 * 64 (32-thread blocks)
 @pytest.mark.parametrize("dims,nrhs", [((1, 3, 1, 5), 1), ((3, 5, 7, 9), 1), ((3, 5, 7, 9), 11), ((8, 8, 8, 9), 3),
                                        ((10, 10, 10, 8), 5), ((7, 9, 11, 13), 5), ((12, 10, 14, 6), 4)])
 def test_apply_routes(dims, nrhs):
