@@ -164,21 +164,27 @@ k_ptc_fwd(float4 *__restrict__ out, const float4 *__restrict__ in, const __nv_bf
 
 // Block partials of G(W)[o] = sum_{x, colour} G(out) (T_o in)^dag, as the GEMM
 // (C_out*4) x (3 sites) times (3 sites) x (C_in*4) over tiles of kTS sites.
-// grid (kGradBlocks, 9); partials [o][block][C_out*4][C_in*4]
+// grid (gridDim.x, 9); partials [o][block][C_out*4][C_in*4].
+// FP32-FMA bound.  Thread (tx, ty) of 16 x 16 keeps RI x CJ complex sums, RI = ceil(C_out / 4)
+// and CJ = ceil(C_in / 4): with 4 x 4 sums for every layer the 1 -> 12 and 16 -> 1 layers
+// (16^4, 4 vectors) took the 6.75 ms of the 12 -> 16 layer.
+template <int RI, int CJ>
 __global__ void __launch_bounds__(256)
 k_ptc_wgrad(float2 *__restrict__ partials, const float4 *__restrict__ gout, const float4 *__restrict__ x,
             const float4 *__restrict__ U, Geom g, int cin, int cout, int nvec) {
     extern __shared__ float2 sm[];
     const int rows = cout * 4, cols = cin * 4;
-    float2 *Gs = sm;                   // [rows][kLD]
-    float2 *Ts = sm + rows * kLD;      // [cols][kLD]
+    float2 *Gs = sm;                   // [16 RI][kLD]
+    float2 *Ts = sm + 16 * RI * kLD;   // [16 CJ][kLD]
     const int o = blockIdx.y;
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    float2 acc[4][4];
+    float2 acc[RI][CJ];
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < RI; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.f, 0.f);
+        for (int j = 0; j < CJ; ++j) acc[i][j] = make_float2(0.f, 0.f);
+    // rows beyond the layer's own stay zero
+    for (int t = threadIdx.x; t < 16 * (RI + CJ) * kLD; t += 256) sm[t] = make_float2(0.f, 0.f);
     const size_t plane = (size_t)6 * g.V;
     const int tiles_per_vec = (g.V + kTS - 1) / kTS;
     const long ntiles = (long)tiles_per_vec * nvec;
@@ -188,57 +194,59 @@ k_ptc_wgrad(float2 *__restrict__ partials, const float4 *__restrict__ gout, cons
         const int s = (int)(tile % tiles_per_vec) * kTS + ls;
         const bool ok = s < g.V;
         __syncthreads();
-        for (int cp = slot; cp < cout; cp += 8) {
+        // the channels of both operands shared out over the 8 slots
+        for (int ch = slot; ch < cout + cin; ch += 8) {
+            const bool is_g = ch < cout;
+            const int c = is_g ? ch : ch - cout;
             float2 p[12];
-            if (ok) Field<float>::load(gout + ((size_t)vec * cout + cp) * plane, g.V, s, p);
-            else {
+            if (!ok) {
 #pragma unroll
                 for (int a = 0; a < 12; ++a) p[a] = make_float2(0.f, 0.f);
+            } else if (is_g) {
+                Field<float>::load(gout + ((size_t)vec * cout + c) * plane, g.V, s, p);
+            } else {
+                load_transported(x + ((size_t)vec * cin + c) * plane, U, g, s, o, p);
             }
+            float2 *dst = (is_g ? Gs : Ts) + c * 4 * kLD + ls;
 #pragma unroll
             for (int sp = 0; sp < 4; ++sp)
 #pragma unroll
-                for (int a = 0; a < 3; ++a) Gs[(cp * 4 + sp) * kLD + a * kTS + ls] = p[3 * sp + a];
-        }
-        for (int ci = slot; ci < cin; ci += 8) {
-            float2 t[12];
-            if (ok) load_transported(x + ((size_t)vec * cin + ci) * plane, U, g, s, o, t);
-            else {
-#pragma unroll
-                for (int a = 0; a < 12; ++a) t[a] = make_float2(0.f, 0.f);
-            }
-#pragma unroll
-            for (int sp = 0; sp < 4; ++sp)
-#pragma unroll
-                for (int a = 0; a < 3; ++a) Ts[(ci * 4 + sp) * kLD + a * kTS + ls] = t[3 * sp + a];
+                for (int a = 0; a < 3; ++a) dst[sp * kLD + a * kTS] = p[3 * sp + a];
         }
         __syncthreads();
+#pragma unroll 2
         for (int k = 0; k < 3 * kTS; ++k) {
-            float2 gv[4], tv[4];
+            float2 gv[RI], tv[CJ];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int r = ty + 16 * i;
-                gv[i] = r < rows ? Gs[r * kLD + k] : make_float2(0.f, 0.f);
-            }
+            for (int i = 0; i < RI; ++i) gv[i] = Gs[(ty + 16 * i) * kLD + k];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int c = tx + 16 * j;
-                tv[j] = c < cols ? Ts[c * kLD + k] : make_float2(0.f, 0.f);
-            }
+            for (int j = 0; j < CJ; ++j) tv[j] = Ts[(tx + 16 * j) * kLD + k];
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+            for (int i = 0; i < RI; ++i)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = cfmaConj(tv[j], gv[i], acc[i][j]);
+                for (int j = 0; j < CJ; ++j) acc[i][j] = cfmaConj(tv[j], gv[i], acc[i][j]);
         }
     }
     float2 *pb = partials + ((size_t)o * gridDim.x + blockIdx.x) * rows * cols;
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < RI; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
+        for (int j = 0; j < CJ; ++j) {
             const int r = ty + 16 * i, c = tx + 16 * j;
             if (r < rows && c < cols) pb[(size_t)r * cols + c] = acc[i][j];
         }
+}
+typedef void (*WgradKernel)(float2 *, const float4 *, const float4 *, const float4 *, Geom, int, int, int);
+template <int RI> WgradKernel wgrad_of(int cj) {
+    return cj == 1 ? (WgradKernel)k_ptc_wgrad<RI, 1> : cj == 2 ? (WgradKernel)k_ptc_wgrad<RI, 2>
+         : cj == 3 ? (WgradKernel)k_ptc_wgrad<RI, 3> : (WgradKernel)k_ptc_wgrad<RI, 4>;
+}
+WgradKernel wgrad_kernel(int cin, int cout) {
+    const int ri = (cout + 3) / 4, cj = (cin + 3) / 4;
+    return ri == 1 ? wgrad_of<1>(cj) : ri == 2 ? wgrad_of<2>(cj) : ri == 3 ? wgrad_of<3>(cj) : wgrad_of<4>(cj);
+}
+inline size_t wgrad_smem(int cin, int cout) {
+    return (size_t)16 * ((cout + 3) / 4 + (cin + 3) / 4) * kLD * sizeof(float2);
 }
 
 // grad[o][c'][c][4 s' + s] += sum over blocks (fixed order) of the partials
@@ -365,7 +373,9 @@ int set_attrs() {
     static bool done = false;
     if (done) return DLZ_OK;
     const int wg = (int)((size_t)(2 * kMaxWidth * 4) * kLD * sizeof(float2));
-    DLZ_CUDA_TRY(cudaFuncSetAttribute(k_ptc_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, wg));
+    for (int co = 4; co <= kMaxWidth; co += 4)
+        for (int ci = 4; ci <= kMaxWidth; ci += 4)
+            DLZ_CUDA_TRY(cudaFuncSetAttribute(wgrad_kernel(ci, co), cudaFuncAttributeMaxDynamicSharedMemorySize, wg));
     const int fw = 9 * 4 * kMaxWidth * 16 * (int)sizeof(__nv_bfloat162);
     DLZ_CUDA_TRY(cudaFuncSetAttribute(k_ptc_fwd<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, fw));
     DLZ_CUDA_TRY(cudaFuncSetAttribute(k_ptc_fwd<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, fw));
@@ -489,10 +499,8 @@ int dlz_net_backward(dlz_net_t net, const void *grad_out, int nvec, void *grad_i
     for (int v = 0; v < nvec; ++v) DLZ_TRY(pack32(op, gc + (size_t)v * plane, (const float2 *)grad_out + (size_t)v * n));
     for (int l = net->nl - 1; l >= 0; --l) {
         const int cin = net->w[l], cout = net->w[l + 1];
-        const size_t sm = (size_t)(cout * 4 + cin * 4) * kLD * sizeof(float2);
-        k_ptc_wgrad<<<dim3(kGradBlocks, 9), 256, sm, op.stream>>>(net->partials.as<float2>(), gc,
-                                                                 net->act[l].as<float4>(), op.gauge32.as<float4>(),
-                                                                 op.g, cin, cout, nvec);
+        wgrad_kernel(cin, cout)<<<dim3(kGradBlocks, 9), 256, wgrad_smem(cin, cout), op.stream>>>(
+            net->partials.as<float2>(), gc, net->act[l].as<float4>(), op.gauge32.as<float4>(), op.g, cin, cout, nvec);
         const long ne = 9L * cin * cout * 16;
         k_ptc_wgrad_sum<<<blocks_for(ne, 256), 256, 0, op.stream>>>(net->grad.as<float2>() + net->off[l],
                                                                     net->partials.as<float2>(), kGradBlocks, cin, cout);
