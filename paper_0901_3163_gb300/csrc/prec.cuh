@@ -187,16 +187,16 @@ k_multidot32(const float4 *__restrict__ V, long ld, int nv, const float4 *__rest
     }
     __shared__ double sm[16][kMdThreads / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    double d[16];
 #pragma unroll
     for (int l = 0; l < 8; ++l) {
-        double a = (double)re[l], b = (double)im[l];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            a += __shfl_down_sync(0xffffffffu, a, o);
-            b += __shfl_down_sync(0xffffffffu, b, o);
-        }
-        if (lane == 0) { sm[2 * l][warp] = a; sm[2 * l + 1][warp] = b; }
+        d[2 * l] = (double)re[l];
+        d[2 * l + 1] = (double)im[l];
     }
+    const double t = warp_sums<16>(d);
+#pragma unroll
+    for (int j = 0; j < 16; ++j)
+        if (lane == warp_sum_lane<16>(j)) sm[j][warp] = t;
     __syncthreads();
     if (threadIdx.x < 16) {
         double t = 0.0;

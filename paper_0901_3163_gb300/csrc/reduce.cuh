@@ -15,16 +15,47 @@
 
 namespace dlz {
 
+// Sums of ND per-lane values over the 32 lanes of a warp, value j in v[0] of lane
+// warp_sum_lane<ND>(j).  Halving: at each step a lane hands half of the values it still holds
+// to its partner and adds the partner's to the other half, so ND = 16 values take 16 FP64
+// additions per lane (8 + 4 + 2 + 1 + 1) where a shuffle tree per value takes 80; at 2 FP64
+// additions per cycle and SM the trees were most of a reduction with 16 values (the FP32
+// multi-dot of 40 vectors of 16^3 x 32: see k_multidot32).
+template <int ND> __host__ __device__ constexpr int warp_sum_lane(int j) {
+    // the lane bits 4, 3, ... select the upper half at each halving step
+    int lane = 0, half = (ND <= 1 ? 1 : ND <= 2 ? 2 : ND <= 4 ? 4 : ND <= 8 ? 8 : ND <= 16 ? 16 : 32) / 2, bit = 16;
+    for (; half >= 1; half /= 2, bit /= 2)
+        if (j & half) lane |= bit;
+    return lane;
+}
+template <int ND> __device__ inline double warp_sums(const double (&in)[ND]) {
+    constexpr int P = ND <= 1 ? 1 : ND <= 2 ? 2 : ND <= 4 ? 4 : ND <= 8 ? 8 : ND <= 16 ? 16 : 32;
+    double v[P];
+#pragma unroll
+    for (int j = 0; j < P; ++j) v[j] = j < ND ? in[j] : 0.0;
+    int bit = 16;
+#pragma unroll
+    for (int half = P / 2; half >= 1; half /= 2) {
+        const bool up = threadIdx.x & bit;
+#pragma unroll
+        for (int j = 0; j < half; ++j) {
+            const double give = up ? v[j] : v[j + half], keep = up ? v[j + half] : v[j];
+            v[j] = keep + __shfl_xor_sync(0xffffffffu, give, bit);
+        }
+        bit /= 2;
+    }
+#pragma unroll
+    for (; bit >= 1; bit /= 2) v[0] += __shfl_xor_sync(0xffffffffu, v[0], bit);
+    return v[0];
+}
+
 template <int ND>
 __device__ inline void block_sum(double (&acc)[ND], double (*sm)[kRedThreads / 32]) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const double t = warp_sums<ND>(acc);
 #pragma unroll
-    for (int j = 0; j < ND; ++j) {
-        double v = acc[j];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if (lane == 0) sm[j][warp] = v;
-    }
+    for (int j = 0; j < ND; ++j)
+        if (lane == warp_sum_lane<ND>(j)) sm[j][warp] = t;
     __syncthreads();
     if (threadIdx.x < ND) {
         double v = 0.0;
