@@ -638,7 +638,9 @@ int dminres_multi(int nlat, Op *const *ops, const dlz_defl_s *const *defls, cons
             Lat &a = L[l];
             const int N = nrhs[l];
             const long n64 = 12L * o.g.V;
-            DLZ_TRY(wilson64_batch(o, a.t, a.x.as<double2>(), DLZ_Q, N));
+            // (from the start x = 0 the residual is b' itself: Q x = 0 without the FP64 stencil)
+            if (outer > 0) DLZ_TRY(wilson64_batch(o, a.t, a.x.as<double2>(), DLZ_Q, N));
+            else DLZ_CUDA_TRY(cudaMemsetAsync(a.t, 0, (size_t)N * n64 * sizeof(double2), o.stream));
             const double2 *pbp = a.bp.as<double2>(), *pt = a.t;
             double2 *pr = a.r;
             double *dn = a.nrm.as<double>();

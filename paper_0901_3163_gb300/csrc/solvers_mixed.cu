@@ -98,7 +98,9 @@ int dsolve_mixed_batch(Op &op, const dlz_defl_s *d, bool minres, const double2 *
     int iters = 0, outer = 0;
     long long mv_batch = 0;
     auto residuals = [&]() -> int {
-        DLZ_TRY(wilson64_batch(op, pt, px, which, N));
+        // (from the start x = 0 the residual is b' itself: A x = 0 without the FP64 stencil)
+        if (outer > 0 || X_init) DLZ_TRY(wilson64_batch(op, pt, px, which, N));
+        else DLZ_CUDA_TRY(cudaMemsetAsync(pt, 0, (size_t)N * n64 * sizeof(double2), op.stream));
         mv_batch += 1;
         DLZ_TRY(reduce<kMaxBatch>(op, n64, [=] __device__(long i, double (&acc)[kMaxBatch]) {
 #pragma unroll
