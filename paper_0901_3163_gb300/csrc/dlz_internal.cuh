@@ -335,6 +335,8 @@ int run_graph(Op &op, GraphExec &ge, F &&body) {
 // Wilson stencil: out = [g5_out] (1 - kappa H) [g5_in] in, FP64 or FP32.
 // which: DLZ_D (0,0), DLZ_DDAG (1,1), DLZ_Q (0,1).
 int wilson64(Op &op, double2 *out, const double2 *in, int which);
+// threads of a plain-order block that spread V x nrhs sites evenly over the SMs
+int balanced_threads(int V, int nrhs);
 int wilson32(Op &op, float4 *out, const float4 *in, int which);
 // nrhs spinors stored one after another (FP32: 6V float4 each, FP64: 12V double2 each)
 int wilson32_batch(Op &op, float4 *out, const float4 *in, int which, int nrhs);

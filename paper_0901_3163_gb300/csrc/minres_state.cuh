@@ -238,8 +238,8 @@ __device__ inline void block_partial_store(float facc, double *__restrict__ out)
 // partials of q in a fixed order and resets the counter (so the sum is deterministic
 // and needs no second launch).  Returns true, with the sum in *total (thread 0), in
 // that block only.  BT: threads per block.
-template <int BT>
-__device__ inline bool partial_then_last_sum(float facc, double *__restrict__ slot0, int b, int nbq,
+template <int BT, typename A>
+__device__ inline bool partial_then_last_sum(A facc, double *__restrict__ slot0, int b, int nbq,
                                              unsigned *__restrict__ counter, double *total) {
     __shared__ double sm[BT / 32];
     __shared__ bool last;
@@ -260,6 +260,7 @@ __device__ inline bool partial_then_last_sum(float facc, double *__restrict__ sl
     if (!last) return false;
     __threadfence();
     double t = 0.0;
+#pragma unroll 8
     for (int i = threadIdx.x; i < nbq; i += BT) t += __ldcg(&slot0[i]);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);

@@ -19,6 +19,8 @@
 #include "small_dense.h"
 #include "solvers.h"
 #include "krylov_util.cuh"
+#include "minres_state.cuh"
+#include "wilson_site.cuh"
 
 namespace dlz {
 
@@ -67,23 +69,25 @@ int deflation_finish(Op &op, dlz_defl_s *d) {
     for (int j = 0; j < k; ++j) {
         double2 *avj = AV.as<double2>();
         DLZ_TRY(apply64(op, avj, V + (size_t)j * n, d->which, tmp.as<double2>()));
-        DLZ_TRY(v64::multidot(op, V, n, k, avj, dots.as<double2>() + (size_t)j * k, 1.0));
-        DLZ_TRY(v64::multidot(op, V, n, k, V + (size_t)j * n, gram.as<double2>() + (size_t)j * k, 1.0));
+        DLZ_TRY(v64::multidot(op, V, n, j + 1, avj, dots.as<double2>() + (size_t)j * k, 1.0));
+        DLZ_TRY(v64::multidot(op, V, n, j + 1, V + (size_t)j * n, gram.as<double2>() + (size_t)j * k, 1.0));
     }
+    // (the other triangles of dots and gram are not written)
     std::vector<double2> hd((size_t)k * k), gd((size_t)k * k);
     DLZ_TRY(d2h_sync(op, hd.data(), dots.p, hd.size() * sizeof(double2)));
     DLZ_TRY(d2h_sync(op, gd.data(), gram.p, gd.size() * sizeof(double2)));
-    // dots[j*k + i] = <v_i, A v_j> = H[i][j]; hermitise (the same for the Gram matrix)
+    // dots[j*k + i] = <v_i, A v_j> = H[i][j] for i <= j (the dots are FP64-ALU-bound, so the
+    // other triangle is the conjugate, not a second computation); the same for the Gram matrix
     d->H.assign((size_t)k * k, zc(0, 0));
     d->G.assign((size_t)k * k, zc(0, 0));
-    for (int i = 0; i < k; ++i)
-        for (int j = 0; j < k; ++j) {
-            const zc hij(hd[(size_t)j * k + i].x, hd[(size_t)j * k + i].y);
-            const zc hji(hd[(size_t)i * k + j].x, hd[(size_t)i * k + j].y);
-            d->H[(size_t)i * k + j] = 0.5 * (hij + std::conj(hji));
-            const zc gij(gd[(size_t)j * k + i].x, gd[(size_t)j * k + i].y);
-            const zc gji(gd[(size_t)i * k + j].x, gd[(size_t)i * k + j].y);
-            d->G[(size_t)i * k + j] = 0.5 * (gij + std::conj(gji));
+    for (int j = 0; j < k; ++j)
+        for (int i = 0; i <= j; ++i) {
+            const zc h(hd[(size_t)j * k + i].x, i == j ? 0.0 : hd[(size_t)j * k + i].y);
+            const zc g(gd[(size_t)j * k + i].x, i == j ? 0.0 : gd[(size_t)j * k + i].y);
+            d->H[(size_t)i * k + j] = h;
+            d->H[(size_t)j * k + i] = std::conj(h);
+            d->G[(size_t)i * k + j] = g;
+            d->G[(size_t)j * k + i] = std::conj(g);
         }
     return deflation_factor(op, d);
 }
@@ -266,19 +270,109 @@ int project64(Op &op, const dlz_defl_s *d, const double2 *b, double2 *x0, DevBuf
 
 // ------------------------------------------------------------------ D-MinRes (FP64)
 struct MinresState {
-    double beta, alpha, beta_next, inv_beta;
+    double beta, alpha, beta_next, inv_beta, inv_beta_prev;
     double c, s, c_old, s_old, phibar;
     double eps, delta, gamma, tau;
+    double a_u;                  // alpha_j / beta_j
+    double d_u, d_1, d_2;        // 1 / (beta gamma), delta / gamma, eps / gamma of the last rotation
 };
 
+// The fused FP64 MinRes step.  u_j is the unnormalised Lanczos vector, v_j = u_j / beta_j:
+//   K1: w = Q u_j / beta_j - beta_j v_{j-1}, alpha_j = <v_j, w>;
+//   K2: u_{j+1} = w - alpha_j v_j, beta_{j+1} = ||u_{j+1}|| and the Givens rotation of step j,
+//       and the direction update of step j - 1, d = (v_{j-1} - delta d_{j-2} - eps d_{j-3}) /
+//       gamma, x += tau d, whose rotation the step before made.
+// The last block of each kernel to finish adds the block partials in a fixed order and writes
+// the scalars.  Both are bound by FP64 arithmetic (about 900 and 170 instructions per site at 2
+// per cycle and SM).  On 12 x 12 x 10 x 22 an iteration of the separate stencil, two reductions
+// and update took 64.7 + 2 x 11.6 + 12.6 us and four launch gaps; the fused one: see dminres64.
+template <int BT>
+__global__ void __launch_bounds__(BT)
+k_minres64_k1(const double2 *__restrict__ Uc, const double2 *__restrict__ Up, double2 *__restrict__ W,
+              const double2 *__restrict__ links, Geom g, double kappa, MinresState *st, double *__restrict__ partials,
+              unsigned *__restrict__ counter) {
+    const int s = blockIdx.x * BT + threadIdx.x;
+    double acc = 0.0;
+    if (s < g.V) {
+        const double ib = st->inv_beta, bp = st->beta_next * st->inv_beta_prev;
+        double2 o[12];
+        wilson_site<double, false, true>(s, g, kappa, Uc, links, o);
+#pragma unroll
+        for (int c = 0; c < 12; ++c) {
+            const size_t i = (size_t)c * g.V + s;
+            const double2 u = Uc[i], up = Up[i];
+            const double2 w = make_double2(fma(-bp, up.x, o[c].x * ib), fma(-bp, up.y, o[c].y * ib));
+            W[i] = w;
+            acc = fma(u.x, w.x, acc);
+            acc = fma(u.y, w.y, acc);
+        }
+    }
+    double a;
+    if (partial_then_last_sum<BT>(acc, partials, blockIdx.x, gridDim.x, counter, &a) && threadIdx.x == 0) {
+        st->beta = st->beta_next;
+        st->alpha = a * st->inv_beta;
+        st->a_u = st->alpha * st->inv_beta;
+    }
+}
+
+constexpr int kK2Elems = 4;      // elements per thread (the block sum's additions are FP64 too)
+
+__global__ void __launch_bounds__(256)
+k_minres64_k2(double2 *__restrict__ W, const double2 *__restrict__ Uc, const double2 *__restrict__ Up,
+              const double2 *__restrict__ D1, double2 *__restrict__ D2, double2 *__restrict__ X, long n,
+              MinresState *st, double *__restrict__ partials, unsigned *__restrict__ counter) {
+    const double al = st->a_u, cu = st->d_u, c1 = st->d_1, c2 = st->d_2, ta = st->tau;
+    double acc = 0.0;
+#pragma unroll
+    for (int e = 0; e < kK2Elems; ++e) {
+        const long i = ((long)blockIdx.x * kK2Elems + e) * 256 + threadIdx.x;
+        if (i >= n) break;
+        const double2 w = W[i], u = Uc[i], up = Up[i], d1 = D1[i], d2 = D2[i];
+        double2 x = X[i];
+        const double2 t = make_double2(fma(-al, u.x, w.x), fma(-al, u.y, w.y));
+        W[i] = t;
+        acc = fma(t.x, t.x, fma(t.y, t.y, acc));
+        const double2 d = make_double2(fma(cu, up.x, fma(-c1, d1.x, -c2 * d2.x)), fma(cu, up.y, fma(-c1, d1.y, -c2 * d2.y)));
+        D2[i] = d;
+        x.x = fma(ta, d.x, x.x);
+        x.y = fma(ta, d.y, x.y);
+        X[i] = x;
+    }
+    double r2;
+    if (partial_then_last_sum<256>(acc, partials, blockIdx.x, gridDim.x, counter, &r2) && threadIdx.x == 0) {
+        MinresState s = *st;
+        const double bn = sqrt(r2);
+        const double eps = s.s_old * s.beta;
+        const double deltabar = s.c_old * s.beta;
+        const double delta = s.c * deltabar + s.s * s.alpha;
+        const double gammabar = -s.s * deltabar + s.c * s.alpha;
+        const double gamma = hypot(gammabar, bn);
+        const double cn = gammabar / gamma, sn = bn / gamma;
+        s.tau = cn * s.phibar;
+        s.phibar = -sn * s.phibar;
+        s.eps = eps; s.delta = delta; s.gamma = gamma;
+        s.c_old = s.c; s.s_old = s.s; s.c = cn; s.s = sn;
+        s.d_u = s.inv_beta / gamma;
+        s.d_1 = delta / gamma;
+        s.d_2 = eps / gamma;
+        s.inv_beta_prev = s.inv_beta;
+        s.beta_next = bn;
+        s.inv_beta = bn > 0 ? 1.0 / bn : 0.0;
+        *st = s;
+    }
+}
+
 static int minres_init(Op &op, MinresState *dst, double *d_norm) {
-    // beta = phibar = ||r||, fresh rotations
+    // beta = phibar = ||r||, fresh rotations, a no-op direction update for the step before
     return map(op, 1, [=] __device__(long) {
         const double b = sqrt(*d_norm);
         MinresState s0;
         s0.beta = 0.0; s0.alpha = 0.0; s0.beta_next = b; s0.inv_beta = b > 0 ? 1.0 / b : 0.0;
+        s0.inv_beta_prev = 0.0;
         s0.c = 1.0; s0.s = 0.0; s0.c_old = 1.0; s0.s_old = 0.0; s0.phibar = b;
-        s0.eps = s0.delta = s0.gamma = s0.tau = 0.0;
+        s0.eps = s0.delta = s0.tau = 0.0;
+        s0.gamma = 1.0;
+        s0.a_u = s0.d_u = s0.d_1 = s0.d_2 = 0.0;
         *dst = s0;
     });
 }
@@ -297,6 +391,13 @@ int dminres64(Op &op, const dlz_defl_s *d, const double2 *b_in, double2 *x_out, 
     DLZ_TRY(d2.alloc(n * sizeof(double2)));
     DLZ_TRY(scal.alloc(64 * sizeof(double)));
     DLZ_TRY(dots.alloc((size_t)std::max(1, d ? d->k : 1) * sizeof(double2)));
+    // block partials of the fused kernels and their block counter (reset by the last block)
+    const int bt = balanced_threads(op.g.V, 1);
+    const size_t nblk = std::max<size_t>((op.g.V + bt - 1) / bt, (n + 255) / 256);
+    DevBuf part;
+    DLZ_TRY(part.alloc((nblk + 1) * sizeof(double)));
+    unsigned *cnt = reinterpret_cast<unsigned *>(part.as<double>() + nblk);
+    DLZ_CUDA_TRY(cudaMemsetAsync(cnt, 0, sizeof(unsigned), op.stream));
     MinresState *ms = reinterpret_cast<MinresState *>(scal.as<double>());
     double *d_norm = scal.as<double>() + 32;
     HostScratch hs;
@@ -359,87 +460,44 @@ int dminres64(Op &op, const dlz_defl_s *d, const double2 *b_in, double2 *x_out, 
         DLZ_TRY(minres_init(op, ms, d_norm));
         double2 *pvp = vp.as<double2>(), *pv = v.as<double2>(), *pw = w.as<double2>();
         double2 *pd1 = d1.as<double2>(), *pd2 = d2.as<double2>();
-        {
-            const double2 *rp = r.as<double2>();
-            DLZ_TRY(map(op, n, [=] __device__(long i) {
-                const double inv = ms->inv_beta;
-                const double2 t = rp[i];
-                pv[i] = make_double2(t.x * inv, t.y * inv);
-                pvp[i] = make_double2(0.0, 0.0);
-                pd1[i] = make_double2(0.0, 0.0);
-                pd2[i] = make_double2(0.0, 0.0);
-            }));
-        }
+        DLZ_TRY(v64::copy(op, pv, r.as<double2>()));          // u_1 = r
+        for (double2 *z : {pvp, pd1, pd2}) DLZ_TRY(v64::zero(op, z));
         double2 *px = x.as<double2>();
         int it_run = 0;
         bool stop_run = false;
         while (!stop_run && st.iterations < p.max_iter) {
-            DLZ_TRY(wilson64(op, pw, pv, DLZ_Q));
-            st.mvps += 1;
-            // w -= beta_j v_{j-1}; alpha_j = <v_j, w>
-            {
-                const double2 *a_vp = pvp, *a_v = pv;
+            if (op.eo) {
+                // (an even-odd operator's stencil is two launches: w = Q u_j, then K1's update)
+                DLZ_TRY(wilson64(op, pw, pv, DLZ_Q));
+                const double2 *a_u = pv, *a_up = pvp;
                 double2 *a_w = pw;
                 DLZ_TRY(reduce<1>(op, n, [=] __device__(long i, double (&acc)[1]) {
-                    const double bt = ms->beta_next;
-                    double2 t = a_w[i];
-                    const double2 u = a_vp[i];
-                    t.x -= bt * u.x; t.y -= bt * u.y;
+                    const double ib = ms->inv_beta, bp = ms->beta_next * ms->inv_beta_prev;
+                    const double2 o = a_w[i], up = a_up[i], u = a_u[i];
+                    const double2 t = make_double2(fma(-bp, up.x, o.x * ib), fma(-bp, up.y, o.y * ib));
                     a_w[i] = t;
-                    const double2 q = a_v[i];
-                    acc[0] += q.x * t.x + q.y * t.y;
+                    acc[0] += u.x * t.x + u.y * t.y;
                 }, [=] __device__(const double *res) {
                     ms->beta = ms->beta_next;
-                    ms->alpha = res[0];
+                    ms->alpha = res[0] * ms->inv_beta;
+                    ms->a_u = ms->alpha * ms->inv_beta;
                 }));
+            } else {
+                const Geom g = op.g;
+                const double2 *U = op.gauge64.as<double2>();
+                const unsigned blocks = (unsigned)((g.V + bt - 1) / bt);
+                op.prof.stencil_start(op.stream, false, g.V, 1, 72, 1);
+                if (bt == 32) k_minres64_k1<32><<<blocks, 32, 0, op.stream>>>(pv, pvp, pw, U, g, op.kappa, ms, part.as<double>(), cnt);
+                else if (bt == 64) k_minres64_k1<64><<<blocks, 64, 0, op.stream>>>(pv, pvp, pw, U, g, op.kappa, ms, part.as<double>(), cnt);
+                else k_minres64_k1<128><<<blocks, 128, 0, op.stream>>>(pv, pvp, pw, U, g, op.kappa, ms, part.as<double>(), cnt);
+                op.prof.stencil_stop(op.stream);
+                op.prof.launches++;
             }
-            // w -= alpha_j v_j; beta_{j+1} = ||w||; Givens update of the QR of Tbar_j
-            {
-                const double2 *a_v = pv;
-                double2 *a_w = pw;
-                DLZ_TRY(reduce<1>(op, n, [=] __device__(long i, double (&acc)[1]) {
-                    const double al = ms->alpha;
-                    double2 t = a_w[i];
-                    const double2 q = a_v[i];
-                    t.x -= al * q.x; t.y -= al * q.y;
-                    a_w[i] = t;
-                    acc[0] += t.x * t.x + t.y * t.y;
-                }, [=] __device__(const double *res) {
-                    MinresState s = *ms;
-                    const double bn = sqrt(res[0]);
-                    const double eps = s.s_old * s.beta;
-                    const double deltabar = s.c_old * s.beta;
-                    const double delta = s.c * deltabar + s.s * s.alpha;
-                    const double gammabar = -s.s * deltabar + s.c * s.alpha;
-                    const double gamma = hypot(gammabar, bn);
-                    const double cn = gammabar / gamma, sn = bn / gamma;
-                    s.tau = cn * s.phibar;
-                    s.phibar = -sn * s.phibar;
-                    s.eps = eps; s.delta = delta; s.gamma = gamma;
-                    s.c_old = s.c; s.s_old = s.s; s.c = cn; s.s = sn;
-                    s.beta_next = bn;
-                    s.inv_beta = bn > 0 ? 1.0 / bn : 0.0;
-                    *ms = s;
-                }));
-            }
-            // d_j = (v_j - delta d_{j-1} - eps d_{j-2}) / gamma ; x += tau d_j ; v_{j+1} = w / beta_{j+1}
-            {
-                const double2 *a_v = pv, *a_d1 = pd1;
-                double2 *a_d2 = pd2, *a_w = pw, *a_x = px;
-                DLZ_TRY(map(op, n, [=] __device__(long i) {
-                    const double de = ms->delta, ep = ms->eps, ig = 1.0 / ms->gamma, ta = ms->tau, ib = ms->inv_beta;
-                    const double2 q = a_v[i], e1 = a_d1[i], e2 = a_d2[i];
-                    double2 dn;
-                    dn.x = (q.x - de * e1.x - ep * e2.x) * ig;
-                    dn.y = (q.y - de * e1.y - ep * e2.y) * ig;
-                    a_d2[i] = dn;
-                    double2 xx = a_x[i];
-                    xx.x += ta * dn.x; xx.y += ta * dn.y;
-                    a_x[i] = xx;
-                    const double2 t = a_w[i];
-                    a_w[i] = make_double2(t.x * ib, t.y * ib);
-                }));
-            }
+            st.mvps += 1;
+            k_minres64_k2<<<(unsigned)((n + 256 * kK2Elems - 1) / (256 * kK2Elems)), 256, 0, op.stream>>>(pw, pv, pvp, pd1, pd2, px, n, ms,
+                                                                            part.as<double>(), cnt);
+            op.prof.launches++;
+            DLZ_CUDA_TRY(cudaGetLastError());
             // rotate: (v_prev, v, w) <- (v, w, v_prev) ; (d1, d2) <- (d2, d1)
             double2 *t0 = pvp; pvp = pv; pv = pw; pw = t0;
             std::swap(pd1, pd2);
@@ -451,6 +509,19 @@ int dminres64(Op &op, const dlz_defl_s *d, const double2 *b_in, double2 *x_out, 
                 if (!std::isfinite(hsm->phibar)) return fail(DLZ_ERR_NONFINITE, "MinRes residual not finite");
                 if (std::fabs(hsm->phibar) <= 0.5 * p.tol * bnorm || hsm->beta_next == 0.0) stop_run = true;
             }
+        }
+        // the direction update of the last step, which the next K2 would have made
+        {
+            const double2 *a_up = pvp, *a_d1 = pd1, *a_d2 = pd2;
+            double2 *a_x = px;
+            DLZ_TRY(map(op, n, [=] __device__(long i) {
+                const double cu = ms->d_u, c1 = ms->d_1, c2 = ms->d_2, ta = ms->tau;
+                const double2 up = a_up[i], e1 = a_d1[i], e2 = a_d2[i];
+                double2 xx = a_x[i];
+                xx.x = fma(ta, fma(cu, up.x, fma(-c1, e1.x, -c2 * e2.x)), xx.x);
+                xx.y = fma(ta, fma(cu, up.y, fma(-c1, e1.y, -c2 * e2.y)), xx.y);
+                a_x[i] = xx;
+            }));
         }
     }
     DLZ_TRY(v64::copy(op, x_out, x.as<double2>()));

@@ -210,6 +210,8 @@ k_wilson_user(typename Field<T>::vec *__restrict__ out, const typename Field<T>:
     }
 }
 
+}  // namespace
+
 // Threads of a plain-order block (32, 64 or 128) for `total` sites of FP64-ALU-bound work:
 // the SM with the most sites ends last, so the size that gives the fullest SMs fewest sites
 // (31680 sites on 152 SMs: 256 with 128 threads, 224 with 32).
@@ -225,6 +227,8 @@ int balanced_threads(int V, int nrhs) {
     }
     return best;
 }
+
+namespace {
 
 template <typename T, bool UIN, bool UOUT, int BT>
 void launch_user_bt(Op &op, typename Field<T>::vec *out, const typename Field<T>::vec *in,
