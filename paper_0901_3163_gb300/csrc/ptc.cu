@@ -27,6 +27,7 @@
 #include <vector>
 
 #include "dlz_internal.cuh"
+#include "ptc_tc.cuh"
 #include "krylov_util.cuh"
 #include "reduce.cuh"
 #include "solvers.h"
@@ -326,6 +327,8 @@ struct dlz_net_s {
     std::vector<size_t> off;            // first complex weight of each layer
     size_t nw = 0;
     dlz::DevBuf master, grad, m1, m2, wb, wadj, partials;
+    dlz::DevBuf img, err;               // weight images of the tensor-core layers; a wait that gave up
+    std::vector<size_t> img_fwd, img_adj;   // their offsets (bf16 elements)
     int adam_t = 0;
     dlz::DevBuf act[dlz::kMaxLayersNet + 1];   // input of every layer from the last forward
     int act_nvec = 0;
@@ -335,7 +338,9 @@ struct dlz_net_s {
 namespace dlz {
 namespace {
 
-int layer_forward(Op &op, float4 *out, const float4 *in, const __nv_bfloat162 *W, int cin, int cout, int nvec) {
+int layer_forward(Op &op, float4 *out, const float4 *in, const __nv_bfloat162 *W, const __nv_bfloat16 *img, int *err,
+                  int cin, int cout, int nvec) {
+    if (ptc_tc_layer(cin, cout)) return ptc_tc_forward(op, out, in, img, cin, cout, nvec, err);
     const Geom g = op.g;
     const float4 *U = op.gauge32.as<float4>();
     const unsigned gx = blocks_for(g.V, kFwdThreads);
@@ -363,15 +368,31 @@ int refresh_bf16(dlz_net_s *net) {
         k_ptc_adjoint<<<blocks_for(n, 256), 256, 0, op.stream>>>(net->wadj.as<__nv_bfloat162>() + net->off[l],
                                                                 net->wb.as<__nv_bfloat162>() + net->off[l],
                                                                 net->w[l], net->w[l + 1]);
+        const int cin = net->w[l], cout = net->w[l + 1];
+        __nv_bfloat16 *img = net->img.as<__nv_bfloat16>();
+        if (ptc_tc_layer(cin, cout))
+            DLZ_TRY(ptc_tc_image(op, img + net->img_fwd[l], net->wb.as<__nv_bfloat162>() + net->off[l], cin, cout));
+        if (ptc_tc_layer(cout, cin))
+            DLZ_TRY(ptc_tc_image(op, img + net->img_adj[l], net->wadj.as<__nv_bfloat162>() + net->off[l], cout, cin));
     }
     op.prof.launches += 1 + net->nl;
     DLZ_CUDA_TRY(cudaGetLastError());
     return DLZ_OK;
 }
 
+// after the stream has finished: whether a wait of a tensor-core layer gave up
+int check_layers(dlz_net_s *net) {
+    int h = 0;
+    DLZ_TRY(d2h_sync(*net->op, &h, net->err.p, sizeof(int)));
+    if (!h) return DLZ_OK;
+    DLZ_CUDA_TRY(cudaMemsetAsync(net->err.p, 0, sizeof(int), net->op->stream));
+    return fail(DLZ_ERR_DEVICE_TIMEOUT, "a wait of a tensor-core network layer gave up");
+}
+
 int set_attrs() {
     static bool done = false;
     if (done) return DLZ_OK;
+    DLZ_TRY(ptc_tc_prepare());
     const int wg = (int)((size_t)(2 * kMaxWidth * 4) * kLD * sizeof(float2));
     for (int co = 4; co <= kMaxWidth; co += 4)
         for (int ci = 4; ci <= kMaxWidth; ci += 4)
@@ -427,6 +448,16 @@ int dlz_net_create(dlz_op_t h, int nlayers, const int *widths, const void *weigh
         DLZ_TRY(net->m2.alloc(o * sizeof(float2)));
         DLZ_TRY(net->wb.alloc(o * sizeof(__nv_bfloat162)));
         DLZ_TRY(net->wadj.alloc(o * sizeof(__nv_bfloat162)));
+        size_t ni = 0;
+        for (int l = 0; l < nlayers; ++l) {
+            net->img_fwd.push_back(ni);
+            ni += ptc_tc_image_size(widths[l], widths[l + 1]);
+            net->img_adj.push_back(ni);
+            ni += ptc_tc_image_size(widths[l + 1], widths[l]);
+        }
+        DLZ_TRY(net->img.alloc(ni * sizeof(__nv_bfloat16)));
+        DLZ_TRY(net->err.alloc(sizeof(int)));
+        DLZ_CUDA_TRY(cudaMemsetAsync(net->err.p, 0, sizeof(int), op.stream));
         int maxp = 0;
         for (int l = 0; l < nlayers; ++l) maxp = std::max(maxp, 16 * widths[l] * widths[l + 1]);
         DLZ_TRY(net->partials.alloc((size_t)9 * kGradBlocks * maxp * sizeof(float2)));
@@ -469,16 +500,14 @@ int dlz_net_forward(dlz_net_t net, const void *in, int nvec, void *out) {
             DLZ_TRY(net->act[l].alloc((size_t)nvec * net->w[l] * plane * sizeof(float4)));
         net->act_nvec = nvec;
     }
-    const long n = 12L * op.g.V;
-    for (int v = 0; v < nvec; ++v)
-        DLZ_TRY(pack32(op, net->act[0].as<float4>() + (size_t)v * plane, (const float2 *)in + (size_t)v * n));
+    DLZ_TRY(pack32(op, net->act[0].as<float4>(), (const float2 *)in, nvec));
     for (int l = 0; l < net->nl; ++l)
         DLZ_TRY(layer_forward(op, net->act[l + 1].as<float4>(), net->act[l].as<float4>(),
-                              net->wb.as<__nv_bfloat162>() + net->off[l], net->w[l], net->w[l + 1], nvec));
-    for (int v = 0; v < nvec; ++v)
-        DLZ_TRY(unpack32(op, (float2 *)out + (size_t)v * n, net->act[net->nl].as<float4>() + (size_t)v * plane));
-    DLZ_CUDA_TRY(cudaStreamSynchronize(op.stream));
-    return DLZ_OK;
+                              net->wb.as<__nv_bfloat162>() + net->off[l],
+                              net->img.as<__nv_bfloat16>() + net->img_fwd[l], net->err.as<int>(), net->w[l],
+                              net->w[l + 1], nvec));
+    DLZ_TRY(unpack32(op, (float2 *)out, net->act[net->nl].as<float4>(), nvec));
+    return check_layers(net);
 }
 
 int dlz_net_backward(dlz_net_t net, const void *grad_out, int nvec, void *grad_in) {
@@ -489,14 +518,13 @@ int dlz_net_backward(dlz_net_t net, const void *grad_out, int nvec, void *grad_i
     Op &op = *net->op;
     op.prof.begin(false, false);
     const size_t plane = (size_t)6 * op.g.V;
-    const long n = 12L * op.g.V;
     int maxw = 1;
     for (int l = 0; l <= net->nl; ++l) maxw = std::max(maxw, net->w[l]);
     for (int b = 0; b < 2; ++b)
         if (net->gbuf[b].bytes < (size_t)nvec * maxw * plane * sizeof(float4))
             DLZ_TRY(net->gbuf[b].alloc((size_t)nvec * maxw * plane * sizeof(float4)));
     float4 *gc = net->gbuf[0].as<float4>(), *gn = net->gbuf[1].as<float4>();
-    for (int v = 0; v < nvec; ++v) DLZ_TRY(pack32(op, gc + (size_t)v * plane, (const float2 *)grad_out + (size_t)v * n));
+    DLZ_TRY(pack32(op, gc, (const float2 *)grad_out, nvec));
     for (int l = net->nl - 1; l >= 0; --l) {
         const int cin = net->w[l], cout = net->w[l + 1];
         wgrad_kernel(cin, cout)<<<dim3(kGradBlocks, 9), 256, wgrad_smem(cin, cout), op.stream>>>(
@@ -507,14 +535,13 @@ int dlz_net_backward(dlz_net_t net, const void *grad_out, int nvec, void *grad_i
         op.prof.launches += 2;
         DLZ_CUDA_TRY(cudaGetLastError());
         if (l > 0 || grad_in) {
-            DLZ_TRY(layer_forward(op, gn, gc, net->wadj.as<__nv_bfloat162>() + net->off[l], cout, cin, nvec));
+            DLZ_TRY(layer_forward(op, gn, gc, net->wadj.as<__nv_bfloat162>() + net->off[l],
+                                  net->img.as<__nv_bfloat16>() + net->img_adj[l], net->err.as<int>(), cout, cin, nvec));
             std::swap(gc, gn);
         }
     }
-    if (grad_in)
-        for (int v = 0; v < nvec; ++v) DLZ_TRY(unpack32(op, (float2 *)grad_in + (size_t)v * n, gc + (size_t)v * plane));
-    DLZ_CUDA_TRY(cudaStreamSynchronize(op.stream));
-    return DLZ_OK;
+    if (grad_in) DLZ_TRY(unpack32(op, (float2 *)grad_in, gc, nvec));
+    return check_layers(net);
 }
 
 int dlz_net_get(dlz_net_t net, int what, void *host_out) {

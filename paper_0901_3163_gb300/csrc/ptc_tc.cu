@@ -1,0 +1,372 @@
+// Tensor-core (tcgen05) form of a parallel-transport convolution layer: no counterpart in
+// arXiv:0901.3163, see ptc.cu for the layer,
+//   out[c'](x) = sum_o sum_c W[o][c'][c] (T_o in[c])(x).
+//
+// For every offset o the layer is a matrix product: a row is a site and colour, K runs over
+// the input channels, spins and re/im, N over the output channels, spins and re/im, with the
+// real form [[Re W, Im W], [-Im W, Re W]]^T of the complex spin matrices.  The weights are
+// bfloat16, exact as they are; a transported FP32 value is the exact sum of three bfloat16
+// parts (8 mantissa bits each, cut off one after another), so every product is exact and only
+// the FP32 accumulation rounds.  The tensor cores cut off their sums instead of rounding them
+// to nearest (measured as about 2e-8 of the result per MMA step), so an accumulator takes
+// kMaxSteps steps of K = 16 at most before it is added, rounding to nearest, to an FP32 sum in
+// registers.  Error against 64 bits of three layers 1 -> 12 -> 16 -> 1 on 16^4: 6.6e-7, 8.2e-7
+// with FP32 arithmetic on the CUDA cores (27 steps per accumulator: 9.5e-7).
+//
+// Block: tiles of 42 sites (126 rows) of one vector.  kGroups groups of four filling warps
+// (thread = site and a third of the chunk's channels) load a neighbour's spinor, transport it,
+// cut the values into parts and store them as the A operands (K-major 8 x 16-byte core
+// matrices, no swizzle); one warp issues the MMAs; eight warps add finished accumulators up and
+// write the tile.  They meet at mbarriers only.
+#include <algorithm>
+
+#include "ptc_tc.cuh"
+#include "tc_util.cuh"
+#include "wilson_site.cuh"
+
+namespace dlz {
+namespace {
+
+constexpr int kGroups = 3, kEpi = 8;
+constexpr int kThreads = 32 * (kEpi + 1) + 128 * kGroups;
+constexpr int kSites = 42;                       // sites of a tile: 126 of the 128 rows
+constexpr int kMaxSteps = 9;
+
+// A chunk is an offset and up to 6 input channels (two per filling thread), an even number
+__host__ __device__ inline int channel_chunks(int cin) { return (cin + 5) / 6; }
+__host__ __device__ inline int chunk_channels(int cin) {
+    const int n = channel_chunks(cin);
+    return ((cin + n - 1) / n + 1) / 2 * 2;
+}
+__host__ __device__ inline int npad_of(int cout) { return (8 * cout + 15) / 16 * 16; }
+
+struct FwdArgs {
+    float4 *out;
+    const float4 *in, *U;
+    const __nv_bfloat16 *img;
+    Geom g;
+    int cin, cout, npad, nvec, nbuf, ncols;
+    int *err;
+};
+
+struct FwdShared {
+    uint64_t full[kGroups], empty[kGroups], acc_full[4], acc_empty[4];
+    uint32_t tbase;
+    int failed;
+};
+
+__device__ __forceinline__ void mma_bf16(uint32_t taddr, uint32_t da, uint32_t db, uint32_t dhi, uint32_t idesc, bool acc) {
+    asm volatile("{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\tmov.b64 a, {%1, %5};\n\tmov.b64 b, {%2, %5};\n\t"
+                 "setp.ne.b32 p, %4, 0;\n\t"
+                 "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p;\n\t}\n" ::"r"(taddr),
+                 "r"(da), "r"(db), "r"(idesc), "r"(acc ? 1u : 0u), "r"(dhi));
+}
+
+// sum[0 .. 15] += columns addr .. addr + 15 of this warp's lane quarter (the first 8 if !wide)
+__device__ __forceinline__ void tmem_add(uint32_t addr, bool wide, float *sum) {
+    uint32_t r[16];
+#pragma unroll
+    for (int j = 0; j < 16; ++j) r[j] = 0u;
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(addr));
+    if (wide)
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                     : "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+                     : "r"(addr + 8));
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                   "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]));
+#pragma unroll
+    for (int j = 0; j < 16; ++j) sum[j] += __uint_as_float(r[j]);
+}
+
+// the upper halves of two words (two bfloat16 by cutting off) in one
+__device__ __forceinline__ uint32_t pack_hi(float a, float b) {
+    return __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632);
+}
+__device__ __forceinline__ float cut(float x) { return __uint_as_float(__float_as_uint(x) & 0xffff0000u); }
+
+// One channel's transported spinor t of the tile's site sl as K octet `oct` of the rows 3 sl +
+// colour of the three parts (part h at h * part): 8 values (spin, re/im) = 16 bytes each
+__device__ __forceinline__ void store_parts(unsigned char *stage, int part, int sbo, int sl, int oct, const float2 (&t)[12]) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const int row = 3 * sl + c;
+        unsigned char *dst = stage + (row >> 3) * sbo + oct * 128 + (row & 7) * 16;
+        float x[8];
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+            x[2 * s] = t[3 * s + c].x;
+            x[2 * s + 1] = t[3 * s + c].y;
+        }
+#pragma unroll
+        for (int h = 0; h < 3; ++h) {
+            *reinterpret_cast<uint4 *>(dst + h * part) =
+                make_uint4(pack_hi(x[0], x[1]), pack_hi(x[2], x[3]), pack_hi(x[4], x[5]), pack_hi(x[6], x[7]));
+            if (h < 2)
+#pragma unroll
+                for (int j = 0; j < 8; ++j) x[j] -= cut(x[j]);
+        }
+    }
+}
+
+// Bound by the filling warps (transport, splitting, stores).  16^4, 4 vectors, one GB300,
+// against the CUDA-core kernel: 12 -> 16 channels 4.95 -> 1.09 ms, 16 -> 12 (its adjoint) 4.9
+// -> 1.48 ms, 1 -> 12 and 1 -> 16 0.57 -> 0.38 ms.  Two filling groups: 1.19 and 1.56 ms; four
+// (fewer registers each): 1.41 and 1.54 ms.  Tiles of 128 sites with an accumulator per colour,
+// whose partial results do not fit in registers and went through global memory: 2.2 and 2.4 ms.
+__global__ void __launch_bounds__(kThreads, 1) k_ptc_tc_fwd(FwdArgs a) {
+    extern __shared__ __align__(1024) unsigned char smem[];
+    __shared__ __align__(8) FwdShared sh;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+    const int cc = chunk_channels(a.cin), ncp = channel_chunks(a.cin), sbo = cc * 128;
+    const int part = 16 * sbo, b_bytes = (a.npad / 8) * sbo, stage_bytes = 3 * part + b_bytes;
+    if (threadIdx.x == 0) {
+        sh.failed = 0;
+        for (int i = 0; i < kGroups; ++i) {
+            mbar_init(&sh.full[i], 4);
+            mbar_init(&sh.empty[i], 1);
+        }
+        for (int i = 0; i < 4; ++i) {
+            mbar_init(&sh.acc_full[i], 1);
+            mbar_init(&sh.acc_empty[i], kEpi);
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;");
+    }
+    tmem_alloc(&sh.tbase, a.ncols);
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;");
+    const uint32_t taddr = sh.tbase;
+    volatile int *failed = &sh.failed;
+    const int V = a.g.V, tiles_per_vec = (V + kSites - 1) / kSites, ntiles = tiles_per_vec * a.nvec;
+    // a tile's chunks, and the segments of chunks that one accumulator takes
+    const int nch = 9 * ncp, per = max(1, kMaxSteps / (3 * cc / 2)), nseg = (nch + per - 1) / per;
+    const size_t plane = (size_t)6 * V;
+    const int mine = (ntiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;     // the block's tiles
+    const int ft = (int)threadIdx.x - 32 * (kEpi + 1);
+    if (ft >= 0) {
+        // ---- fill: group grp takes the chunks (tile, offset, channels) grp, grp + kGroups, ...;
+        // a thread the channels cg and cg + 3 of its site
+        const int grp = ft / 128, tid = ft % 128, sl = tid % kSites, cg = tid / kSites;
+        unsigned char *stage = smem + grp * stage_bytes;
+        const long total = (long)mine * nch;
+        uint32_t round = 0;
+        int tile_of = -1, s = 0, vec = 0;
+        int c4[4] = {0, 0, 0, 0};
+        bool ok = false;
+        int ti = 0, r = grp;                       // chunk r of the block's tile ti
+        for (long q = grp; q < total; q += kGroups, ++round) {
+            while (r >= nch) { r -= nch; ++ti; }
+            const int o = r / ncp, p = r % ncp;
+            if (ti != tile_of) {
+                const int t = (int)blockIdx.x + ti * (int)gridDim.x;
+                vec = t / tiles_per_vec;
+                s = (t % tiles_per_vec) * kSites + sl;
+                ok = s < V;
+                int d = ok ? s : 0;
+                c4[0] = d % a.g.L[0]; d /= a.g.L[0];
+                c4[1] = d % a.g.L[1]; d /= a.g.L[1];
+                c4[2] = d % a.g.L[2];
+                c4[3] = d / a.g.L[2];
+                tile_of = ti;
+            }
+            int sn = ok ? s : 0;
+            float2 u[9];
+            if (o > 0 && ok) {
+                const int mu = (o - 1) >> 1;
+                const bool fwd = ((o - 1) & 1) == 0;
+                const int L = a.g.L[mu], c = mu == 0 ? c4[0] : mu == 1 ? c4[1] : mu == 2 ? c4[2] : c4[3];
+                const int st = mu == 0 ? 1 : mu == 1 ? a.g.L[0] : mu == 2 ? a.g.L[0] * a.g.L[1]
+                                                                          : a.g.L[0] * a.g.L[1] * a.g.L[2];
+                sn = fwd ? (c == L - 1 ? s - (L - 1) * st : s + st) : (c == 0 ? s + (L - 1) * st : s - st);
+                Link<float>::load(a.U, V, mu, fwd ? s : sn, u);
+                if (!fwd) {                       // U^dag
+#pragma unroll
+                    for (int i = 0; i < 3; ++i)
+#pragma unroll
+                        for (int j = i; j < 3; ++j) {
+                            const float2 x = u[3 * i + j], y = u[3 * j + i];
+                            u[3 * i + j] = make_float2(y.x, -y.y);
+                            u[3 * j + i] = make_float2(x.x, -x.y);
+                        }
+                }
+            }
+            const float4 *src = a.in + ((size_t)vec * a.cin + p * cc) * plane;
+            if (round > 0 && !__all_sync(0xffffffffu, mbar_wait(&sh.empty[grp], (round - 1) & 1u, failed))) break;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int ch = cg + 3 * h;
+                if (ch < cc && cg < 3) {
+                    float2 x[12], t[12];
+                    if (ok && p * cc + ch < a.cin) {
+                        Field<float>::load(src + ch * plane, V, sn, x);
+                        if (o > 0) {
+#pragma unroll
+                            for (int sp = 0; sp < 4; ++sp)
+#pragma unroll
+                                for (int i = 0; i < 3; ++i) {
+                                    float2 z = make_float2(0.f, 0.f);
+#pragma unroll
+                                    for (int j = 0; j < 3; ++j) z = cfma(u[3 * i + j], x[3 * sp + j], z);
+                                    t[3 * sp + i] = z;
+                                }
+                        } else {
+#pragma unroll
+                            for (int j = 0; j < 12; ++j) t[j] = x[j];
+                        }
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < 12; ++j) t[j] = make_float2(0.f, 0.f);
+                    }
+                    store_parts(stage, part, sbo, sl, ch, t);
+                }
+            }
+            // the chunk's weights in operand order
+            const uint4 *w = reinterpret_cast<const uint4 *>(a.img) + (size_t)r * (b_bytes / 16);
+            for (int i = tid; i < b_bytes / 16; i += 128) reinterpret_cast<uint4 *>(stage + 3 * part)[i] = w[i];
+            asm volatile("fence.proxy.async.shared::cta;");
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sh.full[grp]);
+            r += kGroups;
+        }
+    } else if (warp == kEpi) {
+        // ---- MMA (the warp is uniform; lane 0 issues): parts from the smallest up
+        const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(a.npad >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+        const uint32_t d0 = sdesc_lo(su32(smem)), dhi = ((uint32_t)sbo >> 4) | 1u << 14, w_stage = stage_bytes >> 4;
+        int st = 0, n = 0;
+        uint32_t round = 0;
+        bool ok = true;
+        for (int ti = 0; ti < mine && ok; ++ti)
+            for (int sg = 0; sg < nseg && ok; ++sg, ++n) {
+                const int acc = n % a.nbuf, use = n / a.nbuf;
+                const int chunks = min(nch, (sg + 1) * per) - sg * per;
+                if (use > 0 && !__all_sync(0xffffffffu, mbar_wait(&sh.acc_empty[acc], (use - 1) & 1, failed))) { ok = false; break; }
+                for (int ch = 0; ch < chunks; ++ch) {
+                    ok = __all_sync(0xffffffffu, mbar_wait(&sh.full[st], round & 1u, failed));
+                    if (!ok) break;
+                    asm volatile("tcgen05.fence::after_thread_sync;");
+                    const uint32_t da = d0 + st * w_stage, db = da + (3 * part >> 4);
+                    if (lane == 0) {
+                        for (int h = 2; h >= 0; --h)
+                            for (int k = 0; k < cc / 2; ++k)
+                                mma_bf16(taddr + acc * a.npad, da + (h * part >> 4) + k * 16, db + k * 16, dhi, idesc,
+                                         ch > 0 || h < 2 || k > 0);
+                        commit_to(&sh.empty[st]);
+                    }
+                    if (++st == kGroups) { st = 0; ++round; }
+                }
+                if (ok && lane == 0) commit_to(&sh.acc_full[acc]);
+            }
+        __syncwarp();
+    } else {
+        // ---- results: warp w has rows 32 (w % 4) .. of a tile and half of the columns; the
+        // thread of row 3 sl + c sums colour c of its output channels in registers
+        const int lq = warp & 3, half = a.npad / 2, c_lo = (warp >> 2) * half;
+        const int row = 32 * lq + lane, sl = row / 3, col = row - 3 * sl;
+        int n = 0;
+        bool ok = true;
+        for (int ti = 0; ti < mine && ok; ++ti) {
+            float sum[64];
+#pragma unroll
+            for (int j = 0; j < 64; ++j) sum[j] = 0.f;
+            for (int sg = 0; sg < nseg; ++sg, ++n) {
+                const int acc = n % a.nbuf, use = n / a.nbuf;
+                ok = __all_sync(0xffffffffu, mbar_wait(&sh.acc_full[acc], use & 1, failed));
+                if (!ok) break;
+                asm volatile("tcgen05.fence::after_thread_sync;");
+#pragma unroll
+                for (int j = 0; j < 64; j += 16)
+                    if (j < half)
+                        tmem_add(taddr + ((uint32_t)(32 * lq) << 16) + (uint32_t)(acc * a.npad + c_lo + j), j + 8 < half, sum + j);
+                asm volatile("tcgen05.fence::before_thread_sync;");
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&sh.acc_empty[acc]);
+            }
+            const int t = (int)blockIdx.x + ti * (int)gridDim.x, vec = t / tiles_per_vec;
+            const int s = (t % tiles_per_vec) * kSites + sl;
+            if (!ok || sl >= kSites || s >= V) continue;
+            // column 8 c' + 2 s' + re/im; component 3 s' + colour is half of plane (..) / 2
+            float4 *dst = a.out + (size_t)vec * a.cout * plane + s;
+#pragma unroll
+            for (int j = 0; j < 64; j += 2) {
+                const int ch = (c_lo + j) / 8, comp = 3 * ((j % 8) / 2) + col;
+                if (j < half && ch < a.cout)
+                    reinterpret_cast<float2 *>(dst + (size_t)ch * plane + (size_t)(comp >> 1) * V)[comp & 1] =
+                        make_float2(sum[j], sum[j + 1]);
+            }
+        }
+    }
+    __syncthreads();
+    if (sh.failed && threadIdx.x == 0) atomicExch(a.err, 1);
+    tc_teardown(taddr, a.ncols);
+}
+
+// the weight image: chunk (o, channels) of npad x 8 cc bf16 (cc channels), element (n, k) of the
+// K-major operand at (n / 8) * 64 cc + (k / 8) * 64 + (n % 8) * 8 + k % 8; n = 8 c' + 2 s' +
+// (0 re, 1 im), k = 8 (c within the chunk) + 2 s + (0 re, 1 im)
+__global__ void k_ptc_tc_image(__nv_bfloat16 *__restrict__ img, const __nv_bfloat162 *__restrict__ w, int cin, int cout,
+                               int npad, long total) {
+    const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= total) return;
+    const int cc = chunk_channels(cin), ncp = channel_chunks(cin), per = npad * 8 * cc;
+    const int e = (int)(i % per), chunk = (int)(i / per), o = chunk / ncp, p = chunk % ncp;
+    const int n = (e / (64 * cc)) * 8 + (e / 8) % 8, k = ((e / 64) % cc) * 8 + e % 8;
+    const int co = n / 8, so = (n % 8) / 2, io = n % 2, ci = p * cc + k / 8, si = (k % 8) / 2, ii = k % 2;
+    __nv_bfloat16 v = __float2bfloat16_rn(0.f);
+    if (co < cout && ci < cin && k / 8 < cc) {
+        const __nv_bfloat162 z = w[(((size_t)o * cout + co) * cin + ci) * 16 + 4 * so + si];
+        v = io == ii ? z.x : io == 1 ? z.y : __hneg(z.y);
+    }
+    img[i] = v;
+}
+
+int stage_bytes_of(int cin, int cout) { return chunk_channels(cin) * 128 * (3 * 16 + npad_of(cout) / 8); }
+
+}  // namespace
+
+size_t ptc_tc_image_size(int cin, int cout) {
+    return (size_t)9 * channel_chunks(cin) * npad_of(cout) * 8 * chunk_channels(cin);
+}
+
+// The tensor-core kernel pads the output channels to N = 16 at least and fills the same operands
+// however few there are: 16 -> 1 channels take 0.67 ms on the CUDA cores, about the 12 -> 16
+// layer's filling time here; from 4 output channels on it is the faster one.
+bool ptc_tc_layer(int, int cout) { return cout >= 4; }
+
+int ptc_tc_prepare() {
+    static int done = 0;
+    if (done) return DLZ_OK;
+    DLZ_CUDA_TRY(cudaFuncSetAttribute(k_ptc_tc_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      kGroups * stage_bytes_of(6, 16)));
+    done = 1;
+    return DLZ_OK;
+}
+
+int ptc_tc_image(Op &op, __nv_bfloat16 *img, const __nv_bfloat162 *w, int cin, int cout) {
+    const long total = (long)ptc_tc_image_size(cin, cout);
+    k_ptc_tc_image<<<(unsigned)((total + 255) / 256), 256, 0, op.stream>>>(img, w, cin, cout, npad_of(cout), total);
+    op.prof.launches++;
+    DLZ_CUDA_TRY(cudaGetLastError());
+    return DLZ_OK;
+}
+
+int ptc_tc_forward(Op &op, float4 *out, const float4 *in, const __nv_bfloat16 *img, int cin, int cout, int nvec,
+                   int *err) {
+    FwdArgs a;
+    a.out = out; a.in = in; a.U = op.gauge32.as<float4>(); a.img = img; a.g = op.g;
+    a.cin = cin; a.cout = cout; a.npad = npad_of(cout); a.nvec = nvec; a.err = err;
+    a.nbuf = 4;
+    const int need = a.npad * a.nbuf;
+    a.ncols = need <= 64 ? 64 : need <= 128 ? 128 : need <= 256 ? 256 : 512;
+    const long tiles = (long)((op.g.V + kSites - 1) / kSites) * nvec;
+    int dev = 0, nsm = 0;
+    DLZ_CUDA_TRY(cudaGetDevice(&dev));
+    DLZ_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    k_ptc_tc_fwd<<<(unsigned)std::min<long>(tiles, nsm), kThreads, kGroups * stage_bytes_of(cin, cout), op.stream>>>(a);
+    op.prof.launches++;
+    DLZ_CUDA_TRY(cudaGetLastError());
+    return DLZ_OK;
+}
+
+}  // namespace dlz

@@ -1,0 +1,21 @@
+// Tensor-core form of a parallel-transport convolution layer (ptc.cu has the layer).
+#pragma once
+
+#include <cuda_bf16.h>
+
+#include "dlz_internal.cuh"
+
+namespace dlz {
+
+// bf16 elements of a layer's weight image (ptc_tc.cu)
+size_t ptc_tc_image_size(int cin, int cout);
+// whether the layer runs on the tensor cores
+bool ptc_tc_layer(int cin, int cout);
+int ptc_tc_prepare();       // kernel attributes, outside graph captures
+// weights [9][cout][cin][16] -> image
+int ptc_tc_image(Op &op, __nv_bfloat16 *img, const __nv_bfloat162 *w, int cin, int cout);
+// the layer on nvec fields; *err (device) is set if a wait gave up
+int ptc_tc_forward(Op &op, float4 *out, const float4 *in, const __nv_bfloat16 *img, int cin, int cout, int nvec,
+                   int *err);
+
+}  // namespace dlz

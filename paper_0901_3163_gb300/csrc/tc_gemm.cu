@@ -26,6 +26,7 @@
 #include <vector>
 
 #include "dlz_internal.cuh"
+#include "tc_util.cuh"
 
 namespace dlz {
 
@@ -45,17 +46,8 @@ constexpr int kEpiWarps = 8;
 constexpr int kFill = 128;                                   // threads of a group, and of the copying warps
 constexpr int tc_threads(int groups) { return 32 * (kEpiWarps + 1) + (groups + 1) * kFill; }
 constexpr int kKC = 32;             // K chunk staged per pipeline stage
-constexpr int kWaitPolls = 1 << 22;     // (each poll may suspend the thread for a while)
 constexpr int kTcMaxSmem = 226 * 1024;      // dynamic shared memory a block may ask for
 constexpr int kABytes = 128 * kKC * 4;      // one part (hi or lo) of an A chunk
-
-__device__ __forceinline__ uint32_t su32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-// Operand descriptor at shared address `saddr`: 14 address bits (16-byte units) and the
-// leading byte offset in the low word, stride byte offset and the descriptor version of the
-// sm_100 family (no swizzle) in the high word.  Only the low word changes along K.
-__device__ __forceinline__ uint32_t sdesc_lo(uint32_t saddr) { return ((saddr >> 4) & 0x3FFF) | (128u >> 4) << 16; }
-constexpr uint32_t kDescHi = (1024u >> 4) | 1u << 14;
 
 // instruction descriptor: D FP32 (bits 4-5), A and B TF32 (7-9, 10-12), both K-major
 // (bits 15, 16 zero), N / 8 (17-22), M / 16 (24-28) with M = 128
@@ -68,31 +60,7 @@ __device__ __forceinline__ void mma_tf32(uint32_t taddr, uint32_t da, uint32_t d
     asm volatile("{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\tmov.b64 a, {%1, %5};\n\tmov.b64 b, {%2, %5};\n\t"
                  "setp.ne.b32 p, %4, 0;\n\t"
                  "tcgen05.mma.cta_group::1.kind::tf32 [%0], a, b, %3, p;\n\t}\n" ::"r"(taddr),
-                 "r"(da), "r"(db), "r"(idesc), "r"(ACC ? 1u : (acc ? 1u : 0u)), "r"(kDescHi));
-}
-
-__device__ __forceinline__ void commit_to(uint64_t *mbar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(su32(mbar)));
-}
-
-// Bounded wait for the completion of phase `parity` of an mbarrier.  A wait that gives up
-// sets the block's fail word, which ends the other waits as well.
-__device__ __forceinline__ bool mbar_wait(uint64_t *mbar, uint32_t parity, volatile int *failed) {
-    uint32_t done = 0;
-    for (int it = 0; it < kWaitPolls && !done; ++it) {
-        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-                     "selp.u32 %0, 1, 0, p;\n\t}\n"
-                     : "=r"(done) : "r"(su32(mbar)), "r"(parity) : "memory");
-        if (!done && *failed) return false;
-    }
-    if (!done) *failed = 1;
-    return done != 0;
-}
-__device__ __forceinline__ void mbar_arrive(uint64_t *mbar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(su32(mbar)) : "memory");
-}
-__device__ __forceinline__ void mbar_init(uint64_t *mbar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(mbar)), "r"(count));
+                 "r"(da), "r"(db), "r"(idesc), "r"(ACC ? 1u : (acc ? 1u : 0u)), "r"(kDescHi<1024>));
 }
 
 // Asynchronous 16-byte copy of the raw ring; valid = false fills the slot with zeros.
@@ -185,21 +153,10 @@ template <int S, int R> __device__ __forceinline__ uint32_t tc_setup(TcShared<S,
         }
         asm volatile("fence.mbarrier_init.release.cluster;");
     }
-    if ((threadIdx.x >> 5) == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(&sh.tbase)), "r"(ncols));
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;");
+    tmem_alloc(&sh.tbase, ncols);
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
     return sh.tbase;
-}
-
-__device__ __forceinline__ void tc_teardown(uint32_t taddr, int ncols) {
-    asm volatile("tcgen05.fence::before_thread_sync;");
-    __syncthreads();
-    if ((threadIdx.x >> 5) == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols));
 }
 
 // One chunk's MMAs into the accumulator at `acc`: hi hi + hi lo + lo hi over 32 k, from the
@@ -217,7 +174,6 @@ __device__ __forceinline__ void chunk_mmas(uint32_t acc, uint32_t ah, uint32_t a
     }
 }
 
-__device__ __forceinline__ int tmem_cols(int n) { return n <= 32 ? 32 : n <= 64 ? 64 : n <= 128 ? 128 : n <= 256 ? 256 : 512; }
 
 // The combine's A operand, item (row quad, k quad kq) of a chunk: vectors 4 kq .. 4 kq + 3 of
 // K chunk kc at rows r .. r + 3 (zero beyond the data; for complex coefficients the second
