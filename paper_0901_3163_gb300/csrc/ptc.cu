@@ -37,11 +37,8 @@ namespace dlz {
 constexpr int kMaxLayersNet = 8;
 namespace {
 
-constexpr int kMaxWidth = 16;      // channels per layer (weight-gradient tile limit)
+constexpr int kMaxWidth = 16;      // channels per layer (128 rows of the tensor-core operands)
 constexpr int kFwdThreads = 128;
-constexpr int kTS = 32;            // sites per weight-gradient tile
-constexpr int kLD = 3 * kTS + 1;   // padded row of a staged tile (float2)
-constexpr int kGradBlocks = 64;    // weight-gradient blocks per offset
 
 __device__ inline int opposite(int o) { return o == 0 ? 0 : (((o - 1) & 1) == 0 ? o + 1 : o - 1); }
 
@@ -81,21 +78,6 @@ __device__ inline void transport(const float2 (&p)[12], const float2 (&u)[9], bo
             t[3 * sp + i] = a;
         }
     }
-}
-
-__device__ inline void load_transported(const float4 *__restrict__ x, const float4 *__restrict__ U,
-                                        const Geom &g, int s, int o, float2 (&t)[12]) {
-    if (o == 0) {
-        Field<float>::load(x, g.V, s, t);
-        return;
-    }
-    int sn, ls, mu;
-    bool fwd;
-    neighbour(s, g, o, sn, ls, mu, fwd);
-    float2 p[12], u[9];
-    Field<float>::load(x, g.V, sn, p);
-    Link<float>::load(U, g.V, mu, ls, u);
-    transport(p, u, fwd, t);
 }
 
 // out[vec][g0 + q] for q < CG; grid (site blocks, C_out / CG, nvec)
@@ -161,93 +143,6 @@ k_ptc_fwd(float4 *__restrict__ out, const float4 *__restrict__ in, const __nv_bf
     float4 *ov = out + (size_t)vec * cout * plane;
 #pragma unroll
     for (int q = 0; q < CG; ++q) Field<float>::store(ov + (size_t)(g0 + q) * plane, g.V, s, acc[q]);
-}
-
-// Block partials of G(W)[o] = sum_{x, colour} G(out) (T_o in)^dag, as the GEMM
-// (C_out*4) x (3 sites) times (3 sites) x (C_in*4) over tiles of kTS sites.
-// grid (gridDim.x, 9); partials [o][block][C_out*4][C_in*4].
-// FP32-FMA bound.  Thread (tx, ty) of 16 x 16 keeps RI x CJ complex sums, RI = ceil(C_out / 4)
-// and CJ = ceil(C_in / 4): with 4 x 4 sums for every layer the 1 -> 12 and 16 -> 1 layers
-// (16^4, 4 vectors) took the 6.75 ms of the 12 -> 16 layer.
-template <int RI, int CJ>
-__global__ void __launch_bounds__(256)
-k_ptc_wgrad(float2 *__restrict__ partials, const float4 *__restrict__ gout, const float4 *__restrict__ x,
-            const float4 *__restrict__ U, Geom g, int cin, int cout, int nvec) {
-    extern __shared__ float2 sm[];
-    const int rows = cout * 4, cols = cin * 4;
-    float2 *Gs = sm;                   // [16 RI][kLD]
-    float2 *Ts = sm + 16 * RI * kLD;   // [16 CJ][kLD]
-    const int o = blockIdx.y;
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    float2 acc[RI][CJ];
-#pragma unroll
-    for (int i = 0; i < RI; ++i)
-#pragma unroll
-        for (int j = 0; j < CJ; ++j) acc[i][j] = make_float2(0.f, 0.f);
-    // rows beyond the layer's own stay zero
-    for (int t = threadIdx.x; t < 16 * (RI + CJ) * kLD; t += 256) sm[t] = make_float2(0.f, 0.f);
-    const size_t plane = (size_t)6 * g.V;
-    const int tiles_per_vec = (g.V + kTS - 1) / kTS;
-    const long ntiles = (long)tiles_per_vec * nvec;
-    const int ls = threadIdx.x % kTS, slot = threadIdx.x / kTS;   // 32 sites x 8 slots
-    for (long tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        const int vec = (int)(tile / tiles_per_vec);
-        const int s = (int)(tile % tiles_per_vec) * kTS + ls;
-        const bool ok = s < g.V;
-        __syncthreads();
-        // the channels of both operands shared out over the 8 slots
-        for (int ch = slot; ch < cout + cin; ch += 8) {
-            const bool is_g = ch < cout;
-            const int c = is_g ? ch : ch - cout;
-            float2 p[12];
-            if (!ok) {
-#pragma unroll
-                for (int a = 0; a < 12; ++a) p[a] = make_float2(0.f, 0.f);
-            } else if (is_g) {
-                Field<float>::load(gout + ((size_t)vec * cout + c) * plane, g.V, s, p);
-            } else {
-                load_transported(x + ((size_t)vec * cin + c) * plane, U, g, s, o, p);
-            }
-            float2 *dst = (is_g ? Gs : Ts) + c * 4 * kLD + ls;
-#pragma unroll
-            for (int sp = 0; sp < 4; ++sp)
-#pragma unroll
-                for (int a = 0; a < 3; ++a) dst[sp * kLD + a * kTS] = p[3 * sp + a];
-        }
-        __syncthreads();
-#pragma unroll 2
-        for (int k = 0; k < 3 * kTS; ++k) {
-            float2 gv[RI], tv[CJ];
-#pragma unroll
-            for (int i = 0; i < RI; ++i) gv[i] = Gs[(ty + 16 * i) * kLD + k];
-#pragma unroll
-            for (int j = 0; j < CJ; ++j) tv[j] = Ts[(tx + 16 * j) * kLD + k];
-#pragma unroll
-            for (int i = 0; i < RI; ++i)
-#pragma unroll
-                for (int j = 0; j < CJ; ++j) acc[i][j] = cfmaConj(tv[j], gv[i], acc[i][j]);
-        }
-    }
-    float2 *pb = partials + ((size_t)o * gridDim.x + blockIdx.x) * rows * cols;
-#pragma unroll
-    for (int i = 0; i < RI; ++i)
-#pragma unroll
-        for (int j = 0; j < CJ; ++j) {
-            const int r = ty + 16 * i, c = tx + 16 * j;
-            if (r < rows && c < cols) pb[(size_t)r * cols + c] = acc[i][j];
-        }
-}
-typedef void (*WgradKernel)(float2 *, const float4 *, const float4 *, const float4 *, Geom, int, int, int);
-template <int RI> WgradKernel wgrad_of(int cj) {
-    return cj == 1 ? (WgradKernel)k_ptc_wgrad<RI, 1> : cj == 2 ? (WgradKernel)k_ptc_wgrad<RI, 2>
-         : cj == 3 ? (WgradKernel)k_ptc_wgrad<RI, 3> : (WgradKernel)k_ptc_wgrad<RI, 4>;
-}
-WgradKernel wgrad_kernel(int cin, int cout) {
-    const int ri = (cout + 3) / 4, cj = (cin + 3) / 4;
-    return ri == 1 ? wgrad_of<1>(cj) : ri == 2 ? wgrad_of<2>(cj) : ri == 3 ? wgrad_of<3>(cj) : wgrad_of<4>(cj);
-}
-inline size_t wgrad_smem(int cin, int cout) {
-    return (size_t)16 * ((cout + 3) / 4 + (cin + 3) / 4) * kLD * sizeof(float2);
 }
 
 // grad[o][c'][c][4 s' + s] += sum over blocks (fixed order) of the partials
@@ -393,10 +288,6 @@ int set_attrs() {
     static bool done = false;
     if (done) return DLZ_OK;
     DLZ_TRY(ptc_tc_prepare());
-    const int wg = (int)((size_t)(2 * kMaxWidth * 4) * kLD * sizeof(float2));
-    for (int co = 4; co <= kMaxWidth; co += 4)
-        for (int ci = 4; ci <= kMaxWidth; ci += 4)
-            DLZ_CUDA_TRY(cudaFuncSetAttribute(wgrad_kernel(ci, co), cudaFuncAttributeMaxDynamicSharedMemorySize, wg));
     const int fw = 9 * 4 * kMaxWidth * 16 * (int)sizeof(__nv_bfloat162);
     DLZ_CUDA_TRY(cudaFuncSetAttribute(k_ptc_fwd<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, fw));
     DLZ_CUDA_TRY(cudaFuncSetAttribute(k_ptc_fwd<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, fw));
@@ -460,7 +351,7 @@ int dlz_net_create(dlz_op_t h, int nlayers, const int *widths, const void *weigh
         DLZ_CUDA_TRY(cudaMemsetAsync(net->err.p, 0, sizeof(int), op.stream));
         int maxp = 0;
         for (int l = 0; l < nlayers; ++l) maxp = std::max(maxp, 16 * widths[l] * widths[l + 1]);
-        DLZ_TRY(net->partials.alloc((size_t)9 * kGradBlocks * maxp * sizeof(float2)));
+        DLZ_TRY(net->partials.alloc((size_t)9 * kPtcMaxGradBlocks * maxp * sizeof(float2)));
         const void *src = weights;
         std::vector<float2> hw;
         if (!device_ptr(weights)) {
@@ -527,12 +418,13 @@ int dlz_net_backward(dlz_net_t net, const void *grad_out, int nvec, void *grad_i
     DLZ_TRY(pack32(op, gc, (const float2 *)grad_out, nvec));
     for (int l = net->nl - 1; l >= 0; --l) {
         const int cin = net->w[l], cout = net->w[l + 1];
-        wgrad_kernel(cin, cout)<<<dim3(kGradBlocks, 9), 256, wgrad_smem(cin, cout), op.stream>>>(
-            net->partials.as<float2>(), gc, net->act[l].as<float4>(), op.gauge32.as<float4>(), op.g, cin, cout, nvec);
+        int blocks = 0;
+        DLZ_TRY(ptc_tc_wgrad(op, net->partials.as<float2>(), gc, net->act[l].as<float4>(), cin, cout, nvec,
+                             net->err.as<int>(), blocks));
         const long ne = 9L * cin * cout * 16;
         k_ptc_wgrad_sum<<<blocks_for(ne, 256), 256, 0, op.stream>>>(net->grad.as<float2>() + net->off[l],
-                                                                    net->partials.as<float2>(), kGradBlocks, cin, cout);
-        op.prof.launches += 2;
+                                                                    net->partials.as<float2>(), blocks, cin, cout);
+        op.prof.launches += 1;
         DLZ_CUDA_TRY(cudaGetLastError());
         if (l > 0 || grad_in) {
             DLZ_TRY(layer_forward(op, gn, gc, net->wadj.as<__nv_bfloat162>() + net->off[l],

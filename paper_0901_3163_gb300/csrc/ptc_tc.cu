@@ -302,6 +302,200 @@ __global__ void __launch_bounds__(kThreads, 1) k_ptc_tc_fwd(FwdArgs a) {
     tc_teardown(taddr, a.ncols);
 }
 
+// ------------------------------------------------------------------ weight gradient
+// G(W)[o][c'][c] = sum over sites and colours of G(out) (T_o in)^dag as P[m][n] = sum_k A[m][k]
+// B[n][k]: m = 8 c' + 2 s' + re/im of G(out), n = 8 c + 2 s + re/im of the transported input, k
+// the sites and colours; re G = P[re][re] + P[im][im], im G = P[im][re] - P[re][im].  Both
+// operands are FP32 values in three bfloat16 parts h, m, l; of the nine products of parts the
+// six down to 2^-16 are formed (the others are below 2^-24), smallest first, so that only the
+// three steps of h h are cut off at the size of the sum.
+// A block has one offset and every gridDim.x-th tile of 16 sites: a stage is one tile, 48 k (K
+// step = colour).  The operands are stored as they come, 16 bytes = the 8 values of a channel at
+// one k, i.e. M- and N-major: 8 x 8 core matrices of 8 k x 16 bytes, k groups 128 bytes apart,
+// row groups 768.  Each tile's accumulator is added to FP32 sums in registers.
+constexpr int kGSites = 16, kGSbo = 3 * kGSites * 16, kGPartA = 16 * kGSbo;
+
+struct GradArgs {
+    float2 *partials;
+    const float4 *gout, *in, *U;
+    Geom g;
+    int cin, cout, npad, nvec, nbuf, ncols;
+    int *err;
+};
+
+// channel octet `oct` at site sl in the three parts (part p at p * part)
+__device__ __forceinline__ void store_parts_k(unsigned char *base, int part, int oct, int sl, const float2 (&t)[12]) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        unsigned char *dst = base + oct * kGSbo + (2 * c + (sl >> 3)) * 128 + (sl & 7) * 16;
+        float x[8];
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+            x[2 * s] = t[3 * s + c].x;
+            x[2 * s + 1] = t[3 * s + c].y;
+        }
+#pragma unroll
+        for (int h = 0; h < 3; ++h) {
+            *reinterpret_cast<uint4 *>(dst + h * part) =
+                make_uint4(pack_hi(x[0], x[1]), pack_hi(x[2], x[3]), pack_hi(x[4], x[5]), pack_hi(x[6], x[7]));
+            if (h < 2)
+#pragma unroll
+                for (int j = 0; j < 8; ++j) x[j] -= cut(x[j]);
+        }
+    }
+}
+
+__global__ void __launch_bounds__(kThreads, 1) k_ptc_tc_wgrad(GradArgs a) {
+    extern __shared__ __align__(1024) unsigned char smem[];
+    __shared__ __align__(8) FwdShared sh;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+    const int part_b = (a.npad / 8) * kGSbo, stage_bytes = 3 * (kGPartA + part_b);
+    if (threadIdx.x == 0) {
+        sh.failed = 0;
+        for (int i = 0; i < kGroups; ++i) {
+            mbar_init(&sh.full[i], 4);
+            mbar_init(&sh.empty[i], 1);
+        }
+        for (int i = 0; i < 4; ++i) {
+            mbar_init(&sh.acc_full[i], 1);
+            mbar_init(&sh.acc_empty[i], kEpi);
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;");
+    }
+    tmem_alloc(&sh.tbase, a.ncols);
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;");
+    const uint32_t taddr = sh.tbase;
+    volatile int *failed = &sh.failed;
+    const int V = a.g.V, tiles_per_vec = (V + kGSites - 1) / kGSites, ntiles = tiles_per_vec * a.nvec;
+    const int o = blockIdx.y, rows = 4 * a.cout, cols = 4 * a.cin;
+    const size_t plane = (size_t)6 * V;
+    const int mine = (int)blockIdx.x < ntiles ? (ntiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
+    const int ft = (int)threadIdx.x - 32 * (kEpi + 1);
+    if (ft >= 0) {
+        // ---- fill: group grp takes the block's tiles grp, grp + kGroups, ...; a thread its site's
+        // channels tid / 16, tid / 16 + 8, ... of G(out) and then of the input
+        const int grp = ft / 128, tid = ft % 128, sl = tid % kGSites;
+        unsigned char *stage = smem + grp * stage_bytes;
+        uint32_t round = 0;
+        for (int q = grp; q < mine; q += kGroups, ++round) {
+            const int t = (int)blockIdx.x + q * (int)gridDim.x, vec = t / tiles_per_vec;
+            const int s = (t % tiles_per_vec) * kGSites + sl;
+            const bool ok = s < V;
+            int sn = ok ? s : 0;
+            float2 u[9];
+            if (o > 0 && ok) {
+                const int mu = (o - 1) >> 1;
+                const bool fwd = ((o - 1) & 1) == 0;
+                int d = s, st = 1;
+                for (int i = 0; i < mu; ++i) { d /= a.g.L[i]; st *= a.g.L[i]; }
+                const int L = a.g.L[mu], c = d % L;
+                sn = fwd ? (c == L - 1 ? s - (L - 1) * st : s + st) : (c == 0 ? s + (L - 1) * st : s - st);
+                Link<float>::load(a.U, V, mu, fwd ? s : sn, u);
+                if (!fwd) {                       // U^dag
+#pragma unroll
+                    for (int i = 0; i < 3; ++i)
+#pragma unroll
+                        for (int j = i; j < 3; ++j) {
+                            const float2 x = u[3 * i + j], y = u[3 * j + i];
+                            u[3 * i + j] = make_float2(y.x, -y.y);
+                            u[3 * j + i] = make_float2(x.x, -x.y);
+                        }
+                }
+            }
+            if (round > 0 && !__all_sync(0xffffffffu, mbar_wait(&sh.empty[grp], (round - 1) & 1u, failed))) break;
+            for (int ch = tid / kGSites; ch < a.cout + a.cin; ch += 128 / kGSites) {
+                const bool is_g = ch < a.cout;
+                const int c = is_g ? ch : ch - a.cout;
+                float2 x[12];
+                if (!ok) {
+#pragma unroll
+                    for (int j = 0; j < 12; ++j) x[j] = make_float2(0.f, 0.f);
+                } else if (is_g) {
+                    Field<float>::load(a.gout + ((size_t)vec * a.cout + c) * plane, V, s, x);
+                } else {
+                    Field<float>::load(a.in + ((size_t)vec * a.cin + c) * plane, V, sn, x);
+                    if (o > 0) {
+#pragma unroll
+                        for (int sp = 0; sp < 4; ++sp) {
+                            const float2 y0 = x[3 * sp], y1 = x[3 * sp + 1], y2 = x[3 * sp + 2];
+#pragma unroll
+                            for (int i = 0; i < 3; ++i)
+                                x[3 * sp + i] = cfma(u[3 * i + 2], y2, cfma(u[3 * i + 1], y1, cfma(u[3 * i], y0, make_float2(0.f, 0.f))));
+                        }
+                    }
+                }
+                store_parts_k(is_g ? stage : stage + 3 * kGPartA, is_g ? kGPartA : part_b, c, sl, x);
+            }
+            asm volatile("fence.proxy.async.shared::cta;");
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sh.full[grp]);
+        }
+    } else if (warp == kEpi) {
+        // ---- MMA (the warp is uniform; lane 0 issues); both operands M- / N-major (bits 15, 16)
+        const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) |
+                               ((uint32_t)(a.npad >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+        const uint32_t d0 = sdesc_lo(su32(smem)), w_stage = stage_bytes >> 4;
+        const int pa[6] = {2, 0, 1, 1, 0, 0}, pb[6] = {0, 2, 1, 0, 1, 0};
+        int st = 0;
+        uint32_t round = 0;
+        for (int n = 0; n < mine; ++n) {
+            const int acc = n % a.nbuf, use = n / a.nbuf;
+            if (use > 0 && !__all_sync(0xffffffffu, mbar_wait(&sh.acc_empty[acc], (use - 1) & 1, failed))) break;
+            if (!__all_sync(0xffffffffu, mbar_wait(&sh.full[st], round & 1u, failed))) break;
+            asm volatile("tcgen05.fence::after_thread_sync;");
+            const uint32_t da = d0 + st * w_stage, db = da + (3 * kGPartA >> 4);
+            if (lane == 0) {
+#pragma unroll
+                for (int p = 0; p < 6; ++p)
+#pragma unroll
+                    for (int k = 0; k < 3; ++k)
+                        mma_bf16(taddr + acc * a.npad, da + (pa[p] * kGPartA >> 4) + k * 16, db + (pb[p] * part_b >> 4) + k * 16,
+                                 kDescHi<kGSbo>, idesc, p > 0 || k > 0);
+                commit_to(&sh.empty[st]);
+                commit_to(&sh.acc_full[acc]);
+            }
+            if (++st == kGroups) { st = 0; ++round; }
+        }
+        __syncwarp();
+    } else {
+        // ---- sums: warp w has rows 32 (w % 4) .. and half of the columns
+        const int lq = warp & 3, half = a.npad / 2, c_lo = (warp >> 2) * half;
+        float sum[64];
+#pragma unroll
+        for (int j = 0; j < 64; ++j) sum[j] = 0.f;
+        for (int n = 0; n < mine; ++n) {
+            const int acc = n % a.nbuf, use = n / a.nbuf;
+            if (!__all_sync(0xffffffffu, mbar_wait(&sh.acc_full[acc], use & 1, failed))) break;
+            asm volatile("tcgen05.fence::after_thread_sync;");
+#pragma unroll
+            for (int j = 0; j < 64; j += 16)
+                if (j < half)
+                    tmem_add(taddr + ((uint32_t)(32 * lq) << 16) + (uint32_t)(acc * a.npad + c_lo + j), j + 8 < half, sum + j);
+            asm volatile("tcgen05.fence::before_thread_sync;");
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sh.acc_empty[acc]);
+        }
+        // row 2 r + (0 re, 1 im): the re lane combines its sums with its neighbour's
+        const int r = (32 * lq + lane) / 2;
+        float2 *pb = a.partials + ((size_t)o * gridDim.x + blockIdx.x) * rows * cols;
+#pragma unroll
+        for (int j = 0; j < 64; j += 2) {
+            const float q0 = __shfl_down_sync(0xffffffffu, sum[j], 1), q1 = __shfl_down_sync(0xffffffffu, sum[j + 1], 1);
+            const int c = (c_lo + j) / 2;
+            if (j < half && (lane & 1) == 0 && r < rows && c < cols)
+                pb[(size_t)r * cols + c] = make_float2(sum[j] + q1, q0 - sum[j + 1]);
+        }
+    }
+    __syncthreads();
+    if (sh.failed && threadIdx.x == 0) atomicExch(a.err, 1);
+    tc_teardown(taddr, a.ncols);
+}
+
+int grad_stage_bytes(int cin) { return 3 * (kGPartA + (npad_of(cin) / 8) * kGSbo); }
+
+int tmem_columns(int need) { return need <= 64 ? 64 : need <= 128 ? 128 : need <= 256 ? 256 : 512; }
+
 // the weight image: chunk (o, channels) of npad x 8 cc bf16 (cc channels), element (n, k) of the
 // K-major operand at (n / 8) * 64 cc + (k / 8) * 64 + (n % 8) * 8 + k % 8; n = 8 c' + 2 s' +
 // (0 re, 1 im), k = 8 (c within the chunk) + 2 s + (0 re, 1 im)
@@ -339,6 +533,8 @@ int ptc_tc_prepare() {
     if (done) return DLZ_OK;
     DLZ_CUDA_TRY(cudaFuncSetAttribute(k_ptc_tc_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       kGroups * stage_bytes_of(6, 16)));
+    DLZ_CUDA_TRY(cudaFuncSetAttribute(k_ptc_tc_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      kGroups * grad_stage_bytes(16)));
     done = 1;
     return DLZ_OK;
 }
@@ -358,12 +554,31 @@ int ptc_tc_forward(Op &op, float4 *out, const float4 *in, const __nv_bfloat16 *i
     a.cin = cin; a.cout = cout; a.npad = npad_of(cout); a.nvec = nvec; a.err = err;
     a.nbuf = 4;
     const int need = a.npad * a.nbuf;
-    a.ncols = need <= 64 ? 64 : need <= 128 ? 128 : need <= 256 ? 256 : 512;
+    a.ncols = tmem_columns(need);
     const long tiles = (long)((op.g.V + kSites - 1) / kSites) * nvec;
     int dev = 0, nsm = 0;
     DLZ_CUDA_TRY(cudaGetDevice(&dev));
     DLZ_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
     k_ptc_tc_fwd<<<(unsigned)std::min<long>(tiles, nsm), kThreads, kGroups * stage_bytes_of(cin, cout), op.stream>>>(a);
+    op.prof.launches++;
+    DLZ_CUDA_TRY(cudaGetLastError());
+    return DLZ_OK;
+}
+
+int ptc_tc_wgrad(Op &op, float2 *partials, const float4 *gout, const float4 *in, int cin, int cout, int nvec, int *err,
+                 int &blocks) {
+    GradArgs a;
+    a.partials = partials; a.gout = gout; a.in = in; a.U = op.gauge32.as<float4>(); a.g = op.g;
+    a.cin = cin; a.cout = cout; a.npad = npad_of(cin); a.nvec = nvec; a.err = err;
+    a.nbuf = 4;
+    a.ncols = tmem_columns(a.npad * a.nbuf);
+    // nine offsets share the SMs
+    const long tiles = (long)((op.g.V + kGSites - 1) / kGSites) * nvec;
+    int dev = 0, nsm = 0;
+    DLZ_CUDA_TRY(cudaGetDevice(&dev));
+    DLZ_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    blocks = (int)std::max<long>(1, std::min<long>({tiles, (long)nsm / 9, (long)kPtcMaxGradBlocks}));
+    k_ptc_tc_wgrad<<<dim3(blocks, 9), kThreads, kGroups * grad_stage_bytes(cin), op.stream>>>(a);
     op.prof.launches++;
     DLZ_CUDA_TRY(cudaGetLastError());
     return DLZ_OK;

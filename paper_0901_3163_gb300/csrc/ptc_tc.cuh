@@ -17,5 +17,10 @@ int ptc_tc_image(Op &op, __nv_bfloat16 *img, const __nv_bfloat162 *w, int cin, i
 // the layer on nvec fields; *err (device) is set if a wait gave up
 int ptc_tc_forward(Op &op, float4 *out, const float4 *in, const __nv_bfloat16 *img, int cin, int cout, int nvec,
                    int *err);
+// block partials [9][blocks][4 cout][4 cin] of the layer's weight gradient from G(out) and the
+// layer's input; blocks <= kPtcMaxGradBlocks
+constexpr int kPtcMaxGradBlocks = 64;
+int ptc_tc_wgrad(Op &op, float2 *partials, const float4 *gout, const float4 *in, int cin, int cout, int nvec, int *err,
+                 int &blocks);
 
 }  // namespace dlz
