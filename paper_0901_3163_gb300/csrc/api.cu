@@ -396,6 +396,7 @@ int dlz_create_operator(const int dims[4], const void *gauge, double kappa, int 
     dlz_op_s *h = new dlz_op_s();
     Op &op = h->op;
     for (int i = 0; i < 4; ++i) op.g.L[i] = dims[i];
+    op.g.set_divisors();
     op.g.V = (int)V;
     op.g.bc_t = bc_t;
     op.kappa = kappa;
@@ -778,20 +779,18 @@ static int dsolve_entry(dlz_op_t h, dlz_defl_t d, const void *B, void *X, int nr
     if (p->precision == DLZ_F32) {
         // batched mixed-precision D-MinRes / D-CG, up to 16 right-hand sides per pass
         const int chunk = std::min(nrhs, 16);
-        DevBuf bi, xi;
-        DLZ_TRY(bi.alloc((size_t)chunk * n * sizeof(double2)));
-        DLZ_TRY(xi.alloc((size_t)chunk * n * sizeof(double2)));
+        ScratchLease ws(op.pool, op.stream);
+        DLZ_TRY(ws.take((size_t)2 * chunk * n * sizeof(double2)));
+        double2 *bi = ws.b->as<double2>(), *xi = bi + (size_t)chunk * n;
         std::vector<dlz_stats> sts(chunk);
         for (int r0 = 0; r0 < nrhs; r0 += chunk) {
             const int nb = std::min(chunk, nrhs - r0);
             CallStats cs(op, nullptr, p->profile != 0, p->precision == DLZ_F32);
-            for (int q = 0; q < nb; ++q)
-                DLZ_TRY(pack64(op, bi.as<double2>() + (size_t)q * n, (const double2 *)sb.dev + (size_t)(r0 + q) * n));
-            const int rc = dsolve_mixed_batch(op, d, minres, bi.as<double2>(), xi.as<double2>(), nb, *p, sts.data());
+            DLZ_TRY(pack64(op, bi, (const double2 *)sb.dev + (size_t)r0 * n, nb));
+            const int rc = dsolve_mixed_batch(op, d, minres, bi, xi, nb, *p, sts.data());
             if (rc != DLZ_OK && rc != DLZ_ERR_NOT_CONVERGED) return rc;
             if (rc != DLZ_OK) worst = rc;
-            for (int q = 0; q < nb; ++q)
-                DLZ_TRY(unpack64(op, (double2 *)sx.dev + (size_t)(r0 + q) * n, xi.as<double2>() + (size_t)q * n));
+            DLZ_TRY(unpack64(op, (double2 *)sx.dev + (size_t)r0 * n, xi, nb));
             DLZ_CUDA_TRY(cudaStreamSynchronize(op.stream));
             dlz_stats shared;
             std::memset(&shared, 0, sizeof(shared));

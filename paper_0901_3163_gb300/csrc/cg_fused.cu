@@ -114,9 +114,9 @@ __device__ inline void cg_step(const float4 *__restrict__ G, const float4 *A, fl
                                int *__restrict__ err) {
     extern __shared__ __align__(128) float4 stage_sm[];
     __shared__ __align__(8) uint64_t mbar;
-    const int q = blockIdx.x % N;
-    int s0, nb;
-    slab_block(w, blockIdx.x / N, s0, nb);
+    int q, sb, s0, nb;
+    slab_rhs(w, blockIdx.x, q, sb);
+    slab_block(w, sb, s0, nb);
     const int s = s0 + threadIdx.x;
     const size_t base = (size_t)q * 6 * g.V;
     if (threadIdx.x == 0 && nb > 0) {
@@ -139,8 +139,7 @@ __device__ inline void cg_step(const float4 *__restrict__ G, const float4 *A, fl
         }
         v[0] = step_update<DAG>(A, O, base, g.V, s, c, o);
     }
-    const int nbq = gridDim.x / N;
-    block_partials<1>(v, partials + (size_t)q * nbq + blockIdx.x / N, 0);
+    block_partials<1>(v, partials + (size_t)q * w.dN.div(gridDim.x) + sb, 0);
 }
 
 // K1: t = D r + beta t; partial |t|^2.  Gathers r only.
@@ -199,9 +198,9 @@ k_cg_directions(CgResiduals R, float4 *__restrict__ P, float4 *__restrict__ E, c
 __global__ void __launch_bounds__(kT)
 k_cg_start_norms(const float4 *__restrict__ R, const float4 *__restrict__ S, int V, SlabWalk w, int N,
                  double *__restrict__ partials) {
-    const int q = blockIdx.x % N;
-    int s0, nb;
-    slab_block(w, blockIdx.x / N, s0, nb);
+    int q, sb, s0, nb;
+    slab_rhs(w, blockIdx.x, q, sb);
+    slab_block(w, sb, s0, nb);
     float v[2] = {0.f, 0.f};
     if ((int)threadIdx.x < nb) {
 #pragma unroll
@@ -212,8 +211,8 @@ k_cg_start_norms(const float4 *__restrict__ R, const float4 *__restrict__ S, int
             v[1] += (s.x * s.x + s.y * s.y) + (s.z * s.z + s.w * s.w);
         }
     }
-    const int nbq = gridDim.x / N;
-    block_partials<2>(v, partials + (size_t)q * nbq + blockIdx.x / N, (size_t)N * nbq);
+    const size_t nbq = w.dN.div(gridDim.x);
+    block_partials<2>(v, partials + q * nbq + sb, N * nbq);
 }
 
 // Even-odd operator (Dhat on the even sites): each stencil is two launches, the odd
@@ -226,9 +225,9 @@ __device__ inline void cg_eo_step(const float4 *__restrict__ X, const float4 *__
                                   float4 *O, const float4 *__restrict__ links, const Geom &gf, const SlabWalk &w,
                                   float kappa2, int N, const CgFusedState *__restrict__ st,
                                   double *__restrict__ partials) {
-    const int q = blockIdx.x % N;
-    int c0, nb;
-    slab_block(w, blockIdx.x / N, c0, nb);
+    int q, sb, c0, nb;
+    slab_rhs(w, blockIdx.x, q, sb);
+    slab_block(w, sb, c0, nb);
     const int cb = c0 + threadIdx.x;
     const int Vh = gf.V >> 1;
     const size_t base = (size_t)q * 6 * Vh;
@@ -243,8 +242,7 @@ __device__ inline void cg_eo_step(const float4 *__restrict__ X, const float4 *__
         wilson_eo_schur_site<float, DAG, DAG>(cb, gf, kappa2, X + base, M + base, links, o);
         v[0] = step_update<DAG>(A, O, base, Vh, cb, c, o);
     }
-    const int nbq = gridDim.x / N;
-    block_partials<1>(v, partials + (size_t)q * nbq + blockIdx.x / N, 0);
+    block_partials<1>(v, partials + (size_t)q * w.dN.div(gridDim.x) + sb, 0);
 }
 __global__ void __launch_bounds__(kT, 6)
 k_cg_eo_k1b(const float4 *__restrict__ R, const float4 *__restrict__ M, float4 *T, const float4 *__restrict__ links,

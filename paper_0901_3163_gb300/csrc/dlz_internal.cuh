@@ -21,6 +21,7 @@
 #include <vector>
 
 #include "../../include/dlz.h"
+#include "fast_div.cuh"
 
 namespace dlz {
 
@@ -71,7 +72,29 @@ struct Geom {
     int L[4];      // Lx, Ly, Lz, Lt
     int V;         // sites
     int bc_t;      // +1 periodic, -1 antiperiodic time
+    FastDiv dL[3]; // divisors Lx, Ly, Lz of device code (set_divisors)
+    void set_divisors() {
+        for (int i = 0; i < 3; ++i) dL[i] = FastDiv((unsigned)L[i]);
+    }
 };
+// coordinates of site s
+__host__ __device__ inline void site_coords(const Geom &g, int s, int (&c)[4]) {
+#if defined(__CUDA_ARCH__)
+    int r = s;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const int n = g.dL[i].div(r);
+        c[i] = r - n * g.L[i];
+        r = n;
+    }
+    c[3] = r;
+#else
+    c[0] = s % g.L[0];
+    c[1] = s / g.L[0] % g.L[1];
+    c[2] = s / g.L[0] / g.L[1] % g.L[2];
+    c[3] = s / g.L[0] / g.L[1] / g.L[2];
+#endif
+}
 
 // ---------------------------------------------------------------- errors
 struct Error {

@@ -44,9 +44,9 @@ __global__ void __launch_bounds__(kThreads, 7)
 k_minres_k1(const float4 *__restrict__ Ub, const float4 *__restrict__ Up, float4 *__restrict__ W,
             const float4 *__restrict__ links, Geom g, SlabWalk w, float kappa, int N,
             FusedState *__restrict__ st, double *__restrict__ partials, unsigned *__restrict__ counters) {
-    const int q = blockIdx.x % N;
-    int s0, nb;
-    slab_block(w, blockIdx.x / N, s0, nb);
+    int q, sb, s0, nb;
+    slab_rhs(w, blockIdx.x, q, sb);
+    slab_block(w, sb, s0, nb);
     const int s = s0 + threadIdx.x;
     const size_t base = (size_t)q * 6 * g.V;
     float facc = 0.f;
@@ -54,13 +54,13 @@ k_minres_k1(const float4 *__restrict__ Ub, const float4 *__restrict__ Up, float4
         facc = minres_k1_site(s, g, kappa, Ub + base, Up + base, W + base, links, st[q]);
     // block partials of alpha_q; with counters, the last block of q to finish forms
     // alpha_q (one right-hand side: saves a launch); without, k_minres_alpha does
-    const int nbq = gridDim.x / N;
+    const int nbq = w.dN.div(gridDim.x);
     if (!counters) {
-        block_partial_store<kThreads>(facc, partials + (size_t)q * nbq + blockIdx.x / N);
+        block_partial_store<kThreads>(facc, partials + (size_t)q * nbq + sb);
         return;
     }
     double a;
-    if (partial_then_last_sum<kThreads>(facc, partials + (size_t)q * nbq, blockIdx.x / N, nbq, counters + q, &a) &&
+    if (partial_then_last_sum<kThreads>(facc, partials + (size_t)q * nbq, sb, nbq, counters + q, &a) &&
         threadIdx.x == 0)
         fused_alpha(st[q], a);
 }

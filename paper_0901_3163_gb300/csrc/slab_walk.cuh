@@ -21,6 +21,8 @@
 #include <algorithm>
 #include <cstdlib>
 
+#include "fast_div.cuh"
+
 namespace dlz {
 
 constexpr int kSlabBlock = 128;     // sites per block
@@ -30,13 +32,20 @@ struct SlabWalk {
     int bps;         // blocks per slab
     int plane;       // sites per plane
     int Lz, Lt;
+    FastDiv dbps, dLt, dN;   // divisors: bps, Lt and the right-hand sides of the launch
 };
+
+// the right-hand side q and site block sb of a launch with right-hand sides fastest
+__device__ inline void slab_rhs(const SlabWalk &w, int block, int &q, int &sb) {
+    sb = w.dN.div(block);
+    q = block - sb * (int)w.dN.d;
+}
 
 // first site s0 and site count nb of site block sb (nb = 0 for the spare blocks of a
 // short last z-slab)
 __host__ __device__ inline void slab_block(const SlabWalk &w, int sb, int &s0, int &nb) {
-    const int j = sb / w.bps, off = (sb % w.bps) * kSlabBlock;
-    const int t = j % w.Lt, z0 = (j / w.Lt) * w.bz;
+    const int j = w.dbps.div(sb), off = (sb - j * w.bps) * kSlabBlock;
+    const int zs = w.dLt.div(j), t = j - zs * w.Lt, z0 = zs * w.bz;
     const int planes = w.bz < w.Lz - z0 ? w.bz : w.Lz - z0;
     const int len = planes * w.plane;
     s0 = (t * w.Lz + z0) * w.plane + off;
@@ -44,14 +53,17 @@ __host__ __device__ inline void slab_block(const SlabWalk &w, int sb, int &s0, i
     nb = rest <= 0 ? 0 : (rest < kSlabBlock ? rest : kSlabBlock);
 }
 
-// The walk with slabs of bz planes
-inline SlabWalk slab_walk_of(int plane, int Lz, int Lt, int bz) {
+// The walk with slabs of bz planes, for N right-hand sides
+inline SlabWalk slab_walk_of(int plane, int Lz, int Lt, int bz, int N = 1) {
     SlabWalk w;
     w.plane = plane;
     w.Lz = Lz;
     w.Lt = Lt;
     w.bz = std::max(1, std::min(bz, Lz));
     w.bps = (w.bz * plane + kSlabBlock - 1) / kSlabBlock;
+    w.dbps = FastDiv((unsigned)w.bps);
+    w.dLt = FastDiv((unsigned)Lt);
+    w.dN = FastDiv((unsigned)(N > 0 ? N : 1));
     return w;
 }
 
@@ -71,7 +83,7 @@ inline SlabWalk make_slab_walk(int plane, int Lz, int Lt, int N, double bytes) {
         const int v = std::atoi(env);
         if (v > 0) bz = v;
     }
-    return slab_walk_of(plane, Lz, Lt, bz);
+    return slab_walk_of(plane, Lz, Lt, bz, N);
 }
 
 // blocks per right-hand side

@@ -61,9 +61,9 @@ template <bool G5IN, bool G5OUT>
 __global__ void __launch_bounds__(kSlabBlock, 6)
 k_wilson_batch32(float4 *__restrict__ out, const float4 *__restrict__ in, const float4 *__restrict__ U, Geom g,
                  SlabWalk w, float kappa, int nrhs, long nel) {
-    const int r = blockIdx.x % nrhs;
-    int s0, nb;
-    slab_block(w, blockIdx.x / nrhs, s0, nb);
+    int r, sb, s0, nb;
+    slab_rhs(w, blockIdx.x, r, sb);
+    slab_block(w, sb, s0, nb);
     if (threadIdx.x == 0 && nb > 0) {
         prefetch_planes_l2(in + (size_t)r * nel, 6, g.V, s0, nb);
         if (r == 0) prefetch_planes_l2(U, 12, g.V, s0, nb);
@@ -180,12 +180,12 @@ __global__ void __launch_bounds__(BT, sizeof(T) == 4 ? 768 / BT : 1)
 k_wilson_user(typename Field<T>::vec *__restrict__ out, const typename Field<T>::vec *__restrict__ in,
               const typename Link<T>::vec *__restrict__ U, Geom g, SlabWalk w, T kappa, int nrhs) {
     __shared__ typename Field<T>::vec sm[UOUT ? BT * UserRow<T>::RS : 1];
-    const int r = blockIdx.x % nrhs;
-    int s0, nb;
+    int r, sb, s0, nb;
+    slab_rhs(w, blockIdx.x, r, sb);
     if (BT == kSlabBlock) {
-        slab_block(w, blockIdx.x / nrhs, s0, nb);
+        slab_block(w, sb, s0, nb);
     } else {
-        s0 = (blockIdx.x / nrhs) * BT;
+        s0 = sb * BT;
         nb = min(BT, g.V - s0);
     }
     const typename Field<T>::vec *inr = in + (size_t)r * UserRow<T>::W * g.V;
@@ -235,7 +235,7 @@ void launch_user_bt(Op &op, typename Field<T>::vec *out, const typename Field<T>
                     const typename Link<T>::vec *U, int which, int nrhs) {
     const Geom &g = op.g;
     const SlabWalk w = sizeof(T) == 4 ? make_slab_walk(g.L[0] * g.L[1], g.L[2], g.L[3], nrhs, 200.0)
-                                      : slab_walk_of(g.L[0] * g.L[1], g.L[2], g.L[3], g.L[2]);
+                                      : slab_walk_of(g.L[0] * g.L[1], g.L[2], g.L[3], g.L[2], nrhs);
     const unsigned blocks = (unsigned)((BT == kSlabBlock ? slab_blocks(w) : (long)(g.V + BT - 1) / BT) * nrhs);
     const T kappa = (T)op.kappa;
     switch (which) {

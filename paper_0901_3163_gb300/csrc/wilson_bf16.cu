@@ -43,14 +43,14 @@ __device__ inline void hop_pair_bf(int s, const int (&c)[4], const Geom &g, int 
                                    const float4 *__restrict__ U, float2 (&acc)[12]) {
     const int L = g.L[MU];
     const int sf = (c[MU] == L - 1) ? s - (L - 1) * stride : s + stride;
-    const float phf = (MU == 3 && c[3] == L - 1) ? (float)g.bc_t : 1.f;
+    const bool phf = MU == 3 && c[3] == L - 1 && g.bc_t < 0;
     const int sb = (c[MU] == 0) ? s + (L - 1) * stride : s - stride;
-    const float phb = (MU == 3 && c[3] == 0) ? (float)g.bc_t : 1.f;
+    const bool phb = MU == 3 && c[3] == 0 && g.bc_t < 0;
     float2 p[12], u[9];
     bf_load(in, g.V, sf, p);
     maybe_g5<G5IN>(p);
     load_link<float>(U, g.V, MU, s, u);
-    hop_fwd<float, MU>(p, u, phf, acc);
+    hop_fwd<float, MU, MU == 0>(p, u, phf, acc);
     bf_load(in, g.V, sb, p);
     maybe_g5<G5IN>(p);
     load_link<float>(U, g.V, MU, sb, u);
@@ -73,8 +73,6 @@ k_wilson_bf16_batch(uint2 *__restrict__ out, const uint2 *__restrict__ in, const
     c[3] = t / g.L[2];
     const int st1 = g.L[0], st2 = g.L[0] * g.L[1], st3 = st2 * g.L[2];
     float2 acc[12], o[12];
-#pragma unroll
-    for (int a = 0; a < 12; ++a) acc[a] = make_float2(0.f, 0.f);
     hop_pair_bf<0, G5IN>(s, c, g, 1, inr, U, acc);
     hop_pair_bf<1, G5IN>(s, c, g, st1, inr, U, acc);
     hop_pair_bf<2, G5IN>(s, c, g, st2, inr, U, acc);

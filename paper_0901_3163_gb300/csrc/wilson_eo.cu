@@ -24,7 +24,7 @@ constexpr int kEoThreads = kSlabBlock;
 // side: slab_walk.cuh in FP32, the plain order in FP64 (FP64-ALU-bound kernels)
 SlabWalk eo_walk(const Geom &gf, int nrhs, double bytes, bool f32) {
     const int plane = gf.L[0] * gf.L[1] / 2;
-    return f32 ? make_slab_walk(plane, gf.L[2], gf.L[3], nrhs, bytes) : slab_walk_of(plane, gf.L[2], gf.L[3], gf.L[2]);
+    return f32 ? make_slab_walk(plane, gf.L[2], gf.L[3], nrhs, bytes) : slab_walk_of(plane, gf.L[2], gf.L[3], gf.L[2], nrhs);
 }
 
 // out (parity par) = H [gamma5]^G5IN in (parity 1 - par), nrhs fields; RHS fastest in
@@ -33,9 +33,9 @@ template <typename T, bool G5IN>
 __global__ void __launch_bounds__(kEoThreads)
 k_eo_hop(typename Field<T>::vec *__restrict__ out, const typename Field<T>::vec *__restrict__ in,
          const typename Link<T>::vec *__restrict__ U, Geom gf, SlabWalk w, int par, int nrhs, long nel) {
-    const int r = blockIdx.x % nrhs;
-    int c0, nb;
-    slab_block(w, blockIdx.x / nrhs, c0, nb);
+    int r, sb, c0, nb;
+    slab_rhs(w, blockIdx.x, r, sb);
+    slab_block(w, sb, c0, nb);
     if ((int)threadIdx.x >= nb) return;
     const int cb = c0 + threadIdx.x;
     cx<T> acc[12];
@@ -49,9 +49,9 @@ __global__ void __launch_bounds__(kEoThreads)
 k_eo_schur(typename Field<T>::vec *__restrict__ out, const typename Field<T>::vec *__restrict__ x,
            const typename Field<T>::vec *__restrict__ t, const typename Link<T>::vec *__restrict__ U, Geom gf,
            SlabWalk w, T kappa2, int nrhs, long nel) {
-    const int r = blockIdx.x % nrhs;
-    int c0, nb;
-    slab_block(w, blockIdx.x / nrhs, c0, nb);
+    int r, sb, c0, nb;
+    slab_rhs(w, blockIdx.x, r, sb);
+    slab_block(w, sb, c0, nb);
     if ((int)threadIdx.x >= nb) return;
     const int cb = c0 + threadIdx.x;
     cx<T> o[12];

@@ -17,14 +17,8 @@ namespace dlz {
 
 // Full coordinates c and index of the site with checkerboard index cb and parity par.
 __host__ __device__ inline int eo_site(int cb, int par, const Geom &g, int (&c)[4]) {
-    const int lxh = g.L[0] >> 1;
-    int r = cb / lxh;
-    const int xh = cb - r * lxh;
-    c[1] = r % g.L[1];
-    r /= g.L[1];
-    c[2] = r % g.L[2];
-    c[3] = r / g.L[2];
-    c[0] = 2 * xh + ((c[1] + c[2] + c[3] + par) & 1);
+    site_coords(g, 2 * cb, c);                  // (the pair of sites 2 cb, 2 cb + 1: x is even)
+    c[0] += (c[1] + c[2] + c[3] + par) & 1;
     return ((c[3] * g.L[2] + c[2]) * g.L[1] + c[1]) * g.L[0] + c[0];
 }
 
@@ -37,14 +31,14 @@ __host__ __device__ inline void hop_pair_eo(int s, const int (&c)[4], const Geom
     const int L = g.L[MU];
     const int Vh = g.V >> 1;
     const int sf = (c[MU] == L - 1) ? s - (L - 1) * stride : s + stride;
-    const T phf = (MU == 3 && c[3] == L - 1) ? (T)g.bc_t : (T)1;
+    const bool phf = MU == 3 && c[3] == L - 1 && g.bc_t < 0;
     const int sb = (c[MU] == 0) ? s + (L - 1) * stride : s - stride;
-    const T phb = (MU == 3 && c[3] == 0) ? (T)g.bc_t : (T)1;
+    const bool phb = MU == 3 && c[3] == 0 && g.bc_t < 0;
     cx<T> p[12], u[9];
     Field<T>::load(in, Vh, sf >> 1, p);
     maybe_g5<G5IN>(p);
     load_link<T>(U, g.V, MU, s, u);
-    hop_fwd<T, MU>(p, u, phf, acc);
+    hop_fwd<T, MU, MU == 0>(p, u, phf, acc);
     Field<T>::load(in, Vh, sb >> 1, p);
     maybe_g5<G5IN>(p);
     load_link<T>(U, g.V, MU, sb, u);
@@ -61,8 +55,6 @@ __host__ __device__ inline void wilson_eo_hop_site(int cb, int par, const Geom &
     int c[4];
     const int s = eo_site(cb, par, g, c);
     const int st1 = g.L[0], st2 = g.L[0] * g.L[1], st3 = st2 * g.L[2];
-#pragma unroll
-    for (int a = 0; a < 12; ++a) acc[a] = mk<T>(0, 0);
     hop_pair_eo<T, 0, G5IN>(s, c, g, 1, in, U, acc);
     hop_pair_eo<T, 1, G5IN>(s, c, g, st1, in, U, acc);
     hop_pair_eo<T, 2, G5IN>(s, c, g, st2, in, U, acc);

@@ -24,6 +24,20 @@
 
 namespace dlz {
 
+// Element s of plane c of a field with V elements of 16 bytes per plane: the plane's base is the
+// same for all threads, so that the address is a 32-bit offset from a uniform register (V is
+// below 2^28: 12 V fits in an int).
+template <typename E> __host__ __device__ inline const E &plane_at(const E *p, int c, int V, int s) {
+#if defined(__CUDA_ARCH__)
+    return *reinterpret_cast<const E *>(reinterpret_cast<const char *>(p + (size_t)c * V) + (unsigned)s * 16u);
+#else
+    return p[(size_t)c * V + s];
+#endif
+}
+template <typename E> __host__ __device__ inline E &plane_at(E *p, int c, int V, int s) {
+    return const_cast<E &>(plane_at(static_cast<const E *>(p), c, V, s));
+}
+
 template <typename T> struct Field;
 template <> struct Field<double> {
     typedef double2 vec;
@@ -31,12 +45,12 @@ template <> struct Field<double> {
     __host__ __device__ static inline void load(const double2 *__restrict__ p, int V, int s,
                                                 double2 (&v)[12]) {
 #pragma unroll
-        for (int a = 0; a < 12; ++a) v[a] = p[(size_t)a * V + s];
+        for (int a = 0; a < 12; ++a) v[a] = plane_at(p, a, V, s);
     }
     __host__ __device__ static inline void store(double2 *__restrict__ p, int V, int s,
                                                  const double2 (&v)[12]) {
 #pragma unroll
-        for (int a = 0; a < 12; ++a) p[(size_t)a * V + s] = v[a];
+        for (int a = 0; a < 12; ++a) plane_at(p, a, V, s) = v[a];
     }
 };
 template <> struct Field<float> {
@@ -46,7 +60,7 @@ template <> struct Field<float> {
                                                 float2 (&v)[12]) {
 #pragma unroll
         for (int c = 0; c < 6; ++c) {
-            float4 q = p[(size_t)c * V + s];
+            float4 q = plane_at(p, c, V, s);
             v[2 * c] = make_float2(q.x, q.y);
             v[2 * c + 1] = make_float2(q.z, q.w);
         }
@@ -55,7 +69,7 @@ template <> struct Field<float> {
                                                  const float2 (&v)[12]) {
 #pragma unroll
         for (int c = 0; c < 6; ++c)
-            p[(size_t)c * V + s] = make_float4(v[2 * c].x, v[2 * c].y, v[2 * c + 1].x, v[2 * c + 1].y);
+            plane_at(p, c, V, s) = make_float4(v[2 * c].x, v[2 * c].y, v[2 * c + 1].x, v[2 * c + 1].y);
     }
 };
 
@@ -72,7 +86,7 @@ template <> struct Link<double> {
     __host__ __device__ static inline void load(const double2 *__restrict__ U, int V, int mu, int s,
                                                 double2 (&u)[9]) {
 #pragma unroll
-        for (int e = 0; e < 9; ++e) u[e] = U[(size_t)(mu * 9 + e) * V + s];
+        for (int e = 0; e < 9; ++e) u[e] = plane_at(U, mu * 9 + e, V, s);
     }
 };
 template <> struct Link<float> {
@@ -86,9 +100,9 @@ template <> struct Link<float> {
     }
     __host__ __device__ static inline void load(const float4 *__restrict__ U, int V, int mu, int s,
                                                 float2 (&u)[9]) {
-        const float4 q0 = U[(size_t)(mu * 3 + 0) * V + s];
-        const float4 q1 = U[(size_t)(mu * 3 + 1) * V + s];
-        const float4 q2 = U[(size_t)(mu * 3 + 2) * V + s];
+        const float4 q0 = plane_at(U, mu * 3 + 0, V, s);
+        const float4 q1 = plane_at(U, mu * 3 + 1, V, s);
+        const float4 q2 = plane_at(U, mu * 3 + 2, V, s);
         u[0] = make_float2(q0.x, q0.y);
         u[1] = make_float2(q0.z, q0.w);
         u[2] = make_float2(q1.x, q1.y);
@@ -115,9 +129,21 @@ template <typename T> struct PackedLinks {
     __host__ __device__ inline void operator()(int mu, int s, cx<T> (&u)[9]) const { Link<T>::load(U, V, mu, s, u); }
 };
 
-// Accumulate (1 - gamma_mu) U h-projection of p into acc (forward hop).
-template <typename T, int MU>
-__host__ __device__ inline void hop_fwd(const cx<T> (&p)[12], const cx<T> (&u)[9], T sign,
+// -x if neg (the boundary phase of a hop across the antiperiodic time edge) by the sign bit: an
+// FP64 multiplication less per value, of which a site has 24
+__host__ __device__ inline double flip(double x, bool neg) {
+#if defined(__CUDA_ARCH__)
+    return __hiloint2double(__double2hiint(x) ^ (neg ? (int)0x80000000 : 0), __double2loint(x));
+#else
+    return neg ? -x : x;
+#endif
+}
+__host__ __device__ inline float flip(float x, bool neg) { return neg ? -x : x; }
+
+// Accumulate (1 - gamma_mu) U h-projection of p into acc (forward hop); neg: times -1.  FIRST:
+// acc is not read (the first hop of a site starts it, 24 additions of zero less).
+template <typename T, int MU, bool FIRST = false>
+__host__ __device__ inline void hop_fwd(const cx<T> (&p)[12], const cx<T> (&u)[9], bool neg,
                                         cx<T> (&acc)[12]) {
     cx<T> h0[3], h1[3];
 #pragma unroll
@@ -127,7 +153,10 @@ __host__ __device__ inline void hop_fwd(const cx<T> (&p)[12], const cx<T> (&u)[9
         if (MU == 1) { h0[c] = u0 + l1;      h1[c] = u1 - l0; }
         if (MU == 2) { h0[c] = addI(u0, l0); h1[c] = subI(u1, l1); }
         if (MU == 3) { h0[c] = u0 - l0;      h1[c] = u1 - l1; }
-        h0[c].x *= sign; h0[c].y *= sign; h1[c].x *= sign; h1[c].y *= sign;
+        if (MU == 3) {
+            h0[c].x = flip(h0[c].x, neg); h0[c].y = flip(h0[c].y, neg);
+            h1[c].x = flip(h1[c].x, neg); h1[c].y = flip(h1[c].y, neg);
+        }
     }
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
@@ -136,6 +165,14 @@ __host__ __device__ inline void hop_fwd(const cx<T> (&p)[12], const cx<T> (&u)[9
         for (int j = 0; j < 3; ++j) {
             H0 = cfma(u[3 * i + j], h0[j], H0);
             H1 = cfma(u[3 * i + j], h1[j], H1);
+        }
+        if (FIRST) {
+            static_assert(!FIRST || MU == 0, "the first hop is x");
+            acc[i] = H0;
+            acc[3 + i] = H1;
+            acc[6 + i] = mk<T>(H1.y, -H1.x);
+            acc[9 + i] = mk<T>(H0.y, -H0.x);
+            continue;
         }
         acc[i] = acc[i] + H0;
         acc[3 + i] = acc[3 + i] + H1;
@@ -148,7 +185,7 @@ __host__ __device__ inline void hop_fwd(const cx<T> (&p)[12], const cx<T> (&u)[9
 
 // Accumulate (1 + gamma_mu) U^dag h-projection of p into acc (backward hop).
 template <typename T, int MU>
-__host__ __device__ inline void hop_bwd(const cx<T> (&p)[12], const cx<T> (&u)[9], T sign,
+__host__ __device__ inline void hop_bwd(const cx<T> (&p)[12], const cx<T> (&u)[9], bool neg,
                                         cx<T> (&acc)[12]) {
     cx<T> h0[3], h1[3];
 #pragma unroll
@@ -158,7 +195,10 @@ __host__ __device__ inline void hop_bwd(const cx<T> (&p)[12], const cx<T> (&u)[9
         if (MU == 1) { h0[c] = u0 - l1;      h1[c] = u1 + l0; }
         if (MU == 2) { h0[c] = subI(u0, l0); h1[c] = addI(u1, l1); }
         if (MU == 3) { h0[c] = u0 + l0;      h1[c] = u1 + l1; }
-        h0[c].x *= sign; h0[c].y *= sign; h1[c].x *= sign; h1[c].y *= sign;
+        if (MU == 3) {
+            h0[c].x = flip(h0[c].x, neg); h0[c].y = flip(h0[c].y, neg);
+            h1[c].x = flip(h1[c].x, neg); h1[c].y = flip(h1[c].y, neg);
+        }
     }
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
@@ -223,14 +263,14 @@ __host__ __device__ inline void hop_pair(int s, const int (&c)[4], const Geom &g
     // forward neighbour and the boundary phase of a hop across the time edge
     const bool wf = c[MU] == L - 1, wb = c[MU] == 0;
     const int sf = wf ? s - (L - 1) * stride : s + stride;
-    const T phf = (MU == 3 && wf) ? (T)g.bc_t : (T)1;
+    const bool phf = MU == 3 && wf && g.bc_t < 0;
     const int sb = wb ? s + (L - 1) * stride : s - stride;
-    const T phb = (MU == 3 && wb) ? (T)g.bc_t : (T)1;
+    const bool phb = MU == 3 && wb && g.bc_t < 0;
     cx<T> p[12], u[9];
     ld.template get<MU, 1>(sf, wf, p);
     maybe_g5<G5IN>(p);
     lk(MU, s, u);
-    hop_fwd<T, MU>(p, u, phf, acc);
+    hop_fwd<T, MU, MU == 0>(p, u, phf, acc);
     ld.template get<MU, -1>(sb, wb, p);
     maybe_g5<G5IN>(p);
     lk(MU, sb, u);
@@ -243,15 +283,9 @@ template <typename T, bool G5IN, bool G5OUT, class G, class LK>
 __host__ __device__ inline void wilson_site_g(int s, const Geom &g, T kappa, const G &ld, const LK &lk,
                                               cx<T> (&out)[12]) {
     int c[4];
-    int r = s;
-    c[0] = r % g.L[0]; r /= g.L[0];
-    c[1] = r % g.L[1]; r /= g.L[1];
-    c[2] = r % g.L[2];
-    c[3] = r / g.L[2];
+    site_coords(g, s, c);
     const int st1 = g.L[0], st2 = g.L[0] * g.L[1], st3 = st2 * g.L[2];
     cx<T> acc[12];
-#pragma unroll
-    for (int a = 0; a < 12; ++a) acc[a] = mk<T>(0, 0);
     hop_pair<T, 0, G5IN>(s, c, g, 1, ld, lk, acc);
     hop_pair<T, 1, G5IN>(s, c, g, st1, ld, lk, acc);
     hop_pair<T, 2, G5IN>(s, c, g, st2, ld, lk, acc);
