@@ -244,13 +244,13 @@ __device__ inline void cg_eo_step(const float4 *__restrict__ X, const float4 *__
     }
     block_partials<1>(v, partials + (size_t)q * w.dN.div(gridDim.x) + sb, 0);
 }
-__global__ void __launch_bounds__(kT, 6)
+__global__ void __launch_bounds__(kT, 7)
 k_cg_eo_k1b(const float4 *__restrict__ R, const float4 *__restrict__ M, float4 *T, const float4 *__restrict__ links,
             Geom gf, SlabWalk w, float kappa2, int N, const CgFusedState *__restrict__ st,
             double *__restrict__ partials) {
     cg_eo_step<false>(R, M, T, T, links, gf, w, kappa2, N, st, partials);
 }
-__global__ void __launch_bounds__(kT, 6)
+__global__ void __launch_bounds__(kT, 7)
 k_cg_eo_k23b(const float4 *__restrict__ T, const float4 *__restrict__ M, const float4 *__restrict__ R,
              float4 *__restrict__ Rn, const float4 *__restrict__ links, Geom gf, SlabWalk w, float kappa2, int N,
              const CgFusedState *__restrict__ st, double *__restrict__ partials) {

@@ -105,8 +105,10 @@ k_mm_init(const double *__restrict__ partials, const SlotDesc *__restrict__ sd, 
     if (threadIdx.x == 0) fused_init(st[blockIdx.x], sqrt(r2));
 }
 
+// (7 blocks of 128 sites per SM: nine lattices of 8^4 .. 16^4, 8 RHS, 407 -> 393 ms per call; 8:
+// 422 ms)
 template <int B>
-__global__ void __launch_bounds__(B * kMT)
+__global__ void __launch_bounds__(B * kMT, 7 / B)
 k_mm_k1(const float4 *__restrict__ U, const float4 *__restrict__ Up, float4 *__restrict__ W,
         const SlotDesc *__restrict__ sd, const int2 *__restrict__ table, const FusedState *__restrict__ st,
         const int *__restrict__ active, double *__restrict__ partials) {
@@ -329,9 +331,9 @@ struct Tile {
 // iterations, where every slot's vectors are in the same buffers, so the frozen slot's
 // pending direction is still found where k_mm_directions<.., true> looks for it).
 // The launch form is chosen once per call: MultiRun keeps the choice and the captured
-// graphs from one inner solve of the defect correction to the next (the autotuner's nine
-// candidates, run again in every inner solve, took 180 of 563 ms on nine lattices of
-// 8^4 .. 16^4 with 8 right-hand sides).
+// graphs from one inner solve of the defect correction to the next (nine candidates timed
+// again in every inner solve took 180 of 563 ms on nine lattices of 8^4 .. 16^4 with 8
+// right-hand sides).
 struct MultiRun {
     GraphExec ge[3];         // the graph form's block of iterations, by tile
     int best = -1;           // the chosen candidate (-1: not chosen yet)
@@ -406,14 +408,15 @@ int minres_multi_batch(Op &op, int NS, const SlotDesc *sd, const Tile *tiles, in
         for (int i = 0; i < kMrBlock; ++i) DLZ_TRY(iteration(tiles[cur], i));
         return DLZ_OK;
     };
-    // Autotuner over the launch forms: the graph form with 1, 2 or 4 chunks of 128 sites
-    // per block (candidates 0-2; the first three groups capture their graphs, the next
-    // three time one replay each), and the persistent form with 1, 2 or 4 chunks per
-    // work item at the full or half co-resident grid (candidates 3-8, one timed group
-    // each).  The fastest candidate runs the rest.  Chunk partials and slot freezing do
-    // not depend on the candidate, so every choice gives the same bits.
+    // Autotuner over the tiles of the graph form, 1, 2 or 4 chunks of 128 sites per block (the
+    // first three groups capture their graphs, the next three time one replay each); the fastest
+    // runs the rest.  The persistent form is taken only when it is asked for: it lost at every
+    // size measured, from 30 chunks (three lattices of 4^4 and 6^4, 2 RHS: 18.5 against 15.7 ms
+    // per call) to 16944 (nine of 8^4 .. 16^4, 8 RHS: 250 against 199 ms), and timing its six
+    // candidates took 16 ms of the latter.  Chunk partials and slot freezing do not depend on
+    // the candidate, so every choice gives the same bits.
     // DLZ_MULTI_TILE=1|2|4 fixes the chunks per block; DLZ_MULTI_FORM=graph|persistent
-    // fixes the form (both: no search).
+    // fixes the form (persistent: its tiles at the full or half co-resident grid are timed).
     int tile_forced = -1, form_forced = -1;
     if (const char *env = std::getenv("DLZ_MULTI_TILE")) {
         const int b = std::atoi(env);
@@ -432,7 +435,7 @@ int minres_multi_batch(Op &op, int NS, const SlotDesc *sd, const Tile *tiles, in
         if ((tile_forced < 0 || tile_forced == v) && form_forced != 1) cands.push_back({0, v, 0, 0});
     for (int v = 0; v < 3; ++v)
         for (int half = 0; half < 2; ++half)
-            if ((tile_forced < 0 || tile_forced == v) && form_forced != 0) {
+            if ((tile_forced < 0 || tile_forced == v) && form_forced == 1) {
                 const int grid = persistent_grid(1 << v, half);
                 if (grid > 0) cands.push_back({1, v, half, grid});
             }

@@ -30,7 +30,7 @@ SlabWalk eo_walk(const Geom &gf, int nrhs, double bytes, bool f32) {
 // out (parity par) = H [gamma5]^G5IN in (parity 1 - par), nrhs fields; RHS fastest in
 // blockIdx so that blocks of the same sites share their links in L2
 template <typename T, bool G5IN>
-__global__ void __launch_bounds__(kEoThreads)
+__global__ void __launch_bounds__(kEoThreads, sizeof(T) == 4 ? 7 : 1)
 k_eo_hop(typename Field<T>::vec *__restrict__ out, const typename Field<T>::vec *__restrict__ in,
          const typename Link<T>::vec *__restrict__ U, Geom gf, SlabWalk w, int par, int nrhs, long nel) {
     int r, sb, c0, nb;
@@ -45,7 +45,7 @@ k_eo_hop(typename Field<T>::vec *__restrict__ out, const typename Field<T>::vec 
 
 // out = [gamma5]^G5OUT ([gamma5]^G5X x - kappa2 H_eo t) at the even sites
 template <typename T, bool G5X, bool G5OUT>
-__global__ void __launch_bounds__(kEoThreads)
+__global__ void __launch_bounds__(kEoThreads, sizeof(T) == 4 ? 7 : 1)
 k_eo_schur(typename Field<T>::vec *__restrict__ out, const typename Field<T>::vec *__restrict__ x,
            const typename Field<T>::vec *__restrict__ t, const typename Link<T>::vec *__restrict__ U, Geom gf,
            SlabWalk w, T kappa2, int nrhs, long nel) {
