@@ -185,6 +185,69 @@ k_lanczos_k2a(float4 *__restrict__ W, const float4 *__restrict__ Vj, const float
     }
 }
 
+// Block partials that the fused kernels of a step write (the counter sits after them): 6 V
+// elements in k_reorth_norm, two kernels of V sites in lanczos_fused_step
+inline long lz_partials(int V) { return std::max((6L * V + kLz - 1) / kLz, 2L * ((V + kLz - 1) / kLz)); }
+
+// The stencil of an unfused FP32 step with the three-term subtraction: W = Q in - beta_{j-1}
+// v_{j-1} (Vp null: none) and alpha_j = Re <v_j, W> by the last block, which saves a pass over
+// three vectors.  Bound by the gathers of a single vector.  With k_reorth_norm, Lan-DR(100, 40)
+// and D-CG on 4 right-hand sides of 16^3 x 32 take 385.3 ms in place of 393.1.
+__global__ void __launch_bounds__(kLz, 7)
+k_lanczos_apply(const float4 *__restrict__ in, const float4 *__restrict__ Vj, const float4 *__restrict__ Vp,
+                const float *__restrict__ bprev, float4 *__restrict__ W, const float4 *__restrict__ links, Geom g,
+                float kappa, double *__restrict__ partials, unsigned *__restrict__ counter, double *__restrict__ d_a,
+                float *__restrict__ s_a) {
+    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    float facc = 0.f;
+    if (s < g.V) {
+        float2 o[12];
+        wilson_site<float, false, true>(s, g, kappa, in, links, o);
+        const float bt = Vp ? *bprev : 0.f;
+#pragma unroll
+        for (int c = 0; c < 6; ++c) {
+            const size_t i = (size_t)c * g.V + s;
+            float4 w = make_float4(o[2 * c].x, o[2 * c].y, o[2 * c + 1].x, o[2 * c + 1].y);
+            if (Vp) w = P32::axpy(-bt, Vp[i], w);
+            W[i] = w;
+            facc += P32::rdot(Vj[i], w);
+        }
+    }
+    double a;
+    if (partial_then_last_sum<kLz>(facc, partials, blockIdx.x, gridDim.x, counter, &a) && threadIdx.x == 0) {
+        *d_a = a;
+        *s_a = (float)a;
+    }
+}
+
+// The end of a re-orthogonalised FP32 step: W += sum_l c_l V_l (complex c_l, l < nv), and
+// beta_{j+1} = ||W|| by the last block (the combine kernel and a reduction in one pass)
+__global__ void __launch_bounds__(kLz)
+k_reorth_norm(float4 *__restrict__ W, const float4 *__restrict__ V, long ld, int nv, const double2 *__restrict__ coef,
+              long n, double *__restrict__ partials, unsigned *__restrict__ counter, double *__restrict__ d_b,
+              float *__restrict__ s_b, float *__restrict__ s_ib) {
+    extern __shared__ float2 cs[];
+    for (int t = threadIdx.x; t < nv; t += kLz) cs[t] = make_float2((float)coef[t].x, (float)coef[t].y);
+    __syncthreads();
+    const long i = (long)blockIdx.x * kLz + threadIdx.x;
+    float facc = 0.f;
+    if (i < n) {
+        float4 a = P32::zero();
+#pragma unroll 8
+        for (int l = 0; l < nv; ++l) P32::cacc(cs[l], V[(size_t)l * ld + i], a);
+        const float4 w = P32::add(W[i], a);
+        W[i] = w;
+        facc = P32::nrm(w);
+    }
+    double r2;
+    if (partial_then_last_sum<kLz>(facc, partials, blockIdx.x, gridDim.x, counter, &r2) && threadIdx.x == 0) {
+        const double b = sqrt(r2);
+        *d_b = b;
+        *s_b = (float)b;
+        *s_ib = (float)(1.0 / b);
+    }
+}
+
 // one fused FP32 Lanczos step (see above)
 int lanczos_fused_step(Op &op, bool ddagd, const float4 *u, const float *s_ib_prev, const float4 *vp,
                        const float *s_b_prev, float4 *vj, float4 *w_out, float4 *tmp, double *partials,
@@ -197,7 +260,7 @@ int lanczos_fused_step(Op &op, bool ddagd, const float4 *u, const float *s_ib_pr
         in = tmp;
     }
     op.prof.stencil_start(op.stream, true, g.V, 1, 96, 1);
-    unsigned *counter = reinterpret_cast<unsigned *>(partials + 2 * blocks);
+    unsigned *counter = reinterpret_cast<unsigned *>(partials + lz_partials(g.V));
     k_lanczos_k1<<<blocks, kLz, 0, op.stream>>>(in, s_ib_prev, u, vp, s_b_prev, vj, w_out, op.gauge32.as<float4>(),
                                                 g, (float)op.kappa, partials, counter, d_a, s_a);
     op.prof.stencil_stop(op.stream);
@@ -227,7 +290,7 @@ int dr_solve_t(Op &op, bool harmonic, const double2 *b_in, double2 *x_out, const
     if (P::kF32) {
         DLZ_TRY(reserve_multidot(op, k));
         DLZ_TRY(w2.alloc(n * sizeof(E)));
-        DLZ_TRY(fpart.alloc((size_t)2 * ((op.g.V + 127) / 128 + 1) * sizeof(double) + 64));
+        DLZ_TRY(fpart.alloc((lz_partials(op.g.V) + 8) * sizeof(double)));
         DLZ_CUDA_TRY(cudaMemsetAsync(fpart.p, 0, fpart.bytes, op.stream));
     }
     DLZ_TRY(bb.alloc(n64 * sizeof(double2)));
@@ -328,6 +391,37 @@ int dr_solve_t(Op &op, bool harmonic, const double2 *b_in, double2 *x_out, const
                 }
             }
             E *vj = V + (size_t)j * n, *wv = ucur;
+            if constexpr (P::kF32) {
+                // a re-orthogonalised step (Lan-DR: every step) in five passes; the coefficients of
+                // more than 6000 kept vectors don't fit in k_reorth_norm's 48 KB
+                if (reorth_j && j > j0 && !op.eo && j0 <= 6000) {
+                    const float4 *in = vj;
+                    if (!harmonic) {
+                        DLZ_TRY(wilson32(op, tmp.as<E>(), vj, DLZ_Q));
+                        in = tmp.as<E>();
+                    }
+                    const unsigned nb = (unsigned)((op.g.V + kLz - 1) / kLz), nb2 = (unsigned)((n + kLz - 1) / kLz);
+                    double *part = fpart.as<double>();
+                    unsigned *counter = reinterpret_cast<unsigned *>(part + lz_partials(op.g.V));
+                    op.prof.stencil_start(op.stream, true, op.g.V, 1, 96, 1);
+                    k_lanczos_apply<<<nb, kLz, 0, op.stream>>>(in, vj, V + (size_t)(j - 1) * n, s_beta + (j - 1), wv,
+                                                               op.gauge32.as<float4>(), op.g, (float)op.kappa, part,
+                                                               counter, d_alpha + j, s_alpha + j);
+                    op.prof.stencil_stop(op.stream);
+                    const S *saj = s_alpha + j, *sib = s_invbeta + j;
+                    DLZ_TRY(map(op, n, [=] __device__(long i) { wv[i] = P::axpy(-*saj, vj[i], wv[i]); }));
+                    double2 *cd = coef.as<double2>() + (m + 1);   // after the coupling block
+                    DLZ_TRY(multidot<P>(op, V, n, j0, wv, cd, -1.0));
+                    k_reorth_norm<<<nb2, kLz, j0 * sizeof(float2), op.stream>>>(wv, V, n, j0, cd, n, part, counter,
+                                                                               d_beta + j, s_beta + j, s_invbeta + j);
+                    op.prof.launches += 2;
+                    DLZ_CUDA_TRY(cudaGetLastError());
+                    E *vn = V + (size_t)(j + 1) * n;
+                    DLZ_TRY(map(op, n, [=] __device__(long i) { vn[i] = P::scal(*sib, wv[i]); }));
+                    vmat = true;
+                    continue;
+                }
+            }
             DLZ_TRY(P::apply(op, wv, vj, which, tmp.as<E>()));
             if (j == j0 && j0 > 0) DLZ_TRY(combine<P>(op, wv, n, 1, V, n, j0, coefr, 1, true, true));
             const E *vprev = (j > j0) ? V + (size_t)(j - 1) * n : nullptr;
