@@ -17,10 +17,11 @@ struct FastDiv {
     }
     __host__ __device__ inline int div(int n) const {
 #if defined(__CUDA_ARCH__)
-        return (int)((__umulhi(m, (unsigned)n) + (unsigned)n) >> s);
+        const unsigned hi = __umulhi(m, (unsigned)n);
 #else
-        return (int)((unsigned)n / d);
+        const unsigned hi = (unsigned)(((unsigned long long)m * (unsigned)n) >> 32);
 #endif
+        return (int)((hi + (unsigned)n) >> s);
     }
 };
 
