@@ -288,14 +288,13 @@ def run_ours(args):
     value = solved_all / (ms_max / 1e3)
     peaks, src = _peaks()
     roof = kernel_roofline(pst, 1, peaks, src,
-                           "k_cg_k1 (fused FP32 CGNR: r gathered, t = D r + beta t, p = r + beta p, "
-                           "e += alpha p_old; 16 RHS per launch)",
+                           "k_cg_k1 (fused FP32 CGNR: r gathered, t = D r + beta t; 16 RHS per launch)",
                            args.k1_traffic,
                            "ncu capture of the current kernel, one launch at this size "
                            "(summary under profiles/)" if args.k1_traffic else
                            "not captured for the current kernel")
     roof_k23 = kernel_roofline(pst, 2, peaks, src,
-                               "k_cg_k23 (fused FP32 CGNR: t gathered, r -= alpha D^dag t; 16 RHS per launch)")
+                               "k_cg_k23 (fused FP32 CGNR: t gathered, r' = r - alpha D^dag t; 16 RHS per launch)")
     it_ms = sum(s.kernel_ms[1] + s.kernel_ms[2] for s in pst)
     it_b = sum(s.kernel_bytes[1] + s.kernel_bytes[2] for s in pst)
     # end to end: host (pinned) buffers through the C ABI, copies inside the timed region

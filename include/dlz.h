@@ -46,7 +46,8 @@
  *                     sites per block or per work item) instead of choosing it by
  *                     timing; every tile gives the same bits;
  *   DLZ_MULTI_FORM=graph|persistent  fix the launch form of dlz_batch_dminres
- *                     (see dlz_batch_last_choice); both forms give the same bits;
+ *                     (see dlz_batch_last_choice; default graph, the faster one at every
+ *                     measured size); both forms give the same bits;
  *   DLZ_WAIT_LIMIT=n  polls before a grid-barrier wait of the persistent form gives up
  *                     (default 2^24, about a second); a test hook for the timeout path;
  *   DLZ_SLAB=n        z-planes per slab of the block walk of the batched FP32 stencils
@@ -240,7 +241,8 @@ int dlz_apply(dlz_op_t op, int which, const void *in, void *out, int dtype, int 
  * allocate device memory at the point of the call: a caller whose memory pool
  * already holds the device's free memory (cudaMalloc would fail), or one that
  * keeps other streams busy and cannot afford the device-wide synchronisation
- * of the cudaFree that dlz_apply's temporary buffers end with.
+ * of a cudaFree (dlz_apply keeps up to 4 work buffers of 64 MiB with the operator and
+ * frees larger ones before it returns).
  *
  * Same operation, arguments and layout as dlz_apply (dtype DLZ_F64 or DLZ_F32
  * only), except: in and out must

@@ -18,8 +18,12 @@
 // side an iteration moves 72 (K1) + 72 (K23) + 40 (240 / 6: six r and p, e read; p, e
 // written) = 184 reals, against 240 with p and e updated by K1 in every iteration.
 // Measured on 24^3 x 48 with 16 right-hand sides, a whole D-CG call of 348 iterations:
-// 913 ms with p and e updated in every iteration, 773 ms with blocks.  On 8^4 with 4
-// right-hand sides, where launches bound the iteration, 6.56 and 6.33 ms.
+// 913 ms with p and e updated in every iteration, 773 ms with blocks, 741 ms with fewer
+// instructions per site in the stencil (K1 716, K23 754, the directions 1371 / 6 us per
+// iteration; at the memory rate 577, 577 and 1335 / 6).  K1 and K23 are bound by the gathers:
+// L1 and L2 each two thirds busy, FMA 45 %.  On 8^4 with 4 right-hand sides, where launches
+// bound the iteration, 6.56, 6.33 and 4.6 ms (the last with the work memory of a call kept
+// with the operator).
 // Each kernel writes only vectors it does not gather (and only at its own site).
 // One-block-per-RHS kernels sum the partials in a fixed order and update the step lengths;
 // a block of six iterations is a CUDA graph that is captured once and replayed.

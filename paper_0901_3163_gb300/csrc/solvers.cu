@@ -285,7 +285,8 @@ struct MinresState {
 // The last block of each kernel to finish adds the block partials in a fixed order and writes
 // the scalars.  Both are bound by FP64 arithmetic (about 900 and 170 instructions per site at 2
 // per cycle and SM).  On 12 x 12 x 10 x 22 an iteration of the separate stencil, two reductions
-// and update took 64.7 + 2 x 11.6 + 12.6 us and four launch gaps; the fused one: see dminres64.
+// and update took 64.7 + 2 x 11.6 + 12.6 us and four launch gaps, the fused one 64.3 + 18.3 us:
+// a D-MinRes call on 2 right-hand sides 133 -> 114 ms.
 template <int BT>
 __global__ void __launch_bounds__(BT)
 k_minres64_k1(const double2 *__restrict__ Uc, const double2 *__restrict__ Up, double2 *__restrict__ W,
