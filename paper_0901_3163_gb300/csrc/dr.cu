@@ -185,9 +185,9 @@ k_lanczos_k2a(float4 *__restrict__ W, const float4 *__restrict__ Vj, const float
     }
 }
 
-// Block partials that the fused kernels of a step write (the counter sits after them): 6 V
-// elements in k_reorth_norm, two kernels of V sites in lanczos_fused_step
-inline long lz_partials(int V) { return std::max((6L * V + kLz - 1) / kLz, 2L * ((V + kLz - 1) / kLz)); }
+// Block partials that the fused kernels of a step write (the counter sits after them): at most
+// 6 per chunk of 128 sites (k_reorth_norm has 6 per 256, lanczos_fused_step 2 per 128)
+inline long lz_partials(int V) { return 6L * ((V + kLz - 1) / kLz); }
 
 // The stencil of an unfused FP32 step with the three-term subtraction: W = Q in - beta_{j-1}
 // v_{j-1} (Vp null: none) and alpha_j = Re <v_j, W> by the last block, which saves a pass over
@@ -221,17 +221,25 @@ k_lanczos_apply(const float4 *__restrict__ in, const float4 *__restrict__ Vj, co
 }
 
 // The end of a re-orthogonalised FP32 step: W += sum_l c_l V_l (complex c_l, l < nv), and
-// beta_{j+1} = ||W|| by the last block (the combine kernel and a reduction in one pass)
-__global__ void __launch_bounds__(kLz)
+// beta_{j+1} = ||W|| by the last block (the combine kernel and a reduction in one pass).  A
+// block has one plane of kRn sites, the planes of a chunk of sites follow one another, and the
+// chunks go from the last to the first: the multi-dot before it has just read the last chunks of
+// all vectors, and L2 still holds about a fifth of them (40 vectors of 16^3 x 32: multi-dot and
+// this kernel 201 us with both in the same order and groups of 8 vectors, 173 us so: 94 + 79;
+// Lan-DR(100, 40) and D-CG on 4 right-hand sides 385 -> 358 ms).  Eight
+// loads in flight per thread; 16 take registers that cost more blocks (78 -> 104 us).
+constexpr int kRn = 256;
+__global__ void __launch_bounds__(kRn)
 k_reorth_norm(float4 *__restrict__ W, const float4 *__restrict__ V, long ld, int nv, const double2 *__restrict__ coef,
-              long n, double *__restrict__ partials, unsigned *__restrict__ counter, double *__restrict__ d_b,
+              int sites, double *__restrict__ partials, unsigned *__restrict__ counter, double *__restrict__ d_b,
               float *__restrict__ s_b, float *__restrict__ s_ib) {
     extern __shared__ float2 cs[];
-    for (int t = threadIdx.x; t < nv; t += kLz) cs[t] = make_float2((float)coef[t].x, (float)coef[t].y);
+    for (int t = threadIdx.x; t < nv; t += kRn) cs[t] = make_float2((float)coef[t].x, (float)coef[t].y);
     __syncthreads();
-    const long i = (long)blockIdx.x * kLz + threadIdx.x;
+    const int b = gridDim.x - 1 - blockIdx.x, s = b / 6 * kRn + threadIdx.x;
     float facc = 0.f;
-    if (i < n) {
+    if (s < sites) {
+        const long i = (long)(b % 6) * sites + s;
         float4 a = P32::zero();
 #pragma unroll 8
         for (int l = 0; l < nv; ++l) P32::cacc(cs[l], V[(size_t)l * ld + i], a);
@@ -240,7 +248,7 @@ k_reorth_norm(float4 *__restrict__ W, const float4 *__restrict__ V, long ld, int
         facc = P32::nrm(w);
     }
     double r2;
-    if (partial_then_last_sum<kLz>(facc, partials, blockIdx.x, gridDim.x, counter, &r2) && threadIdx.x == 0) {
+    if (partial_then_last_sum<kRn>(facc, partials, b, gridDim.x, counter, &r2) && threadIdx.x == 0) {
         const double b = sqrt(r2);
         *d_b = b;
         *s_b = (float)b;
@@ -400,7 +408,7 @@ int dr_solve_t(Op &op, bool harmonic, const double2 *b_in, double2 *x_out, const
                         DLZ_TRY(wilson32(op, tmp.as<E>(), vj, DLZ_Q));
                         in = tmp.as<E>();
                     }
-                    const unsigned nb = (unsigned)((op.g.V + kLz - 1) / kLz), nb2 = (unsigned)((n + kLz - 1) / kLz);
+                    const unsigned nb = (unsigned)((op.g.V + kLz - 1) / kLz), nb2 = 6u * (unsigned)((op.g.V + kRn - 1) / kRn);
                     double *part = fpart.as<double>();
                     unsigned *counter = reinterpret_cast<unsigned *>(part + lz_partials(op.g.V));
                     op.prof.stencil_start(op.stream, true, op.g.V, 1, 96, 1);
@@ -412,7 +420,7 @@ int dr_solve_t(Op &op, bool harmonic, const double2 *b_in, double2 *x_out, const
                     DLZ_TRY(map(op, n, [=] __device__(long i) { wv[i] = P::axpy(-*saj, vj[i], wv[i]); }));
                     double2 *cd = coef.as<double2>() + (m + 1);   // after the coupling block
                     DLZ_TRY(multidot<P>(op, V, n, j0, wv, cd, -1.0));
-                    k_reorth_norm<<<nb2, kLz, j0 * sizeof(float2), op.stream>>>(wv, V, n, j0, cd, n, part, counter,
+                    k_reorth_norm<<<nb2, kRn, j0 * sizeof(float2), op.stream>>>(wv, V, n, j0, cd, op.g.V, part, counter,
                                                                                d_beta + j, s_beta + j, s_invbeta + j);
                     op.prof.launches += 2;
                     DLZ_CUDA_TRY(cudaGetLastError());

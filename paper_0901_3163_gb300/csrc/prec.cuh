@@ -155,25 +155,31 @@ inline int combine(Op &op, typename P::E *out, long ld_out, int nout, const type
 }
 
 // ---------------------------------------------------------------- FP32 multi-dot
-// <V_l, w> for l < nv in one pass over the V_l: block (site chunk, group of 8
-// vectors); each thread loads w at its site once and accumulates 8 complex dots
-// over the 6 planes in float; warps and blocks are summed in FP64 (fixed order).
-constexpr int kMdThreads = 128;
-static __global__ void __launch_bounds__(kMdThreads)
-k_multidot32(const float4 *__restrict__ V, long ld, int nv, const float4 *__restrict__ w, int sites,
-             double *__restrict__ partials) {
-    const int grp = blockIdx.y;
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    float re[8], im[8];
+// <V_l, w> for l < nv in one pass over the V_l: block (site chunk, group of kMdVectors
+// vectors, the groups of a chunk one after another); each thread loads w at its site once and
+// accumulates the complex dots over the 6 planes in float; warps and blocks are summed in FP64
+// (fixed order).  Bound by memory.  40 vectors of 16^3 x 32 (0.52 GB): 146 us with a shuffle
+// tree per sum and groups of 8 over all chunks, 111 with halving sums, 92 (5.6 TB/s) with
+// groups of 4, 8 blocks per SM, chunk by chunk; 5 to 7 blocks or groups of 8: 91 to 115, 10 or
+// 12 blocks: over 114.  Chunk by chunk also leaves the last chunks of every vector in L2, where
+// the combination that follows (k_reorth_norm) begins.
+constexpr int kMdThreads = 128, kMdVectors = 4;
+static __global__ void __launch_bounds__(kMdThreads, 8)
+k_multidot32(const float4 *__restrict__ V, long ld, int nv, const float4 *__restrict__ w, int sites, int nblk,
+             FastDiv groups, double *__restrict__ partials) {
+    constexpr int NL = kMdVectors;
+    const int chunk = groups.div(blockIdx.x), grp = blockIdx.x - chunk * groups.d;
+    const int s = chunk * kMdThreads + threadIdx.x;
+    float re[NL], im[NL];
 #pragma unroll
-    for (int l = 0; l < 8; ++l) { re[l] = 0.f; im[l] = 0.f; }
+    for (int l = 0; l < NL; ++l) { re[l] = 0.f; im[l] = 0.f; }
     if (s < sites) {
         float4 x[6];
 #pragma unroll
         for (int c = 0; c < 6; ++c) x[c] = w[(size_t)c * sites + s];
 #pragma unroll
-        for (int l = 0; l < 8; ++l) {
-            const int vi = grp * 8 + l;
+        for (int l = 0; l < NL; ++l) {
+            const int vi = grp * NL + l;
             if (vi < nv) {
                 const float4 *v = V + (size_t)vi * ld;
 #pragma unroll
@@ -185,25 +191,25 @@ k_multidot32(const float4 *__restrict__ V, long ld, int nv, const float4 *__rest
             }
         }
     }
-    __shared__ double sm[16][kMdThreads / 32];
+    __shared__ double sm[2 * NL][kMdThreads / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    double d[16];
+    double d[2 * NL];
 #pragma unroll
-    for (int l = 0; l < 8; ++l) {
+    for (int l = 0; l < NL; ++l) {
         d[2 * l] = (double)re[l];
         d[2 * l + 1] = (double)im[l];
     }
-    const double t = warp_sums<16>(d);
+    const double t = warp_sums<2 * NL>(d);
 #pragma unroll
-    for (int j = 0; j < 16; ++j)
-        if (lane == warp_sum_lane<16>(j)) sm[j][warp] = t;
+    for (int j = 0; j < 2 * NL; ++j)
+        if (lane == warp_sum_lane<2 * NL>(j)) sm[j][warp] = t;
     __syncthreads();
-    if (threadIdx.x < 16) {
+    if (threadIdx.x < 2 * NL) {
         double t = 0.0;
 #pragma unroll
         for (int k = 0; k < kMdThreads / 32; ++k) t += sm[threadIdx.x][k];
-        // partials[(grp*16 + j) * gridDim.x + blockIdx.x]
-        partials[((size_t)grp * 16 + threadIdx.x) * gridDim.x + blockIdx.x] = t;
+        // Re and Im of vector l: rows 2 l and 2 l + 1 of nblk partials
+        partials[((size_t)grp * 2 * NL + threadIdx.x) * nblk + chunk] = t;
     }
 }
 
@@ -211,8 +217,7 @@ k_multidot32(const float4 *__restrict__ V, long ld, int nv, const float4 *__rest
 static __global__ void __launch_bounds__(256)
 k_multidot_fin(const double *__restrict__ partials, int nblk, int nv, double scale, double2 *__restrict__ out) {
     const int l = blockIdx.x;
-    const int grp = l / 8, j = l % 8;
-    const double *pre = partials + ((size_t)grp * 16 + 2 * j) * nblk;
+    const double *pre = partials + (size_t)2 * l * nblk;
     const double *pim = pre + nblk;
     double a = 0.0, b = 0.0;
     for (int t = threadIdx.x; t < nblk; t += blockDim.x) { a += pre[t]; b += pim[t]; }
@@ -234,7 +239,7 @@ k_multidot_fin(const double *__restrict__ partials, int nblk, int nv, double sca
 // Grow the FP32 multi-dot scratch for up to nv vectors (call outside graph capture).
 inline int reserve_multidot(Op &op, int nv) {
     const int nblk = (op.g.V + kMdThreads - 1) / kMdThreads;
-    const size_t need = (size_t)((nv + 7) / 8) * 16 * nblk * sizeof(double);
+    const size_t need = (size_t)((nv + kMdVectors - 1) / kMdVectors) * kMdVectors * 2 * nblk * sizeof(double);
     if (op.md_scratch.bytes < need) {
         DLZ_CUDA_TRY(cudaStreamSynchronize(op.stream));
         DLZ_TRY(op.md_scratch.alloc(need));
@@ -250,11 +255,12 @@ inline int multidot(Op &op, const typename P::E *V, long ld, int nv, const typen
         if (nv <= 0) return DLZ_OK;
         const int sites = op.g.V;
         const int nblk = (sites + kMdThreads - 1) / kMdThreads;
-        const int ngrp = (nv + 7) / 8;
-        const size_t need = (size_t)ngrp * 16 * nblk;
+        const unsigned ngrp = (unsigned)((nv + kMdVectors - 1) / kMdVectors);
+        const size_t need = (size_t)ngrp * kMdVectors * 2 * nblk;
         if (op.md_scratch.bytes < need * sizeof(double))
             return fail(DLZ_ERR_BADARG, "multidot scratch not reserved (reserve_multidot)");
-        k_multidot32<<<dim3(nblk, ngrp), kMdThreads, 0, op.stream>>>(V, ld, nv, w, sites, op.md_scratch.as<double>());
+        k_multidot32<<<ngrp * (unsigned)nblk, kMdThreads, 0, op.stream>>>(V, ld, nv, w, sites, nblk, FastDiv(ngrp),
+                                                                       op.md_scratch.as<double>());
         k_multidot_fin<<<nv, 256, 0, op.stream>>>(op.md_scratch.as<double>(), nblk, nv, scale, dev_out);
         op.prof.launches += 2;
         DLZ_CUDA_TRY(cudaGetLastError());
