@@ -20,8 +20,8 @@ struct P64 {
     static int apply(Op &op, E *out, const E *in, int which, E *tmp) { return apply64(op, out, in, which, tmp); }
     __device__ static double rdot(E a, E b) { return a.x * b.x + a.y * b.y; }
     __device__ static void cdot(E a, E b, double &re, double &im) {
-        re += a.x * b.x + a.y * b.y;
-        im += a.x * b.y - a.y * b.x;
+        re = fma(a.y, b.y, fma(a.x, b.x, re));
+        im = fma(-a.y, b.x, fma(a.x, b.y, im));
     }
     __device__ static double nrm(E a) { return a.x * a.x + a.y * a.y; }
     __device__ static E axpy(double s, E x, E y) { return make_double2(fma(s, x.x, y.x), fma(s, x.y, y.y)); }
