@@ -57,7 +57,7 @@ REF_FIRST_RHS_MVPS = 27830
 # DRAM bytes (read + write) of one k_cg_k1 launch (16 RHS, 24^3x48), the dominant kernel,
 # from one single-pass ncu capture of the kernel at this size (summarised under
 # profiles/); None until taken for the current kernel
-K1_TRAFFIC_BYTES = 8.30e9
+K1_TRAFFIC_BYTES = 3.75e9
 METRIC = "RHS solved/s to |r|/|b|<1e-10 (Lan-DR(120,60) + D-CG, 49 Gaussian RHS, 24^3x48)"
 UNIT = "RHS/s"
 
