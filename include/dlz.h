@@ -408,8 +408,8 @@ int dlz_basis_dots(const float *V, long long ldv, int nin, const float *R, long 
 /*
  * (Measurement of the uneven multi-lattice batch; no counterpart in the paper.)
  * The launch form the autotuner of the last DLZ_F32 dlz_batch_dminres call chose (op:
- * that call's ops[0]): form 0 = one launch per stage replayed from CUDA graphs, 1 = one
- * persistent cooperative launch over all slots and iterations (grid barriers whose waits
+ * that call's ops[0]): form 0 = one launch per stage replayed from CUDA graphs, 1 (only
+ * with DLZ_MULTI_FORM=persistent) = one persistent cooperative launch over all slots and iterations (grid barriers whose waits
  * give up after a bounded number of polls, about a second, and then make the call return
  * DLZ_ERR_DEVICE_TIMEOUT); chunks_per_block: 128-site chunks per block (or per work
  * item); half_grid: 1 if the persistent grid was half the co-resident maximum.  Any
