@@ -52,7 +52,7 @@ C2_DR_CYCLES = 150
 # per iteration with these counts (taken from the FP64 form of the library on this
 # workload, mean of 2 RHS; the default line reports the counts of its own FP64 run in
 # plain_fp64)
-REF_ITERS_PER_RHS = 2328
+REF_ITERS_PER_RHS = 968
 REF_FIRST_RHS_MVPS = 27830
 # DRAM bytes (read + write) of one k_cg_k1 launch (16 RHS, 24^3x48), the dominant kernel,
 # from one single-pass ncu capture of the kernel at this size (summarised under
