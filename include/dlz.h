@@ -32,6 +32,10 @@
  * by the library and released with their destroy call.  All GPU work is
  * ordered on the stream given to dlz_create_operator (0 = legacy default
  * stream); the solver calls return when their results are complete.
+ * dlz_apply and the DLZ_F32 forms of dlz_dcg and dlz_dminres keep work memory on the device
+ * from one call to the next: at most 4 buffers of at most 64 MiB per operator and 512 MiB
+ * over all operators of the process.  It is freed with the operator, and all of it whenever
+ * a device allocation of the library would otherwise fail.
  *
  * Errors: every call returns DLZ_OK (0) or a negative DLZ_ERR_* code; no
  * C++ exception crosses the ABI.  dlz_strerror() names a code,
@@ -241,8 +245,8 @@ int dlz_apply(dlz_op_t op, int which, const void *in, void *out, int dtype, int 
  * allocate device memory at the point of the call: a caller whose memory pool
  * already holds the device's free memory (cudaMalloc would fail), or one that
  * keeps other streams busy and cannot afford the device-wide synchronisation
- * of a cudaFree (dlz_apply keeps up to 4 work buffers of 64 MiB with the operator and
- * frees larger ones before it returns).
+ * of a cudaFree (dlz_apply frees work buffers that it cannot keep before it returns; see
+ * "Memory" at the top).
  *
  * Same operation, arguments and layout as dlz_apply (dtype DLZ_F64 or DLZ_F32
  * only), except: in and out must

@@ -30,62 +30,6 @@ int fail(int code, const std::string &msg) {
     return code;
 }
 
-int DevBuf::alloc(size_t nbytes) {
-    release();
-    if (nbytes == 0) return DLZ_OK;
-    cudaError_t e = cudaMalloc(&p, nbytes);
-    if (e != cudaSuccess) {
-        p = nullptr;
-        cudaGetLastError();
-        return fail(e == cudaErrorMemoryAllocation ? DLZ_ERR_OOM : DLZ_ERR_CUDA,
-                    "cudaMalloc(" + std::to_string(nbytes) + "): " + cudaGetErrorString(e));
-    }
-    bytes = nbytes;
-    return DLZ_OK;
-}
-DevBuf *ScratchPool::take(size_t bytes, int &rc) {
-    {
-        std::lock_guard<std::mutex> lk(mu);
-        int best = -1;
-        for (int i = 0; i < (int)idle.size(); ++i)
-            if (idle[i]->bytes >= bytes && (best < 0 || idle[i]->bytes < idle[best]->bytes)) best = i;
-        if (best >= 0) {
-            DevBuf *b = idle[best];
-            idle.erase(idle.begin() + best);
-            rc = DLZ_OK;
-            return b;
-        }
-    }
-    DevBuf *b = new DevBuf();
-    rc = b->alloc(bytes);
-    if (rc != DLZ_OK) {
-        delete b;
-        return nullptr;
-    }
-    return b;
-}
-void ScratchPool::give(DevBuf *b) {
-    if (b->bytes <= kKeepBytes) {
-        std::lock_guard<std::mutex> lk(mu);
-        if ((int)idle.size() < kKeep) {
-            idle.push_back(b);
-            return;
-        }
-        // full: the smallest one goes
-        auto it = std::min_element(idle.begin(), idle.end(), [](DevBuf *x, DevBuf *y) { return x->bytes < y->bytes; });
-        if ((*it)->bytes < b->bytes) std::swap(*it, b);
-    }
-    delete b;
-}
-ScratchPool::~ScratchPool() {
-    for (DevBuf *b : idle) delete b;
-}
-void DevBuf::release() {
-    if (p) cudaFree(p);
-    p = nullptr;
-    bytes = 0;
-}
-
 void Profiler::begin(bool on, bool f32) {
     enabled = on;
     hot_f32 = f32;

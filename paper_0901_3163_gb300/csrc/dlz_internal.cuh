@@ -15,8 +15,8 @@
 
 #include <cuda_runtime.h>
 
+#include <cmath>
 #include <cstdint>
-#include <mutex>
 #include <string>
 #include <vector>
 
@@ -194,18 +194,23 @@ struct GrowBuf {
 };
 // Device work memory that an operator keeps between calls: a call takes a buffer for its
 // own use and gives it back when its work is complete, so calls of several host threads
-// never share one.  At most kKeep buffers of at most kKeepBytes each are kept (a cudaMalloc
-// and cudaFree pair costs about as much as a whole application on a 8^4 lattice); larger
-// ones are freed at once, all of them with the operator.
+// never share one.  At most kKeep buffers of at most kKeepBytes each are kept per operator (a
+// cudaMalloc and cudaFree pair costs about as much as a whole application on a 8^4 lattice), and
+// at most kKeepAllBytes by all operators together; the others are freed at once, an operator's
+// with it, and all idle ones when an allocation of the library does not fit (DevBuf::alloc).
 struct ScratchPool {
     static constexpr int kKeep = 4;
-    static constexpr size_t kKeepBytes = (size_t)64 << 20;
-    std::mutex mu;
+    static constexpr size_t kKeepBytes = (size_t)64 << 20, kKeepAllBytes = (size_t)512 << 20;
     std::vector<DevBuf *> idle;
+    ScratchPool();
+    ScratchPool(const ScratchPool &) = delete;
+    ScratchPool &operator=(const ScratchPool &) = delete;
+    ~ScratchPool();
     // the smallest idle buffer that is large enough, or a new one; null: out of memory
     DevBuf *take(size_t bytes, int &rc);
     void give(DevBuf *b);
-    ~ScratchPool();
+    // frees the idle buffers of every operator; false: there were none
+    static bool free_idle();
 };
 // a pool buffer for one call; waits for the stream before giving it back unless the call
 // has already waited (done)
@@ -265,7 +270,7 @@ struct Op {
     DevBuf md_scratch;   // block partials of the FP32 multi-dot (grown on demand, outside graphs)
     int multi_choice = 0;   // launch form the multi-lattice autotuner chose last (100 form + 10 chunks + half)
     TcScratch tc;           // scratch of the tensor-core basis products
-    ScratchPool pool;       // work memory of dlz_apply
+    ScratchPool pool;       // work memory of dlz_apply and of the FP32 D-CG and D-MinRes calls
     DevBuf stage_err;       // int: set by a stencil kernel whose staging wait gave up
 };
 
