@@ -455,6 +455,8 @@ int dlz_stencil_bench(dlz_op_t op, int dtype, int which, int nrhs, int iters, co
  *   are used from now on (a network is trained over many gauge fields).
  * dlz_net_forward: in, out: device complex64 [nvec][V][4][3]; keeps every
  *   layer's input for the next dlz_net_backward.
+ *   Infinities and NaN go through the layers and their gradients as in FP32 arithmetic
+ *   (a pass with a result that is not finite is computed a second time).
  * dlz_net_backward: grad_out = G(out) of the last forward (same nvec);
  *   adds G(W) to the gradient buffer; grad_in (may be NULL) receives G(in).
  * dlz_net_get: what = 0 master weights, 1 gradients, 2 the bfloat16 weights in

@@ -145,13 +145,72 @@ k_ptc_fwd(float4 *__restrict__ out, const float4 *__restrict__ in, const __nv_bf
     for (int q = 0; q < CG; ++q) Field<float>::store(ov + (size_t)(g0 + q) * plane, g.V, s, acc[q]);
 }
 
-// grad[o][c'][c][4 s' + s] += sum over blocks (fixed order) of the partials
+// The weight gradient in plain FP32 arithmetic (for passes that are not finite, see run_layers):
+// partials of G(W)[o][c'][c] as ptc_tc_wgrad leaves them; grid (blocks, 9 C_out C_in), a thread
+// per site
+constexpr int kGradThreads = 128, kGradBlocks = 16;
+static_assert(kGradBlocks <= kPtcMaxGradBlocks, "partials");
+__global__ void __launch_bounds__(kGradThreads)
+k_ptc_wgrad(float2 *__restrict__ partials, const float4 *__restrict__ gout, const float4 *__restrict__ x,
+            const float4 *__restrict__ U, Geom g, int cin, int cout, int nvec) {
+    const int o = blockIdx.y / (cout * cin), cp = blockIdx.y / cin % cout, c = blockIdx.y % cin;
+    const size_t plane = (size_t)6 * g.V;
+    float2 acc[16];
+#pragma unroll
+    for (int e = 0; e < 16; ++e) acc[e] = make_float2(0.f, 0.f);
+    for (long i = (long)blockIdx.x * kGradThreads + threadIdx.x; i < (long)g.V * nvec; i += (long)gridDim.x * kGradThreads) {
+        const int vec = (int)(i / g.V), s = (int)(i % g.V);
+        float2 q[12], t[12];
+        Field<float>::load(gout + ((size_t)vec * cout + cp) * plane, g.V, s, q);
+        const float4 *xv = x + ((size_t)vec * cin + c) * plane;
+        if (o == 0) {
+            Field<float>::load(xv, g.V, s, t);
+        } else {
+            int sn, ls, mu;
+            bool fwd;
+            neighbour(s, g, o, sn, ls, mu, fwd);
+            float2 p[12], u[9];
+            Field<float>::load(xv, g.V, sn, p);
+            Link<float>::load(U, g.V, mu, ls, u);
+            transport(p, u, fwd, t);
+        }
+#pragma unroll
+        for (int e = 0; e < 16; ++e)
+#pragma unroll
+            for (int col = 0; col < 3; ++col) acc[e] = cfmaConj(t[3 * (e % 4) + col], q[3 * (e / 4) + col], acc[e]);
+    }
+    __shared__ float2 sm[16][kGradThreads / 32];
+#pragma unroll
+    for (int e = 0; e < 16; ++e) {
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) {
+            acc[e].x += __shfl_down_sync(0xffffffffu, acc[e].x, d);
+            acc[e].y += __shfl_down_sync(0xffffffffu, acc[e].y, d);
+        }
+        if ((threadIdx.x & 31) == 0) sm[e][threadIdx.x >> 5] = acc[e];
+    }
+    __syncthreads();
+    const int e = threadIdx.x;
+    if (e >= 16) return;
+    float2 a = make_float2(0.f, 0.f);
+    for (int w = 0; w < kGradThreads / 32; ++w) {
+        a.x += sm[e][w].x;
+        a.y += sm[e][w].y;
+    }
+    const int rows = cout * 4, cols = cin * 4;
+    partials[(((size_t)o * gridDim.x + blockIdx.x) * rows + 4 * cp + e / 4) * cols + 4 * c + e % 4] = a;
+}
+
+// grad[o][c'][c][4 s' + s] += sum over blocks (fixed order) of the partials.  state (may be
+// null): the pass's error bits; nothing is added once one is set.  *added: whether it was.
 __global__ void k_ptc_wgrad_sum(float2 *__restrict__ grad, const float2 *__restrict__ partials, int nblk,
-                                int cin, int cout) {
+                                int cin, int cout, const int *__restrict__ state, int *__restrict__ added) {
     const int rows = cout * 4, cols = cin * 4;
     const long n = 9L * rows * cols;
     const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
+    const bool skip = state && *state;
+    if (i == 0) *added = skip ? 0 : 1;
+    if (i >= n || skip) return;
     const int o = (int)(i / ((long)rows * cols));
     const int rc = (int)(i % ((long)rows * cols));
     const int r = rc / cols, c = rc % cols;
@@ -222,7 +281,7 @@ struct dlz_net_s {
     std::vector<size_t> off;            // first complex weight of each layer
     size_t nw = 0;
     dlz::DevBuf master, grad, m1, m2, wb, wadj, partials;
-    dlz::DevBuf img, err;               // weight images of the tensor-core layers; a wait that gave up
+    dlz::DevBuf img, state;             // weight images of the tensor-core layers; PassState
     std::vector<size_t> img_fwd, img_adj;   // their offsets (bf16 elements)
     int adam_t = 0;
     dlz::DevBuf act[dlz::kMaxLayersNet + 1];   // input of every layer from the last forward
@@ -233,9 +292,17 @@ struct dlz_net_s {
 namespace dlz {
 namespace {
 
+// What a pass leaves on the device for the host: the error bits of the tensor-core kernels, and
+// which layers' weight gradients were added
+struct PassState {
+    int err;
+    int added[kMaxLayersNet];
+};
+
+// img null: on the CUDA cores whatever the widths
 int layer_forward(Op &op, float4 *out, const float4 *in, const __nv_bfloat162 *W, const __nv_bfloat16 *img, int *err,
                   int cin, int cout, int nvec) {
-    if (ptc_tc_layer(cin, cout)) return ptc_tc_forward(op, out, in, img, cin, cout, nvec, err);
+    if (img && ptc_tc_layer(cin, cout)) return ptc_tc_forward(op, out, in, img, cin, cout, nvec, err);
     const Geom g = op.g;
     const float4 *U = op.gauge32.as<float4>();
     const unsigned gx = blocks_for(g.V, kFwdThreads);
@@ -275,13 +342,62 @@ int refresh_bf16(dlz_net_s *net) {
     return DLZ_OK;
 }
 
-// after the stream has finished: whether a wait of a tensor-core layer gave up
-int check_layers(dlz_net_s *net) {
-    int h = 0;
-    DLZ_TRY(d2h_sync(*net->op, &h, net->err.p, sizeof(int)));
-    if (!h) return DLZ_OK;
-    DLZ_CUDA_TRY(cudaMemsetAsync(net->err.p, 0, sizeof(int), net->op->stream));
-    return fail(DLZ_ERR_DEVICE_TIMEOUT, "a wait of a tensor-core network layer gave up");
+// waits for the pass and reads its state (its error bits are cleared for the next pass); fails if
+// a wait gave up
+int read_state(dlz_net_s *net, PassState &st) {
+    DLZ_TRY(d2h_sync(*net->op, &st, net->state.p, sizeof(PassState)));
+    if (!st.err) return DLZ_OK;
+    DLZ_CUDA_TRY(cudaMemsetAsync(net->state.p, 0, sizeof(int), net->op->stream));
+    if (st.err & kPtcTimeout) return fail(DLZ_ERR_DEVICE_TIMEOUT, "a wait of a tensor-core network layer gave up");
+    return DLZ_OK;
+}
+
+// The layers forward, act[0] to act[nl]; tc: on the tensor cores where that is faster.  A pass
+// with a result that is not finite is run again on the CUDA cores, whose FP32 arithmetic keeps
+// infinities: on the tensor cores the parts of an infinite value give NaN.
+int run_layers(dlz_net_s *net, int nvec, bool tc) {
+    for (int l = 0; l < net->nl; ++l)
+        DLZ_TRY(layer_forward(*net->op, net->act[l + 1].as<float4>(), net->act[l].as<float4>(),
+                              net->wb.as<__nv_bfloat162>() + net->off[l],
+                              tc ? net->img.as<__nv_bfloat16>() + net->img_fwd[l] : nullptr, net->state.as<int>(),
+                              net->w[l], net->w[l + 1], nvec));
+    return DLZ_OK;
+}
+
+// The layers backward from grad_out in the user layout; *gin: the input's gradient (made if
+// want_in).  done (may be null): layers whose weight gradients are there already.
+int run_layers_back(dlz_net_s *net, const void *grad_out, int nvec, bool want_in, bool tc, const int *done, float4 **gin) {
+    Op &op = *net->op;
+    PassState *st = net->state.as<PassState>();
+    float4 *gc = net->gbuf[0].as<float4>(), *gn = net->gbuf[1].as<float4>();
+    DLZ_TRY(pack32(op, gc, (const float2 *)grad_out, nvec));
+    for (int l = net->nl - 1; l >= 0; --l) {
+        const int cin = net->w[l], cout = net->w[l + 1];
+        if (!done || !done[l]) {
+            int blocks = kGradBlocks;
+            if (tc) {
+                DLZ_TRY(ptc_tc_wgrad(op, net->partials.as<float2>(), gc, net->act[l].as<float4>(), cin, cout, nvec,
+                                     &st->err, blocks));
+            } else {
+                k_ptc_wgrad<<<dim3(blocks, 9 * cin * cout), kGradThreads, 0, op.stream>>>(
+                    net->partials.as<float2>(), gc, net->act[l].as<float4>(), op.gauge32.as<float4>(), op.g, cin, cout, nvec);
+                op.prof.launches++;
+            }
+            const long ne = 9L * cin * cout * 16;
+            k_ptc_wgrad_sum<<<blocks_for(ne, 256), 256, 0, op.stream>>>(
+                net->grad.as<float2>() + net->off[l], net->partials.as<float2>(), blocks, cin, cout,
+                tc ? &st->err : nullptr, &st->added[l]);
+            op.prof.launches += 1;
+            DLZ_CUDA_TRY(cudaGetLastError());
+        }
+        if (l > 0 || want_in) {
+            DLZ_TRY(layer_forward(op, gn, gc, net->wadj.as<__nv_bfloat162>() + net->off[l],
+                                  tc ? net->img.as<__nv_bfloat16>() + net->img_adj[l] : nullptr, &st->err, cout, cin, nvec));
+            std::swap(gc, gn);
+        }
+    }
+    *gin = gc;
+    return DLZ_OK;
 }
 
 int set_attrs() {
@@ -347,8 +463,8 @@ int dlz_net_create(dlz_op_t h, int nlayers, const int *widths, const void *weigh
             ni += ptc_tc_image_size(widths[l + 1], widths[l]);
         }
         DLZ_TRY(net->img.alloc(ni * sizeof(__nv_bfloat16)));
-        DLZ_TRY(net->err.alloc(sizeof(int)));
-        DLZ_CUDA_TRY(cudaMemsetAsync(net->err.p, 0, sizeof(int), op.stream));
+        DLZ_TRY(net->state.alloc(sizeof(PassState)));
+        DLZ_CUDA_TRY(cudaMemsetAsync(net->state.p, 0, sizeof(PassState), op.stream));
         int maxp = 0;
         for (int l = 0; l < nlayers; ++l) maxp = std::max(maxp, 16 * widths[l] * widths[l + 1]);
         DLZ_TRY(net->partials.alloc((size_t)9 * kPtcMaxGradBlocks * maxp * sizeof(float2)));
@@ -392,13 +508,15 @@ int dlz_net_forward(dlz_net_t net, const void *in, int nvec, void *out) {
         net->act_nvec = nvec;
     }
     DLZ_TRY(pack32(op, net->act[0].as<float4>(), (const float2 *)in, nvec));
-    for (int l = 0; l < net->nl; ++l)
-        DLZ_TRY(layer_forward(op, net->act[l + 1].as<float4>(), net->act[l].as<float4>(),
-                              net->wb.as<__nv_bfloat162>() + net->off[l],
-                              net->img.as<__nv_bfloat16>() + net->img_fwd[l], net->err.as<int>(), net->w[l],
-                              net->w[l + 1], nvec));
+    DLZ_TRY(run_layers(net, nvec, true));
     DLZ_TRY(unpack32(op, (float2 *)out, net->act[net->nl].as<float4>(), nvec));
-    return check_layers(net);
+    PassState st;
+    DLZ_TRY(read_state(net, st));
+    if (!(st.err & kPtcNonfinite)) return DLZ_OK;
+    DLZ_TRY(run_layers(net, nvec, false));
+    DLZ_TRY(unpack32(op, (float2 *)out, net->act[net->nl].as<float4>(), nvec));
+    DLZ_CUDA_TRY(cudaStreamSynchronize(op.stream));
+    return DLZ_OK;
 }
 
 int dlz_net_backward(dlz_net_t net, const void *grad_out, int nvec, void *grad_in) {
@@ -414,26 +532,20 @@ int dlz_net_backward(dlz_net_t net, const void *grad_out, int nvec, void *grad_i
     for (int b = 0; b < 2; ++b)
         if (net->gbuf[b].bytes < (size_t)nvec * maxw * plane * sizeof(float4))
             DLZ_TRY(net->gbuf[b].alloc((size_t)nvec * maxw * plane * sizeof(float4)));
-    float4 *gc = net->gbuf[0].as<float4>(), *gn = net->gbuf[1].as<float4>();
-    DLZ_TRY(pack32(op, gc, (const float2 *)grad_out, nvec));
-    for (int l = net->nl - 1; l >= 0; --l) {
-        const int cin = net->w[l], cout = net->w[l + 1];
-        int blocks = 0;
-        DLZ_TRY(ptc_tc_wgrad(op, net->partials.as<float2>(), gc, net->act[l].as<float4>(), cin, cout, nvec,
-                             net->err.as<int>(), blocks));
-        const long ne = 9L * cin * cout * 16;
-        k_ptc_wgrad_sum<<<blocks_for(ne, 256), 256, 0, op.stream>>>(net->grad.as<float2>() + net->off[l],
-                                                                    net->partials.as<float2>(), blocks, cin, cout);
-        op.prof.launches += 1;
-        DLZ_CUDA_TRY(cudaGetLastError());
-        if (l > 0 || grad_in) {
-            DLZ_TRY(layer_forward(op, gn, gc, net->wadj.as<__nv_bfloat162>() + net->off[l],
-                                  net->img.as<__nv_bfloat16>() + net->img_adj[l], net->err.as<int>(), cout, cin, nvec));
-            std::swap(gc, gn);
-        }
-    }
-    if (grad_in) DLZ_TRY(unpack32(op, (float2 *)grad_in, gc, nvec));
-    return check_layers(net);
+    float4 *gin = nullptr;
+    DLZ_TRY(run_layers_back(net, grad_out, nvec, grad_in != nullptr, true, nullptr, &gin));
+    // (grad_in written before the state is read, unless it would overwrite what a second pass reads)
+    const size_t bytes = (size_t)12 * op.g.V * nvec * sizeof(float2);
+    const char *pi = (const char *)grad_in, *po = (const char *)grad_out;
+    const bool early = grad_in && !(pi < po + bytes && po < pi + bytes);
+    if (early) DLZ_TRY(unpack32(op, (float2 *)grad_in, gin, nvec));
+    PassState st;
+    DLZ_TRY(read_state(net, st));
+    const bool again = st.err & kPtcNonfinite;
+    if (again) DLZ_TRY(run_layers_back(net, grad_out, nvec, grad_in != nullptr, false, st.added, &gin));
+    if (grad_in && (again || !early)) DLZ_TRY(unpack32(op, (float2 *)grad_in, gin, nvec));
+    if (again || (grad_in && !early)) DLZ_CUDA_TRY(cudaStreamSynchronize(op.stream));
+    return DLZ_OK;
 }
 
 int dlz_net_get(dlz_net_t net, int what, void *host_out) {

@@ -266,6 +266,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ptc_tc_fwd(FwdArgs a) {
         const int row = 32 * lq + lane, sl = row / 3, col = row - 3 * sl;
         int n = 0;
         bool ok = true;
+        float nan = 0.f;                  // 0 times every result: NaN if one is not finite
         for (int ti = 0; ti < mine && ok; ++ti) {
             float sum[64];
 #pragma unroll
@@ -291,14 +292,17 @@ __global__ void __launch_bounds__(kThreads, 1) k_ptc_tc_fwd(FwdArgs a) {
 #pragma unroll
             for (int j = 0; j < 64; j += 2) {
                 const int ch = (c_lo + j) / 8, comp = 3 * ((j % 8) / 2) + col;
-                if (j < half && ch < a.cout)
+                if (j < half && ch < a.cout) {
                     reinterpret_cast<float2 *>(dst + (size_t)ch * plane + (size_t)(comp >> 1) * V)[comp & 1] =
                         make_float2(sum[j], sum[j + 1]);
+                    nan = fmaf(sum[j], 0.f, fmaf(sum[j + 1], 0.f, nan));
+                }
             }
         }
+        if (__any_sync(0xffffffffu, nan != 0.f) && lane == 0) atomicOr(a.err, kPtcNonfinite);
     }
     __syncthreads();
-    if (sh.failed && threadIdx.x == 0) atomicExch(a.err, 1);
+    if (sh.failed && threadIdx.x == 0) atomicOr(a.err, kPtcTimeout);
     tc_teardown(taddr, a.ncols);
 }
 
@@ -479,16 +483,21 @@ __global__ void __launch_bounds__(kThreads, 1) k_ptc_tc_wgrad(GradArgs a) {
         // row 2 r + (0 re, 1 im): the re lane combines its sums with its neighbour's
         const int r = (32 * lq + lane) / 2;
         float2 *pb = a.partials + ((size_t)o * gridDim.x + blockIdx.x) * rows * cols;
+        float nan = 0.f;                  // 0 times every result: NaN if one is not finite
 #pragma unroll
         for (int j = 0; j < 64; j += 2) {
             const float q0 = __shfl_down_sync(0xffffffffu, sum[j], 1), q1 = __shfl_down_sync(0xffffffffu, sum[j + 1], 1);
             const int c = (c_lo + j) / 2;
-            if (j < half && (lane & 1) == 0 && r < rows && c < cols)
-                pb[(size_t)r * cols + c] = make_float2(sum[j] + q1, q0 - sum[j + 1]);
+            if (j < half && (lane & 1) == 0 && r < rows && c < cols) {
+                const float2 v = make_float2(sum[j] + q1, q0 - sum[j + 1]);
+                pb[(size_t)r * cols + c] = v;
+                nan = fmaf(v.x, 0.f, fmaf(v.y, 0.f, nan));
+            }
         }
+        if (__any_sync(0xffffffffu, nan != 0.f) && lane == 0) atomicOr(a.err, kPtcNonfinite);
     }
     __syncthreads();
-    if (sh.failed && threadIdx.x == 0) atomicExch(a.err, 1);
+    if (sh.failed && threadIdx.x == 0) atomicOr(a.err, kPtcTimeout);
     tc_teardown(taddr, a.ncols);
 }
 

@@ -14,7 +14,11 @@ bool ptc_tc_layer(int cin, int cout);
 int ptc_tc_prepare();       // kernel attributes, outside graph captures
 // weights [9][cout][cin][16] -> image
 int ptc_tc_image(Op &op, __nv_bfloat16 *img, const __nv_bfloat162 *w, int cin, int cout);
-// the layer on nvec fields; *err (device) is set if a wait gave up
+// Bits of the device word *err of the two kernels below: a wait gave up; a result is not finite
+// (an infinite operand has no finite remainder for its second part, so it gives NaN where FP32
+// arithmetic may give an infinity: the caller computes such a pass again without tensor cores)
+constexpr int kPtcTimeout = 1, kPtcNonfinite = 2;
+// the layer on nvec fields
 int ptc_tc_forward(Op &op, float4 *out, const float4 *in, const __nv_bfloat16 *img, int cin, int cout, int nvec,
                    int *err);
 // block partials [9][blocks][4 cout][4 cin] of the layer's weight gradient from G(out) and the
