@@ -106,9 +106,12 @@ int dsolve_mixed_batch(Op &op, const dlz_defl_s *d, bool minres, const double2 *
     long long mv_batch = 0;
     auto residuals = [&]() -> int {
         // (from the start x = 0 the residual is b' itself: A x = 0 without the FP64 stencil)
-        if (outer > 0 || X_init) DLZ_TRY(wilson64_batch(op, pt, px, which, N));
-        else DLZ_CUDA_TRY(cudaMemsetAsync(pt, 0, (size_t)N * n64 * sizeof(double2), op.stream));
-        mv_batch += 1;
+        if (outer > 0 || X_init) {
+            DLZ_TRY(wilson64_batch(op, pt, px, which, N));
+            mv_batch += 1;
+        } else {
+            DLZ_CUDA_TRY(cudaMemsetAsync(pt, 0, (size_t)N * n64 * sizeof(double2), op.stream));
+        }
         DLZ_TRY(reduce<kMaxBatch>(op, n64, [=] __device__(long i, double (&acc)[kMaxBatch]) {
 #pragma unroll
             for (int q = 0; q < kMaxBatch; ++q) {
