@@ -310,9 +310,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_ptc_tc_fwd(FwdArgs a) {
 // G(W)[o][c'][c] = sum over sites and colours of G(out) (T_o in)^dag as P[m][n] = sum_k A[m][k]
 // B[n][k]: m = 8 c' + 2 s' + re/im of G(out), n = 8 c + 2 s + re/im of the transported input, k
 // the sites and colours; re G = P[re][re] + P[im][im], im G = P[im][re] - P[re][im].  Both
-// operands are FP32 values in three bfloat16 parts h, m, l; of the nine products of parts the
-// six down to 2^-16 are formed (the others are below 2^-24), smallest first, so that only the
-// three steps of h h are cut off at the size of the sum.
+// operands are FP32 values in three bfloat16 parts h, m, l of up to 8 bits, all with the value's
+// sign: m is below 2^-7 and l below 2^-15 of the value.  All products of parts but l l (below
+// 2^-30) are formed, smallest first, so that only the three steps of h h are cut off at the size of
+// the sum.  (Without m l and l m, together below 2^-21, every term of a sum of products of one
+// sign loses a little on the same side.)
 // A block has one offset and every gridDim.x-th tile of 16 sites: a stage is one tile, 48 k (K
 // step = colour).  The operands are stored as they come, 16 bytes = the 8 values of a channel at
 // one k, i.e. M- and N-major: 8 x 8 core matrices of 8 k x 16 bytes, k groups 128 bytes apart,
@@ -440,7 +442,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ptc_tc_wgrad(GradArgs a) {
         const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) |
                                ((uint32_t)(a.npad >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
         const uint32_t d0 = sdesc_lo(su32(smem)), w_stage = stage_bytes >> 4;
-        const int pa[6] = {2, 0, 1, 1, 0, 0}, pb[6] = {0, 2, 1, 0, 1, 0};
+        const int pa[8] = {2, 1, 2, 0, 1, 1, 0, 0}, pb[8] = {1, 2, 0, 2, 1, 0, 1, 0};
         int st = 0;
         uint32_t round = 0;
         for (int n = 0; n < mine; ++n) {
@@ -451,7 +453,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ptc_tc_wgrad(GradArgs a) {
             const uint32_t da = d0 + st * w_stage, db = da + (3 * kGPartA >> 4);
             if (lane == 0) {
 #pragma unroll
-                for (int p = 0; p < 6; ++p)
+                for (int p = 0; p < 8; ++p)
 #pragma unroll
                     for (int k = 0; k < 3; ++k)
                         mma_bf16(taddr + acc * a.npad, da + (pa[p] * kGPartA >> 4) + k * 16, db + (pb[p] * part_b >> 4) + k * 16,
