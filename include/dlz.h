@@ -451,8 +451,8 @@ int dlz_stencil_bench(dlz_op_t op, int dtype, int which, int nrhs, int iters, co
  * dlz_net_create: nlayers in [1, 8], widths[0] = widths[nlayers] = 1, every
  *   width in [1, 16]; weights: complex64, the layers one after another, each
  *   [9][widths[l+1]][widths[l]][16] (host or device; copied).
- * dlz_net_bind: the links (and stream) of another operator on the same lattice
- *   are used from now on (a network is trained over many gauge fields).
+ * dlz_net_bind: the links (and stream) of another operator on the same lattice (not an
+ *   even-odd one) are used from now on (a network is trained over many gauge fields).
  * dlz_net_forward: in, out: device complex64 [nvec][V][4][3]; keeps every
  *   layer's input for the next dlz_net_backward.
  *   Infinities and NaN go through the layers and their gradients as in FP32 arithmetic

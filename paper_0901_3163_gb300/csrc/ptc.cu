@@ -600,6 +600,7 @@ int dlz_net_adam_step(dlz_net_t net, double lr, double beta1, double beta2, doub
 
 int dlz_net_bind(dlz_net_t net, dlz_op_t h) {
     if (!net || !h) return fail(DLZ_ERR_BADARG, "null argument");
+    if (h->op.eo) return fail(DLZ_ERR_BADARG, "the network runs on full-lattice operators");
     const Geom &a = net->op->g, &b = h->op.g;
     for (int d = 0; d < 4; ++d)
         if (a.L[d] != b.L[d]) return fail(DLZ_ERR_BADARG, "net_bind needs an operator on the same lattice");
