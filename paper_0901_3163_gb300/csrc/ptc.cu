@@ -503,6 +503,7 @@ int dlz_net_forward(dlz_net_t net, const void *in, int nvec, void *out) {
     op.prof.begin(false, false);
     const size_t plane = (size_t)6 * op.g.V;      // float4 per channel
     if (net->act_nvec != nvec) {
+        net->act_nvec = 0;            // (an allocation that fails leaves no buffers for either size)
         for (int l = 0; l <= net->nl; ++l)
             DLZ_TRY(net->act[l].alloc((size_t)nvec * net->w[l] * plane * sizeof(float4)));
         net->act_nvec = nvec;

@@ -26,3 +26,18 @@ def test_no_even_odd_operator():
         dlz.net_bind(net, dlz.create_operator_eo(DIMS, U, 0.2))
     assert e.value.code == dlz.ERR_BADARG
     assert torch.equal(dlz.net_forward(net, x), want)
+
+
+def test_after_an_allocation_that_failed():
+    dlz, U, op, net, x = _net()
+    want = dlz.net_forward(net, x)
+    out = torch.empty_like(x)
+    # activations of 320 GB: refused when the first buffer is allocated, before any kernel
+    nvec = (320 << 30) // (96 * synth.volume(DIMS))
+    with pytest.raises(dlz.DlzError) as e:
+        dlz._check(dlz.lib.dlz_net_forward(net.handle, x.data_ptr(), nvec, out.data_ptr()))
+    assert e.value.code == dlz.ERR_OOM
+    with pytest.raises(dlz.DlzError) as e:
+        dlz.net_backward(net, x)                          # the forward's activations are gone
+    assert e.value.code == dlz.ERR_BADARG
+    assert torch.equal(dlz.net_forward(net, x), want)
