@@ -50,7 +50,7 @@ struct FwdArgs {
 };
 
 struct FwdShared {
-    uint64_t full[kGroups], empty[kGroups], acc_full[4], acc_empty[4];
+    uint64_t full[kGroups], empty[kGroups], acc_full[4], acc_empty[4], drained;
     uint32_t tbase;
     int failed;
 };
@@ -132,6 +132,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ptc_tc_fwd(FwdArgs a) {
             mbar_init(&sh.acc_full[i], 1);
             mbar_init(&sh.acc_empty[i], kEpi);
         }
+        mbar_init(&sh.drained, 1);
         asm volatile("fence.mbarrier_init.release.cluster;");
     }
     tmem_alloc(&sh.tbase, a.ncols);
@@ -236,7 +237,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ptc_tc_fwd(FwdArgs a) {
         const uint32_t d0 = sdesc_lo(su32(smem)), dhi = ((uint32_t)sbo >> 4) | 1u << 14, w_stage = stage_bytes >> 4;
         int st = 0, n = 0;
         uint32_t round = 0;
-        bool ok = true;
+        bool ok = true, issued = false;
         for (int ti = 0; ti < mine && ok; ++ti)
             for (int sg = 0; sg < nseg && ok; ++sg, ++n) {
                 const int acc = n % a.nbuf, use = n / a.nbuf;
@@ -253,12 +254,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_ptc_tc_fwd(FwdArgs a) {
                                 mma_bf16(taddr + acc * a.npad, da + (h * part >> 4) + k * 16, db + k * 16, dhi, idesc,
                                          ch > 0 || h < 2 || k > 0);
                         commit_to(&sh.empty[st]);
+                        issued = true;
                     }
                     if (++st == kGroups) { st = 0; ++round; }
                 }
                 if (ok && lane == 0) commit_to(&sh.acc_full[acc]);
             }
-        __syncwarp();
+        mma_drain(&sh.drained, issued, failed);
     } else {
         // ---- results: warp w has rows 32 (w % 4) .. of a tile and half of the columns; the
         // thread of row 3 sl + c sums colour c of its output channels in registers
@@ -366,6 +368,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ptc_tc_wgrad(GradArgs a) {
             mbar_init(&sh.acc_full[i], 1);
             mbar_init(&sh.acc_empty[i], kEpi);
         }
+        mbar_init(&sh.drained, 1);
         asm volatile("fence.mbarrier_init.release.cluster;");
     }
     tmem_alloc(&sh.tbase, a.ncols);
@@ -445,6 +448,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ptc_tc_wgrad(GradArgs a) {
         const int pa[8] = {2, 1, 2, 0, 1, 1, 0, 0}, pb[8] = {1, 2, 0, 2, 1, 0, 1, 0};
         int st = 0;
         uint32_t round = 0;
+        bool issued = false;
         for (int n = 0; n < mine; ++n) {
             const int acc = n % a.nbuf, use = n / a.nbuf;
             if (use > 0 && !__all_sync(0xffffffffu, mbar_wait(&sh.acc_empty[acc], (use - 1) & 1, failed))) break;
@@ -460,10 +464,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_ptc_tc_wgrad(GradArgs a) {
                                  kDescHi<kGSbo>, idesc, p > 0 || k > 0);
                 commit_to(&sh.empty[st]);
                 commit_to(&sh.acc_full[acc]);
+                issued = true;
             }
             if (++st == kGroups) { st = 0; ++round; }
         }
-        __syncwarp();
+        mma_drain(&sh.drained, issued, failed);
     } else {
         // ---- sums: warp w has rows 32 (w % 4) .. and half of the columns
         const int lq = warp & 3, half = a.npad / 2, c_lo = (warp >> 2) * half;

@@ -125,12 +125,12 @@ struct CombineArgs {
 // thread's part has landed, raw_empty[r] when the group that took it has read it.  Operand
 // stage s of S: full[s] when every warp of its group has written it, empty[s] when the MMAs
 // that read it are done.  Accumulator a of two: acc_full[a] when a tile's MMAs are done,
-// acc_empty[a] when it has been read.  A wait on a phase's parity is only right while the
+// acc_empty[a] when it has been read; drained when no MMA is in flight any more.  A wait on a phase's parity is only right while the
 // waiter is at most one phase behind: each stage has a group of its own, and R is a multiple
 // of S, so that one group takes all chunks of a slot.
 template <int S, int R> struct TcShared {
     static_assert(R % S == 0, "ring slots per group");
-    uint64_t raw_full[R], raw_empty[R], full[S], empty[S], acc_full[2], acc_empty[2];
+    uint64_t raw_full[R], raw_empty[R], full[S], empty[S], acc_full[2], acc_empty[2], drained;
     uint32_t tbase;
     int failed;
 };
@@ -151,6 +151,7 @@ template <int S, int R> __device__ __forceinline__ uint32_t tc_setup(TcShared<S,
             mbar_init(&sh.acc_full[i], 1);
             mbar_init(&sh.acc_empty[i], kEpiWarps);
         }
+        mbar_init(&sh.drained, 1);
         asm volatile("fence.mbarrier_init.release.cluster;");
     }
     tmem_alloc(&sh.tbase, ncols);
@@ -297,7 +298,7 @@ __global__ void __launch_bounds__(tc_threads(S), 1) k_tc_combine(CombineArgs a) 
         const uint32_t w_stage = stage_bytes >> 4, w_b = b_bytes >> 4;
         int st = 0, n = 0;
         uint32_t round = 0;
-        bool ok = true;
+        bool ok = true, issued = false;
         for (long t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++n) {
             const int acc = n & 1;
             if (n >= 2 && !__all_sync(0xffffffffu, mbar_wait(&sh.acc_empty[acc], ((n >> 1) - 1) & 1, failed))) break;
@@ -310,12 +311,13 @@ __global__ void __launch_bounds__(tc_threads(S), 1) k_tc_combine(CombineArgs a) 
                 if (lane == 0) {
                     chunk_mmas(taddr + acc * a.npad, da, da + (kABytes >> 4), db, db + w_b, idesc, kc == 0);
                     commit_to(&sh.empty[st]);
+                    issued = true;
                 }
                 if (++st == S) { st = 0; ++round; }
             }
             if (ok && lane == 0) commit_to(&sh.acc_full[acc]);
         }
-        __syncwarp();
+        mma_drain(&sh.drained, issued, failed);
     } else {
         // ---- results: warp w reads rows 32 (w % 4) .. of each tile, half of the columns (with
         // four warps and 8 columns per read the stores, not the loads, set the pace)
@@ -461,7 +463,7 @@ __global__ void __launch_bounds__(tc_threads(kDotsStages), 1) k_tc_dots(DotsArgs
         const uint32_t d_stage = sdesc_lo(su32(smem)), w_stage = stage_bytes >> 4, w_b = b_bytes >> 4;
         int st = 0, n = 0;
         uint32_t round = 0;
-        bool ok = true;
+        bool ok = true, issued = false;
         for (long ch0 = first; ch0 < last && ok; ch0 += kSegChunks, ++n) {
             const int acc = n & 1, nch = (int)(min(last, ch0 + kSegChunks) - ch0);
             if (n >= 2 && !__all_sync(0xffffffffu, mbar_wait(&sh.acc_empty[acc], ((n >> 1) - 1) & 1, failed))) break;
@@ -473,12 +475,13 @@ __global__ void __launch_bounds__(tc_threads(kDotsStages), 1) k_tc_dots(DotsArgs
                 if (lane == 0) {
                     chunk_mmas(taddr + acc * a.npad, da, da + (kABytes >> 4), db, db + w_b, idesc, ch == 0);
                     commit_to(&sh.empty[st]);
+                    issued = true;
                 }
                 if (++st == kDotsStages) { st = 0; ++round; }
             }
             if (ok && lane == 0) commit_to(&sh.acc_full[acc]);
         }
-        __syncwarp();
+        mma_drain(&sh.drained, issued, failed);
     } else {
         // ---- sums over the segments in FP64: a thread has one row (basis vector) and half of
         // the columns

@@ -33,6 +33,17 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *mbar, uint32_t parity, volat
     if (!done) *failed = 1;
     return done != 0;
 }
+// The issuing warp, before it leaves: waits (lane 0, bounded) until the MMAs it has issued are
+// done.  A block gives its tensor and shared memory back after this, also when one of its waits
+// has given up and nobody waits for the last MMAs any more.  mbar: one arrival, used only here.
+__device__ __forceinline__ void mma_drain(uint64_t *mbar, bool issued, volatile int *failed) {
+    if (issued && (threadIdx.x & 31) == 0) {
+        commit_to(mbar);
+        int none = 0;                      // (not the block's fail word, which ends a wait)
+        if (!mbar_wait(mbar, 0, &none)) *failed = 1;
+    }
+    __syncwarp();
+}
 __device__ __forceinline__ void mbar_arrive(uint64_t *mbar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(su32(mbar)) : "memory");
 }
