@@ -268,7 +268,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_ptc_tc_fwd(FwdArgs a) {
         const int row = 32 * lq + lane, sl = row / 3, col = row - 3 * sl;
         int n = 0;
         bool ok = true;
-        float nan = 0.f;                  // 0 times every result: NaN if one is not finite
         for (int ti = 0; ti < mine && ok; ++ti) {
             float sum[64];
 #pragma unroll
@@ -291,6 +290,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ptc_tc_fwd(FwdArgs a) {
             if (!ok || sl >= kSites || s >= V) continue;
             // column 8 c' + 2 s' + re/im; component 3 s' + colour is half of plane (..) / 2
             float4 *dst = a.out + (size_t)vec * a.cout * plane + s;
+            float nan = 0.f;              // 0 times every result: NaN if one is not finite
 #pragma unroll
             for (int j = 0; j < 64; j += 2) {
                 const int ch = (c_lo + j) / 8, comp = 3 * ((j % 8) / 2) + col;
@@ -300,8 +300,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_ptc_tc_fwd(FwdArgs a) {
                     nan = fmaf(sum[j], 0.f, fmaf(sum[j + 1], 0.f, nan));
                 }
             }
+            if (nan != 0.f) atomicOr(a.err, kPtcNonfinite);
         }
-        if (__any_sync(0xffffffffu, nan != 0.f) && lane == 0) atomicOr(a.err, kPtcNonfinite);
     }
     __syncthreads();
     if (sh.failed && threadIdx.x == 0) atomicOr(a.err, kPtcTimeout);
@@ -501,7 +501,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ptc_tc_wgrad(GradArgs a) {
                 nan = fmaf(v.x, 0.f, fmaf(v.y, 0.f, nan));
             }
         }
-        if (__any_sync(0xffffffffu, nan != 0.f) && lane == 0) atomicOr(a.err, kPtcNonfinite);
+        if (nan != 0.f) atomicOr(a.err, kPtcNonfinite);
     }
     __syncthreads();
     if (sh.failed && threadIdx.x == 0) atomicOr(a.err, kPtcTimeout);
