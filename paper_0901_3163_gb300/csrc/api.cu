@@ -219,7 +219,7 @@ int check_op(dlz_op_t op) {
 int check_params(const dlz_params *p) {
     if (!p) return fail(DLZ_ERR_BADARG, "null params");
     if (p->m < 2 || p->k < 0 || p->k >= p->m) return fail(DLZ_ERR_BADARG, "need m >= 2 and 0 <= k < m");
-    if (p->m > 1000) return fail(DLZ_ERR_BADARG, "m > 1000");
+    if (p->m > kMaxM) return fail(DLZ_ERR_BADARG, "m > " + std::to_string(kMaxM));
     if (!(p->tol > 0.0)) return fail(DLZ_ERR_BADARG, "tol must be > 0");
     if (p->max_cycles < 1 || p->max_iter < 1 || p->check_every < 1)
         return fail(DLZ_ERR_BADARG, "max_cycles, max_iter, check_every must be >= 1");
@@ -985,7 +985,7 @@ int dlz_defl_load(dlz_op_t h, const char *path, dlz_defl_t *out) {
     FileHeader hd;
     bool ok = std::fread(&hd, sizeof(hd), 1, f) == 1 && std::memcmp(hd.magic, kMagic, 8) == 0;
     for (int i = 0; ok && i < 4; ++i) ok = hd.dims[i] == op.g.L[i];
-    ok = ok && hd.bc_t == op.g.bc_t && hd.kappa == op.kappa && hd.k >= 0 && hd.k <= 1000 &&
+    ok = ok && hd.bc_t == op.g.bc_t && hd.kappa == op.kappa && hd.k >= 0 && hd.k <= kMaxM &&
          hd.reserved == (op.eo ? 1 : 0) &&
          (hd.which == DLZ_Q || hd.which == DLZ_DDAGD);
     if (!ok) {

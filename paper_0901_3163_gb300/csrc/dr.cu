@@ -229,6 +229,7 @@ k_lanczos_apply(const float4 *__restrict__ in, const float4 *__restrict__ Vj, co
 // Lan-DR(100, 40) and D-CG on 4 right-hand sides 385 -> 358 ms).  Eight
 // loads in flight per thread; 16 take registers that cost more blocks (78 -> 104 us).
 constexpr int kRn = 256;
+static_assert(kMaxM * sizeof(float2) <= 48 * 1024, "the coefficients of the kept vectors in shared memory");
 __global__ void __launch_bounds__(kRn)
 k_reorth_norm(float4 *__restrict__ W, const float4 *__restrict__ V, long ld, int nv, const double2 *__restrict__ coef,
               int sites, double *__restrict__ partials, unsigned *__restrict__ counter, double *__restrict__ d_b,
@@ -400,9 +401,8 @@ int dr_solve_t(Op &op, bool harmonic, const double2 *b_in, double2 *x_out, const
             }
             E *vj = V + (size_t)j * n, *wv = ucur;
             if constexpr (P::kF32) {
-                // a re-orthogonalised step (Lan-DR: every step) in five passes; the coefficients of
-                // more than 6000 kept vectors don't fit in k_reorth_norm's 48 KB
-                if (reorth_j && j > j0 && !op.eo && j0 <= 6000) {
+                // a re-orthogonalised step (Lan-DR: every step) in five passes
+                if (reorth_j && j > j0 && !op.eo) {
                     const float4 *in = vj;
                     if (!harmonic) {
                         DLZ_TRY(wilson32(op, tmp.as<E>(), vj, DLZ_Q));
@@ -430,6 +430,7 @@ int dr_solve_t(Op &op, bool harmonic, const double2 *b_in, double2 *x_out, const
                     continue;
                 }
             }
+            // FP64; FP32: a cycle's first step, and every step of an even-odd operator
             DLZ_TRY(P::apply(op, wv, vj, which, tmp.as<E>()));
             if (j == j0 && j0 > 0) DLZ_TRY(combine<P>(op, wv, n, 1, V, n, j0, coefr, 1, true, true));
             const E *vprev = (j > j0) ? V + (size_t)(j - 1) * n : nullptr;

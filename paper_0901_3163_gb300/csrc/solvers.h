@@ -6,6 +6,10 @@
 
 #include "dlz_internal.cuh"
 
+namespace dlz {
+constexpr int kMaxM = 1000;      // largest subspace (dlz_params.m), and more than the kept vectors
+}
+
 // The deflation set of Sec. 2: k orthonormal vectors (regular Ritz vectors
 // of Lan-DR or the span of the harmonic Ritz vectors of MinRes-DR) and the
 // projected operator H = V^dag A V used by the Galerkin projection of
