@@ -77,23 +77,21 @@ struct Geom {
         for (int i = 0; i < 3; ++i) dL[i] = FastDiv((unsigned)L[i]);
     }
 };
-// coordinates of site s
+// coordinates of site s.  Device code divides by dL (set by dlz_create_operator, the one place
+// that fills an operator's geometry); so does host code, unless they have not been set.
 __host__ __device__ inline void site_coords(const Geom &g, int s, int (&c)[4]) {
-#if defined(__CUDA_ARCH__)
     int r = s;
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
+#if defined(__CUDA_ARCH__)
         const int n = g.dL[i].div(r);
+#else
+        const int n = g.dL[i].d == (unsigned)g.L[i] ? g.dL[i].div(r) : r / g.L[i];
+#endif
         c[i] = r - n * g.L[i];
         r = n;
     }
     c[3] = r;
-#else
-    c[0] = s % g.L[0];
-    c[1] = s / g.L[0] % g.L[1];
-    c[2] = s / g.L[0] / g.L[1] % g.L[2];
-    c[3] = s / g.L[0] / g.L[1] / g.L[2];
-#endif
 }
 
 // ---------------------------------------------------------------- errors
