@@ -302,7 +302,7 @@ struct PassState {
 // img null: on the CUDA cores whatever the widths
 int layer_forward(Op &op, float4 *out, const float4 *in, const __nv_bfloat162 *W, const __nv_bfloat16 *img, int *err,
                   int cin, int cout, int nvec) {
-    if (img && ptc_tc_layer(cin, cout)) return ptc_tc_forward(op, out, in, img, cin, cout, nvec, err);
+    if (img && ptc_tc_layer(cin, cout, op.g.V)) return ptc_tc_forward(op, out, in, img, cin, cout, nvec, err);
     const Geom g = op.g;
     const float4 *U = op.gauge32.as<float4>();
     const unsigned gx = blocks_for(g.V, kFwdThreads);
@@ -332,9 +332,9 @@ int refresh_bf16(dlz_net_s *net) {
                                                                 net->w[l], net->w[l + 1]);
         const int cin = net->w[l], cout = net->w[l + 1];
         __nv_bfloat16 *img = net->img.as<__nv_bfloat16>();
-        if (ptc_tc_layer(cin, cout))
+        if (ptc_tc_layer(cin, cout, op.g.V))
             DLZ_TRY(ptc_tc_image(op, img + net->img_fwd[l], net->wb.as<__nv_bfloat162>() + net->off[l], cin, cout));
-        if (ptc_tc_layer(cout, cin))
+        if (ptc_tc_layer(cout, cin, op.g.V))
             DLZ_TRY(ptc_tc_image(op, img + net->img_adj[l], net->wadj.as<__nv_bfloat162>() + net->off[l], cout, cin));
     }
     op.prof.launches += 1 + net->nl;

@@ -540,9 +540,16 @@ size_t ptc_tc_image_size(int cin, int cout) {
 }
 
 // The tensor-core kernel pads the output channels to N = 16 at least and fills the same operands
-// however few there are: 16 -> 1 channels take 0.67 ms on the CUDA cores, about the 12 -> 16
-// layer's filling time here; from 4 output channels on it is the faster one.
-bool ptc_tc_layer(int, int cout) { return cout >= 4; }
+// however few there are, so its time hardly depends on C_out, while the CUDA cores' goes with C_in
+// C_out.  us on 16^4 with 4 vectors, tensor cores / CUDA cores: 1 -> 4 318 / 144, 1 -> 8 331 /
+// 283, 1 -> 9 350 / 449; 2 -> 4 309 / 245, 2 -> 5 315 / 405; 3 -> 4 447 / 346, 3 -> 5 451 / 558; 4
+// -> 3 450 / 434, 4 -> 4 450 / 451; 8 -> 3 868 / 805, 8 -> 4 868 / 866; 16 -> 1 1401 / 650.
+// Below 4096 sites both are bound by latency: 8^4 with 1 vector 1 -> 4 and 1 -> 8 13 / 17 (with 4
+// vectors 27 / 17 and 28 / 22), 4^4 12 / 16.  The rule does not look at the number of vectors: a
+// vector's result is the same in every batch.
+bool ptc_tc_layer(int cin, int cout, int sites) {
+    return cout >= (sites < 4096 ? 4 : cin == 1 ? 9 : cin < 4 ? 5 : 4);
+}
 
 int ptc_tc_prepare() {
     static int done = 0;

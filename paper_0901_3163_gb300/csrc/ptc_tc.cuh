@@ -9,8 +9,8 @@ namespace dlz {
 
 // bf16 elements of a layer's weight image (ptc_tc.cu)
 size_t ptc_tc_image_size(int cin, int cout);
-// whether the layer runs on the tensor cores
-bool ptc_tc_layer(int cin, int cout);
+// whether the layer runs on the tensor cores on a lattice of `sites` sites
+bool ptc_tc_layer(int cin, int cout, int sites);
 int ptc_tc_prepare();       // kernel attributes, outside graph captures
 // weights [9][cout][cin][16] -> image
 int ptc_tc_image(Op &op, __nv_bfloat16 *img, const __nv_bfloat162 *w, int cin, int cout);
