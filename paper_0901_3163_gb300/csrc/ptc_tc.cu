@@ -6,7 +6,7 @@
 // the input channels, spins and re/im, N over the output channels, spins and re/im, with the
 // real form [[Re W, Im W], [-Im W, Re W]]^T of the complex spin matrices.  The weights are
 // bfloat16, exact as they are; a transported FP32 value is the exact sum of three bfloat16
-// parts (8 mantissa bits each, cut off one after another), so every product is exact and only
+// parts (8 mantissa bits each, rounded off one after another), so every product is exact and only
 // the FP32 accumulation rounds.  The tensor cores cut off their sums instead of rounding them
 // to nearest (measured as about 2e-8 of the result per MMA step), so an accumulator takes
 // kMaxSteps steps of K = 16 at most before it is added, rounding to nearest, to an FP32 sum in
@@ -19,6 +19,7 @@
 // matrices, no swizzle); one warp issues the MMAs; eight warps add finished accumulators up and
 // write the tile.  They meet at mbarriers only.
 #include <algorithm>
+#include <cstring>
 
 #include "ptc_tc.cuh"
 #include "tc_util.cuh"
@@ -81,11 +82,15 @@ __device__ __forceinline__ void tmem_add(uint32_t addr, bool wide, float *sum) {
     for (int j = 0; j < 16; ++j) sum[j] += __uint_as_float(r[j]);
 }
 
-// the upper halves of two words (two bfloat16 by cutting off) in one
-__device__ __forceinline__ uint32_t pack_hi(float a, float b) {
-    return __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632);
+// two values rounded to bfloat16 in one word (a in the low half), which are taken off them
+__device__ __forceinline__ uint32_t take_part(float &a, float &b) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+    uint32_t w;
+    memcpy(&w, &h, 4);
+    a -= __uint_as_float(w << 16);
+    b -= __uint_as_float(w & 0xffff0000u);
+    return w;
 }
-__device__ __forceinline__ float cut(float x) { return __uint_as_float(__float_as_uint(x) & 0xffff0000u); }
 
 // One channel's transported spinor t of the tile's site sl as K octet `oct` of the rows 3 sl +
 // colour of the three parts (part h at h * part): 8 values (spin, re/im) = 16 bytes each
@@ -101,13 +106,9 @@ __device__ __forceinline__ void store_parts(unsigned char *stage, int part, int 
             x[2 * s + 1] = t[3 * s + c].y;
         }
 #pragma unroll
-        for (int h = 0; h < 3; ++h) {
+        for (int h = 0; h < 3; ++h)
             *reinterpret_cast<uint4 *>(dst + h * part) =
-                make_uint4(pack_hi(x[0], x[1]), pack_hi(x[2], x[3]), pack_hi(x[4], x[5]), pack_hi(x[6], x[7]));
-            if (h < 2)
-#pragma unroll
-                for (int j = 0; j < 8; ++j) x[j] -= cut(x[j]);
-        }
+                make_uint4(take_part(x[0], x[1]), take_part(x[2], x[3]), take_part(x[4], x[5]), take_part(x[6], x[7]));
     }
 }
 
@@ -312,11 +313,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_ptc_tc_fwd(FwdArgs a) {
 // G(W)[o][c'][c] = sum over sites and colours of G(out) (T_o in)^dag as P[m][n] = sum_k A[m][k]
 // B[n][k]: m = 8 c' + 2 s' + re/im of G(out), n = 8 c + 2 s + re/im of the transported input, k
 // the sites and colours; re G = P[re][re] + P[im][im], im G = P[im][re] - P[re][im].  Both
-// operands are FP32 values in three bfloat16 parts h, m, l of up to 8 bits, all with the value's
-// sign: m is below 2^-7 and l below 2^-15 of the value.  All products of parts but l l (below
-// 2^-30) are formed, smallest first, so that only the three steps of h h are cut off at the size of
-// the sum.  (Without m l and l m, together below 2^-21, every term of a sum of products of one
-// sign loses a little on the same side.)
+// operands are FP32 values in three bfloat16 parts h, m, l, rounded: |m| <= 2^-8 and |l| <= 2^-17 of
+// the value's power of two, with either sign.  Of the nine products of parts the six down to 2^-16
+// are formed, smallest first, so that only the three steps of h h are cut off at the size of the
+// sum.  The others are 2^-24 together at most and of either sign.  (Parts that are cut off have
+// the value's sign: what they leave out reaches 2^-21 and adds up in sums of one sign.)
 // A block has one offset and every gridDim.x-th tile of 16 sites: a stage is one tile, 48 k (K
 // step = colour).  The operands are stored as they come, 16 bytes = the 8 values of a channel at
 // one k, i.e. M- and N-major: 8 x 8 core matrices of 8 k x 16 bytes, k groups 128 bytes apart,
@@ -343,13 +344,9 @@ __device__ __forceinline__ void store_parts_k(unsigned char *base, int part, int
             x[2 * s + 1] = t[3 * s + c].y;
         }
 #pragma unroll
-        for (int h = 0; h < 3; ++h) {
+        for (int h = 0; h < 3; ++h)
             *reinterpret_cast<uint4 *>(dst + h * part) =
-                make_uint4(pack_hi(x[0], x[1]), pack_hi(x[2], x[3]), pack_hi(x[4], x[5]), pack_hi(x[6], x[7]));
-            if (h < 2)
-#pragma unroll
-                for (int j = 0; j < 8; ++j) x[j] -= cut(x[j]);
-        }
+                make_uint4(take_part(x[0], x[1]), take_part(x[2], x[3]), take_part(x[4], x[5]), take_part(x[6], x[7]));
     }
 }
 
@@ -445,7 +442,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ptc_tc_wgrad(GradArgs a) {
         const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) |
                                ((uint32_t)(a.npad >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
         const uint32_t d0 = sdesc_lo(su32(smem)), w_stage = stage_bytes >> 4;
-        const int pa[8] = {2, 1, 2, 0, 1, 1, 0, 0}, pb[8] = {1, 2, 0, 2, 1, 0, 1, 0};
+        const int pa[6] = {2, 0, 1, 1, 0, 0}, pb[6] = {0, 2, 1, 0, 1, 0};
         int st = 0;
         uint32_t round = 0;
         bool issued = false;
@@ -457,7 +454,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_ptc_tc_wgrad(GradArgs a) {
             const uint32_t da = d0 + st * w_stage, db = da + (3 * kGPartA >> 4);
             if (lane == 0) {
 #pragma unroll
-                for (int p = 0; p < 8; ++p)
+                for (int p = 0; p < 6; ++p)
 #pragma unroll
                     for (int k = 0; k < 3; ++k)
                         mma_bf16(taddr + acc * a.npad, da + (pa[p] * kGPartA >> 4) + k * 16, db + (pb[p] * part_b >> 4) + k * 16,
