@@ -282,6 +282,11 @@ struct dlz_net_s {
     size_t nw = 0;
     dlz::DevBuf master, grad, m1, m2, wb, wadj, partials;
     dlz::DevBuf img, state;             // weight images of the tensor-core layers; PassState
+    int *flag = nullptr;                // mapped host word, set when PassState::err is
+    dlz::PtcStatus status() const { return {state.as<int>(), flag}; }
+    ~dlz_net_s() {
+        if (flag) cudaFreeHost(flag);
+    }
     std::vector<size_t> img_fwd, img_adj;   // their offsets (bf16 elements)
     int adam_t = 0;
     dlz::DevBuf act[dlz::kMaxLayersNet + 1];   // input of every layer from the last forward
@@ -300,9 +305,9 @@ struct PassState {
 };
 
 // img null: on the CUDA cores whatever the widths
-int layer_forward(Op &op, float4 *out, const float4 *in, const __nv_bfloat162 *W, const __nv_bfloat16 *img, int *err,
-                  int cin, int cout, int nvec) {
-    if (img && ptc_tc_layer(cin, cout, op.g.V)) return ptc_tc_forward(op, out, in, img, cin, cout, nvec, err);
+int layer_forward(Op &op, float4 *out, const float4 *in, const __nv_bfloat162 *W, const __nv_bfloat16 *img,
+                  PtcStatus status, int cin, int cout, int nvec) {
+    if (img && ptc_tc_layer(cin, cout, op.g.V)) return ptc_tc_forward(op, out, in, img, cin, cout, nvec, status);
     const Geom g = op.g;
     const float4 *U = op.gauge32.as<float4>();
     const unsigned gx = blocks_for(g.V, kFwdThreads);
@@ -342,11 +347,16 @@ int refresh_bf16(dlz_net_s *net) {
     return DLZ_OK;
 }
 
-// waits for the pass and reads its state (its error bits are cleared for the next pass); fails if
-// a wait gave up
+// waits for the pass; its state, cleared for the next one.  Nothing is read back from the device
+// unless a bit is set (a copy took 10 us of a forward pass that takes 70 on 8^4).  Fails if a
+// wait gave up.
 int read_state(dlz_net_s *net, PassState &st) {
+    st.err = 0;
+    DLZ_CUDA_TRY(cudaStreamSynchronize(net->op->stream));
+    volatile int *flag = net->flag;
+    if (!*flag) return DLZ_OK;
+    *flag = 0;
     DLZ_TRY(d2h_sync(*net->op, &st, net->state.p, sizeof(PassState)));
-    if (!st.err) return DLZ_OK;
     DLZ_CUDA_TRY(cudaMemsetAsync(net->state.p, 0, sizeof(int), net->op->stream));
     if (st.err & kPtcTimeout) return fail(DLZ_ERR_DEVICE_TIMEOUT, "a wait of a tensor-core network layer gave up");
     return DLZ_OK;
@@ -359,7 +369,7 @@ int run_layers(dlz_net_s *net, int nvec, bool tc) {
     for (int l = 0; l < net->nl; ++l)
         DLZ_TRY(layer_forward(*net->op, net->act[l + 1].as<float4>(), net->act[l].as<float4>(),
                               net->wb.as<__nv_bfloat162>() + net->off[l],
-                              tc ? net->img.as<__nv_bfloat16>() + net->img_fwd[l] : nullptr, net->state.as<int>(),
+                              tc ? net->img.as<__nv_bfloat16>() + net->img_fwd[l] : nullptr, net->status(),
                               net->w[l], net->w[l + 1], nvec));
     return DLZ_OK;
 }
@@ -377,7 +387,7 @@ int run_layers_back(dlz_net_s *net, const void *grad_out, int nvec, bool want_in
             int blocks = kGradBlocks;
             if (tc) {
                 DLZ_TRY(ptc_tc_wgrad(op, net->partials.as<float2>(), gc, net->act[l].as<float4>(), cin, cout, nvec,
-                                     &st->err, blocks));
+                                     net->status(), blocks));
             } else {
                 k_ptc_wgrad<<<dim3(blocks, 9 * cin * cout), kGradThreads, 0, op.stream>>>(
                     net->partials.as<float2>(), gc, net->act[l].as<float4>(), op.gauge32.as<float4>(), op.g, cin, cout, nvec);
@@ -392,7 +402,7 @@ int run_layers_back(dlz_net_s *net, const void *grad_out, int nvec, bool want_in
         }
         if (l > 0 || want_in) {
             DLZ_TRY(layer_forward(op, gn, gc, net->wadj.as<__nv_bfloat162>() + net->off[l],
-                                  tc ? net->img.as<__nv_bfloat16>() + net->img_adj[l] : nullptr, &st->err, cout, cin, nvec));
+                                  tc ? net->img.as<__nv_bfloat16>() + net->img_adj[l] : nullptr, net->status(), cout, cin, nvec));
             std::swap(gc, gn);
         }
     }
@@ -464,6 +474,8 @@ int dlz_net_create(dlz_op_t h, int nlayers, const int *widths, const void *weigh
         }
         DLZ_TRY(net->img.alloc(ni * sizeof(__nv_bfloat16)));
         DLZ_TRY(net->state.alloc(sizeof(PassState)));
+        DLZ_CUDA_TRY(cudaHostAlloc(&net->flag, sizeof(int), cudaHostAllocMapped));
+        *net->flag = 0;
         DLZ_CUDA_TRY(cudaMemsetAsync(net->state.p, 0, sizeof(PassState), op.stream));
         int maxp = 0;
         for (int l = 0; l < nlayers; ++l) maxp = std::max(maxp, 16 * widths[l] * widths[l + 1]);

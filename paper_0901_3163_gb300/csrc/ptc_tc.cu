@@ -47,8 +47,13 @@ struct FwdArgs {
     const __nv_bfloat16 *img;
     Geom g;
     int cin, cout, npad, nvec, nbuf, ncols;
-    int *err;
+    PtcStatus status;
 };
+
+__device__ __forceinline__ void report(const PtcStatus &s, int bit) {
+    atomicOr(s.bits, bit);
+    *static_cast<volatile int *>(s.host) = 1;
+}
 
 struct FwdShared {
     uint64_t full[kGroups], empty[kGroups], acc_full[4], acc_empty[4], drained;
@@ -301,11 +306,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_ptc_tc_fwd(FwdArgs a) {
                     nan = fmaf(sum[j], 0.f, fmaf(sum[j + 1], 0.f, nan));
                 }
             }
-            if (nan != 0.f) atomicOr(a.err, kPtcNonfinite);
+            if (nan != 0.f) report(a.status, kPtcNonfinite);
         }
     }
     __syncthreads();
-    if (sh.failed && threadIdx.x == 0) atomicOr(a.err, kPtcTimeout);
+    if (sh.failed && threadIdx.x == 0) report(a.status, kPtcTimeout);
     tc_teardown(taddr, a.ncols);
 }
 
@@ -329,7 +334,7 @@ struct GradArgs {
     const float4 *gout, *in, *U;
     Geom g;
     int cin, cout, npad, nvec, nbuf, ncols;
-    int *err;
+    PtcStatus status;
 };
 
 // channel octet `oct` at site sl in the three parts (part p at p * part)
@@ -498,10 +503,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_ptc_tc_wgrad(GradArgs a) {
                 nan = fmaf(v.x, 0.f, fmaf(v.y, 0.f, nan));
             }
         }
-        if (nan != 0.f) atomicOr(a.err, kPtcNonfinite);
+        if (nan != 0.f) report(a.status, kPtcNonfinite);
     }
     __syncthreads();
-    if (sh.failed && threadIdx.x == 0) atomicOr(a.err, kPtcTimeout);
+    if (sh.failed && threadIdx.x == 0) report(a.status, kPtcTimeout);
     tc_teardown(taddr, a.ncols);
 }
 
@@ -568,10 +573,10 @@ int ptc_tc_image(Op &op, __nv_bfloat16 *img, const __nv_bfloat162 *w, int cin, i
 }
 
 int ptc_tc_forward(Op &op, float4 *out, const float4 *in, const __nv_bfloat16 *img, int cin, int cout, int nvec,
-                   int *err) {
+                   PtcStatus status) {
     FwdArgs a;
     a.out = out; a.in = in; a.U = op.gauge32.as<float4>(); a.img = img; a.g = op.g;
-    a.cin = cin; a.cout = cout; a.npad = npad_of(cout); a.nvec = nvec; a.err = err;
+    a.cin = cin; a.cout = cout; a.npad = npad_of(cout); a.nvec = nvec; a.status = status;
     a.nbuf = 4;
     const int need = a.npad * a.nbuf;
     a.ncols = tmem_columns(need);
@@ -585,11 +590,11 @@ int ptc_tc_forward(Op &op, float4 *out, const float4 *in, const __nv_bfloat16 *i
     return DLZ_OK;
 }
 
-int ptc_tc_wgrad(Op &op, float2 *partials, const float4 *gout, const float4 *in, int cin, int cout, int nvec, int *err,
+int ptc_tc_wgrad(Op &op, float2 *partials, const float4 *gout, const float4 *in, int cin, int cout, int nvec, PtcStatus status,
                  int &blocks) {
     GradArgs a;
     a.partials = partials; a.gout = gout; a.in = in; a.U = op.gauge32.as<float4>(); a.g = op.g;
-    a.cin = cin; a.cout = cout; a.npad = npad_of(cin); a.nvec = nvec; a.err = err;
+    a.cin = cin; a.cout = cout; a.npad = npad_of(cin); a.nvec = nvec; a.status = status;
     a.nbuf = 4;
     a.ncols = tmem_columns(a.npad * a.nbuf);
     // nine offsets share the SMs
