@@ -55,8 +55,8 @@
  *   DLZ_WAIT_LIMIT=n  polls before a grid-barrier wait of the persistent form gives up
  *                     (default 2^24, about a second); a test hook for the timeout path;
  *   DLZ_SLAB=n        z-planes per slab of the block walk of the batched FP32 stencils
- *                     (default: the largest divisor of Lz whose slab's traffic fits in
- *                     36 MB; Lz is the plain site order); the block sums, and so the
+ *                     (default: by the lattice and the number of right-hand sides, from
+ *                     measurements; Lz is the plain site order); the block sums, and so the
  *                     rounding, follow the blocks;
  *   DLZ_CG_STAGE=1    the fused CGNR kernels copy their gather ranges into shared
  *                     memory first (bulk asynchronous copies); same bits as the default,

@@ -329,8 +329,8 @@ __global__ void __launch_bounds__(kSumMax) k_cg_beta(const double *__restrict__ 
     }
 }
 
-// The slab walk of the fused kernels for an N-RHS batch (~900 bytes per site and
-// right-hand side: K23's streams); the even-odd kernels walk the even sites
+// The slab walk of the fused kernels for an N-RHS batch (its weight: slab_walk.cuh); the
+// even-odd kernels walk the even sites
 SlabWalk cg_slab_walk(const Op &op, int N) {
     const Geom &g = op.eo ? op.gf : op.g;
     return make_slab_walk(g.L[0] * g.L[1] / (op.eo ? 2 : 1), g.L[2], g.L[3], N, 900.0);
@@ -340,7 +340,7 @@ SlabWalk cg_slab_walk(const Op &op, int N) {
 // (DLZ_CG_STAGE=1, when the block's ranges fit).  Off by default: on 24^3 x 48 with 16
 // right-hand sides the staged kernels took 2.17 (K23) and 1.67 ms (K1) per launch against
 // 1.54 and 1.04 ms reading the neighbours from global memory (both in slabs of 4
-// z-planes).  With 66 KB of shared memory per block only 3 blocks fit on an SM (12 warps
+// z-planes, with the p and e updates that K1 made then).  With 66 KB of shared memory per block only 3 blocks fit on an SM (12 warps
 // against 24), and a block computes nothing until all of its copies have landed.
 bool cg_staged(const Op &op) {
     if (op.eo || stage_bytes(op.g.L[0]) > 200 * 1024) return false;

@@ -144,7 +144,7 @@ k_minres_k2b(const double *__restrict__ partials, int nbq, int iter, FusedState 
 
 }  // namespace
 
-// The slab walk of K1 for an N-RHS batch
+// The slab walk of K1 for an N-RHS batch (its weight: slab_walk.cuh)
 static SlabWalk minres_slab_walk(const Op &op, int N) {
     const Geom &g = op.g;
     return make_slab_walk(g.L[0] * g.L[1], g.L[2], g.L[3], N, 900.0);

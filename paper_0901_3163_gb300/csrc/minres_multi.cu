@@ -408,12 +408,13 @@ int minres_multi_batch(Op &op, int NS, const SlotDesc *sd, const Tile *tiles, in
         for (int i = 0; i < kMrBlock; ++i) DLZ_TRY(iteration(tiles[cur], i));
         return DLZ_OK;
     };
-    // Autotuner over the tiles of the graph form, 1, 2 or 4 chunks of 128 sites per block (the
-    // first three groups capture their graphs, the next three time one replay each); the fastest
-    // runs the rest.  The persistent form is taken only when it is asked for: it lost at every
-    // size measured, from 30 chunks (three lattices of 4^4 and 6^4, 2 RHS: 18.5 against 15.7 ms
-    // per call) to 16944 (nine of 8^4 .. 16^4, 8 RHS: 250 against 199 ms), and timing its six
-    // candidates took 16 ms of the latter.  Chunk partials and slot freezing do not depend on
+    // Autotuner over the tiles of the graph form, 1, 2 or 4 chunks of 128 sites per block: in the
+    // call's first inner solve the first three groups of iterations capture their graphs and the
+    // next three time one replay each; the fastest runs the rest of the call.  The persistent form
+    // is taken only when it is asked for: it lost at every size measured, from 30 chunks (three
+    // lattices of 4^4 and 6^4, 2 RHS, kappa 0.22: 16.6 against 14.6 ms per call) to 16944 (nine of
+    // 8^4 .. 16^4, 8 RHS, kappa 0.25: 490 against 381 ms), and timing its six candidates took 13
+    // ms of the latter.  Chunk partials and slot freezing do not depend on
     // the candidate, so every choice gives the same bits.
     // DLZ_MULTI_TILE=1|2|4 fixes the chunks per block; DLZ_MULTI_FORM=graph|persistent
     // fixes the form (persistent: its tiles at the full or half co-resident grid are timed).

@@ -3,9 +3,9 @@
 // A stencil kernel over N right-hand sides runs one block per (site block, right-hand
 // side), right-hand side fastest, so each block's neighbour gathers hit data that other
 // blocks brought into L2.  In the plain site order (x fastest, t slowest) a t-neighbour
-// lies one whole 3-D slice away.  With 16 right-hand sides on 24^3 x 48 the traffic of a
-// slice (~13824 sites x 16 x ~900 bytes for the fused CGNR kernels) is larger than L2, so
-// those gathers go to DRAM a second time.
+// lies one whole 3-D slice away.  With 16 right-hand sides on 24^3 x 48 the vectors that the
+// kernels of an iteration go through in a slice do not stay in L2, so those gathers go to DRAM
+// a second time.
 //
 // The walk here takes slabs of bz z-planes at one t, each a contiguous range of
 // bz * plane sites: the slabs of z-slab 0 for t = 0 .. Lt-1, then those of z-slab 1, and so
@@ -67,12 +67,16 @@ inline SlabWalk slab_walk_of(int plane, int Lz, int Lt, int bz, int N = 1) {
     return w;
 }
 
-// The walk for N right-hand sides moving about `bytes` per site and right-hand side: the
-// plain order when a slab's traffic fits in 36 MB, else the largest divisor of Lz whose
-// slab does (at least one plane).  On 24^3 x 48 with 16 right-hand sides that is 4 planes
-// for the fused CGNR kernels, which took 1.54 / 1.05 ms (K23 / K1) per launch against
-// 1.88 / 1.20 ms in the plain order (3: 1.54 / 1.07; 6: 1.70 / 1.06; 2: 1.64 / 1.18).
-// DLZ_SLAB=n fixes n planes.
+// The walk for N right-hand sides of weight `bytes` per site and right-hand side: the plain
+// order when a slab weighs 36 MB at most, else the largest divisor of Lz whose slab does (at
+// least one plane).  The weights are set by measurement, not equal to a kernel's streams.  With
+// 900 the fused kernels take 4 planes on 24^3 x 48 with 16 right-hand sides, where K1 / K23 took,
+// relative to that, 1.29 / 1.27 with 1 plane, 1.06 / 1.06 with 2, 1.03 / 1.03 with 3, 0.99 / 1.00
+// with 6, 1.02 / 1.02 with 8, 1.03 / 1.05 with 12 and 1.12 / 1.16 in the plain order; MinRes K1
+// with 11 right-hand sides (6 planes) 1.05, 1.01, 1.00, 1.00 and 1.04 with 3, 4, 8, 12 and 24.  The
+// even-odd pairs with 16 (8 planes, the hop in the plain order) are fastest so.  Lighter launches
+// (24^3 x 48 with 4 right-hand sides, 16^3 x 32 with 11 and 16) would gain 1 to 3 % in the plain
+// order.  DLZ_SLAB=n fixes n planes.
 inline SlabWalk make_slab_walk(int plane, int Lz, int Lt, int N, double bytes) {
     const double per_plane = (double)plane * N * bytes;
     int bmax = per_plane > 0.0 ? (int)std::min((double)Lz, 36.0e6 / per_plane) : Lz;
