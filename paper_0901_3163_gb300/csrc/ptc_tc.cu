@@ -10,7 +10,7 @@
 // the FP32 accumulation rounds.  The tensor cores cut off their sums instead of rounding them
 // to nearest (measured as about 2e-8 of the result per MMA step), so an accumulator takes
 // kMaxSteps steps of K = 16 at most before it is added, rounding to nearest, to an FP32 sum in
-// registers.  Error against 64 bits of three layers 1 -> 12 -> 16 -> 1 on 16^4: 6.6e-7, 8.2e-7
+// registers.  Error against 64 bits of three layers 1 -> 12 -> 16 -> 1 on 16^4: 6.5e-7, 8.2e-7
 // with FP32 arithmetic on the CUDA cores (27 steps per accumulator: 9.5e-7).
 //
 // Block: tiles of 42 sites (126 rows) of one vector.  kGroups groups of four filling warps
